@@ -24,7 +24,7 @@ UNITS = [("lb_kernels.cu", [f"-DLB_PREC={p}"], f"lb_kernels_p{p}.o") for p in ra
     ("lb_noalloc.cu", [], "lb_noalloc.o"),
 ]
 SOURCES = sorted({u[0] for u in UNITS})
-HEADERS = ["lb_internal.h", "lb_layout.cuh", "lb_engine.h"]
+HEADERS = ["lb_internal.h", "lb_layout.cuh", "lb_engine.h", "lb_exp_table.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--expt-relaxed-constexpr"]

@@ -150,19 +150,23 @@ static void fill_coef(Coef<C>& k, const lb_params* p) {
         k.KC[r].x = K[0] * f;
         k.KC[r].y = K[1] * f;
     }
-    k.WC[0].x = k.WC[0].y = (C)w_weight(1);
-    k.WC[1].x = k.WC[1].y = (C)w_weight(2);
+    const bool f64 = sizeof(C) == 8;
+    k.WC[0].x = k.WC[0].y = f64 ? C(4) : (C)w_weight(1);
+    k.WC[1].x = k.WC[1].y = f64 ? C(1) : (C)w_weight(2);
     // Offsets are taken from rho_ref rounded to the compute precision, so that
     // rho = rho_ref + sum_i h_i holds with the same rho_ref on every path.
     const double rref = (double)(C)(p->rho_ref > 0.0 ? p->rho_ref : p->rho0);
     const double pref = p->psi_form == LB_PSI_RHO0 ? p->rho0 : std::sqrt(p->rho0);
-    k.gx_rho0 = (C)(p->G_X / p->rho0);
+    k.gx_rho0 = (C)(p->G_X / p->rho0 * (f64 ? w_weight(2) : 1.0));
     k.rho_ref = (C)rref;
     k.psi_ref = (C)(pref * (1.0 - std::exp(-rref / p->rho0)));
     k.psi_scale = (C)(pref * std::exp(-rref / p->rho0));
     k.inv_rho0 = (C)(1.0 / p->rho0);
-    k.tau3[0] = (C)(3.0 * p->tau_A);
-    k.tau3[1] = (C)(3.0 * p->tau_B);
+    k.exp_c = (C)(-64.0 / (M_LN2 * p->rho0));
+    k.psi_a = k.psi_ref * k.psi_scale;
+    k.psi_b = -k.psi_scale * k.psi_scale;
+    k.tau15[0] = (C)(1.5 * p->tau_A);
+    k.tau15[1] = (C)(1.5 * p->tau_B);
     k.omega[0] = (C)(1.0 / p->tau_A);
     k.omega[1] = (C)(1.0 / p->tau_B);
     // omega w times the storage scale (a power of two: exact), per class of
@@ -172,6 +176,10 @@ static void fill_coef(Coef<C>& k, const lb_params* p) {
     for (int c = 0; c < 3; ++c) {
         k.omw[c].x = (C)(sc * wc[c] / p->tau_A);
         k.omw[c].y = (C)(sc * wc[c] / p->tau_B);
+    }
+    for (int c = 0; c < 2; ++c) {
+        k.omw2[c].x = C(2) * k.omw[c + 1].x;
+        k.omw2[c].y = C(2) * k.omw[c + 1].y;
     }
     k.omm.x = (C)(1.0 - 1.0 / p->tau_A);
     k.omm.y = (C)(1.0 - 1.0 / p->tau_B);
@@ -183,19 +191,6 @@ static void fill_coef(Coef<C>& k, const lb_params* p) {
             (p->precision == LB_FP16_OFFSET || p->precision == LB_BF16_OFFSET)) ? 1 : 0;
     k.source = p->force_scheme == LB_FORCE_SOURCE ? 1 : 0;
     k.has_accel = (p->g_x != 0.0 || p->kolmo_amp != 0.0) ? 1 : 0;
-}
-
-template <typename C>
-static LatVals<C> vals_of(const Coef<C>& k) {
-    LatVals<C> v;
-    v.rho_ref = k.rho_ref;
-    v.psi_ref = k.psi_ref;
-    v.psi_scale = k.psi_scale;
-    v.inv_rho0 = k.inv_rho0;
-    v.gx_rho0 = k.gx_rho0;
-    v.u_wall = k.u_wall;
-    v.kolmo_w = k.kolmo_w;
-    return v;
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,

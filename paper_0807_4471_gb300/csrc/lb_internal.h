@@ -69,19 +69,26 @@ template <> struct PairOf<double> { typedef double2 T; };
 // weights are the (A, B) pairs KC = {K(1), K(2), K(5), 2 K(4), 2 K(5),
 // 2 K(8)} (the factors 2 are the stencil components |d_x| or |d_y| = 2,
 // exact), and the cross-species ones WC = {w(1), w(2)} for both species.
+// FP64 folds factors so that a site takes fewer FP64 operations: its window
+// holds E = exp(-(rho - rho_ref)/rho0) - 1 in place of the Psi deviation
+// -psi_scale E, its cross weights are {4, 1} = {w(1), w(2)} / w(2), and
+// psi_a, psi_b and gx_rho0 carry the factors.
 template <typename C>
 struct Coef {
     typedef typename PairOf<C>::T C2;
     C2 KC[6];          // like-species row weights, (A, B) pairs
     C2 WC[2];          // cross-species row weights, equal in both lanes
-    C gx_rho0;         // G_X / rho0
+    C gx_rho0;         // G_X / rho0 (FP64: times w(2))
     C psi_ref;         // Psi(rho_ref)
     C psi_scale;       // P exp(-rho_ref / rho0)
     C inv_rho0;        // 1 / rho0
+    C exp_c;           // FP64: -64 / (ln2 rho0), see pexpm1_scaled
+    C psi_a, psi_b;    // FP64: psi_ref psi_scale, -psi_scale^2
     C rho_ref;         // reference density of the stored offsets
-    C tau3[2];         // 3 tau_s (the velocity shift is taken for v = 3u)
+    C tau15[2];        // 1.5 tau_s (the velocity shift is taken for v = 1.5u)
     C omega[2];        // 1 / tau
     C2 omw[3];         // omega_s S w for the D2Q9 classes |c|^2 = 0, 1, 2 (S the storage scale)
+    C2 omw2[2];        // 2 omega_s S w for the classes |c|^2 = 1, 2 (exact doubles of omw[1..2])
     C2 omm;            // 1 - omega_s
     C u_wall;          // Couette wall speed (top +, bottom -)
     C g_x;             // uniform body acceleration
@@ -97,7 +104,23 @@ template <typename C>
 struct LatVals {
     C rho_ref, psi_ref, psi_scale, inv_rho0, gx_rho0, u_wall;
     C kolmo_w;         // 2 pi kolmo_k / ny (ny is per lattice)
+    C exp_c, psi_a, psi_b;   // (FP64)
 };
+template <typename C>
+__host__ __device__ inline LatVals<C> vals_of(const Coef<C>& k) {
+    LatVals<C> v;
+    v.rho_ref = k.rho_ref;
+    v.psi_ref = k.psi_ref;
+    v.psi_scale = k.psi_scale;
+    v.inv_rho0 = k.inv_rho0;
+    v.gx_rho0 = k.gx_rho0;
+    v.u_wall = k.u_wall;
+    v.kolmo_w = k.kolmo_w;
+    v.exp_c = k.exp_c;
+    v.psi_a = k.psi_a;
+    v.psi_b = k.psi_b;
+    return v;
+}
 
 // One lattice of a step launch, in device memory (128-byte aligned for the
 // tensor maps).  Both buffers are described; the device-side DevStats::cur

@@ -225,11 +225,36 @@ __device__ __forceinline__ void load_site(const typename Prec<P>::T2* bm,
     }
 }
 
+#if LB_PREC == 0
+static __device__ const double2 g_exp_tab[kExpN] = {LB_EXP_TABLE};
+__device__ __noinline__ double expm1_slow(double x) { return expm1(x); }
+#endif
+
 // Deviation of the pseudo-potential from Psi(rho_ref), both species:
 // Psi(rho_ref + d) - Psi(rho_ref) = -P exp(-rho_ref/rho0) expm1(-d/rho0).
-template <typename C, typename C2>
-__device__ __forceinline__ C2 dpsi_of(C2 d, const LatVals<C>& v) {
+// FP64: without the factor -P exp(-rho_ref/rho0), which neg_psi carries; tab:
+// the exponential table.
+__device__ __forceinline__ float2 dpsi_of(float2 d, const LatVals<float>& v, const double2*) {
     return pmul(pset(-v.psi_scale), pexpm1(pmul(d, pset(-v.inv_rho0))));
+}
+__device__ __forceinline__ double2 dpsi_of(double2 d, const LatVals<double>& v, const double2* tab) {
+    return pexpm1_scaled(d, v.exp_c, v.inv_rho0, tab);
+}
+// -Psi_s(r) from the window value; FP64: times the factor that the stencil
+// sums of the window values lack, -psi_scale:
+// -(psi_ref - psi_scale E)(-psi_scale) = psi_ref psi_scale - psi_scale^2 E.
+__device__ __forceinline__ float2 neg_psi(float2 dpsi, const LatVals<float>& v) {
+    return psub(pset(-v.psi_ref), dpsi);
+}
+__device__ __forceinline__ double2 neg_psi(double2 E, const LatVals<double>& v) {
+    return pfma(pset(v.psi_b), E, pset(v.psi_a));
+}
+// Adds 0 * rho to nf: NaN from the first inf or NaN density on, else zero.
+// (FP64: by the exponent bits, without an FP64 operation.)
+__device__ __forceinline__ void note_nonfinite(float2 rho, float2& nf) { nf = pfma(rho, pset(0.0f), nf); }
+__device__ __forceinline__ void note_nonfinite(double2 rho, double2& nf) {
+    const int a = __double2hiint(rho.x) & 0x7ff00000, b = __double2hiint(rho.y) & 0x7ff00000;
+    if (max(a, b) == 0x7ff00000) nf.x = __hiloint2double(0x7ff80000, 0);
 }
 
 // Momentum j = sum_i c_i f_i of both species from the offsets (sum_i w_i c_i
@@ -258,55 +283,57 @@ __device__ __forceinline__ void cell_dev(const typename Prec<P>::T2* bm,
                                          const typename Prec<P>::T2* bp, int y, bool per, int pull,
                                          const Geom& g, const LatVals<typename Prec<P>::C>& v,
                                          typename Prec<P>::C2& r, typename Prec<P>::C2& q,
-                                         typename Prec<P>::C2* j = nullptr) {
+                                         const double2* tab, typename Prec<P>::C2* j = nullptr) {
     typename Prec<P>::C2 h[9];
     load_site<P, PS>(bm, b0, bp, y, per, pull, g, v, h);
     r = sum9(h);
     if constexpr (Prec<P>::SCALE_LOG2 != 0) r = pmul(r, pset(inv_scale_of<P>()));
-    q = dpsi_of(r, v);
+    q = dpsi_of(r, v, tab);
     if constexpr (J) moments<P, false>(h, j[0], j[1]);
 }
 
 // Post-collision offsets of both species (Eq. (1), BGK toward the
-// equilibrium at velocity u, per species), written with v = 3u:
+// equilibrium at velocity u, per species), written with z = 1.5u (half of
+// 3u, so that the halves below are exact and take no operation):
 //   h*_i = (1 - omega) h_i + omega heq_i [+ 3 w_i c_i . F for the source scheme],
 //   heq_i = f^eq_i - w_i rho_ref = w_i [d_rho + rho (3 c.u + 4.5 (c.u)^2 - 1.5 u^2)]
-//         = w_i [Q + rho (c.v) + rho (c.v)^2 / 2],  Q = d_rho - rho v^2 / 6,
-// evaluated per pair (i, opp(i)), whose c.v differ only in sign:
-// heq = w (g +- rho c.v) with g = Q + rho (c.v)^2 / 2.  h and out are in
+//         = w_i [Q + (2 rho) (c.z) + (2 rho) (c.z)^2],  Q = d_rho - (2/3) rho z^2,
+// evaluated per pair (i, opp(i)), whose c.z differ only in sign:
+// heq = w (g +- 2 rho c.z) with g = Q + (2 rho c.z) (c.z).  h and out are in
 // the storage scale SC (a power of two); k.omw holds omega SC w per class
 // of |c|^2 and k.omm = 1 - omega.
-// TAU1: omega = 1 for both species, where h*_i = heq_i and h is not read.
 //
 // TAU1 (omega = 1): h*_i = heq_i, taken per class c of |c_i|^2 as
-//   h*_{i, opp(i)} = E +- kv,  E = T_c + kv (c.v) / 2,  kv = K_c (c.v),
-// with T_c = omega S w_c Q and K_c = omega S w_c rho per site; h is not read.
+//   h*_{i, opp(i)} = E +- kv,  E = T_c + kv (c.z),  kv = K_c (c.z),
+// with T_c = omega S w_c Q and K_c = 2 omega S w_c rho per site; h is not read.
 template <typename C, typename C2, bool SRC, bool TAU1 = false>
-__device__ __forceinline__ void collide(const C2 h[9], C2 out[9], C2 drho, C2 rho, C2 vx, C2 vy,
+__device__ __forceinline__ void collide(const C2 h[9], C2 out[9], C2 drho, C2 rho, C2 zx, C2 zy,
                                         const Coef<C>& k, C2 Fx, C2 Fy, C SC) {
-    const C2 Q = pfma(pmul(rho, pset(C(-1) / C(6))), pfma(vx, vx, pmul(vy, vy)), drho);
+    const C2 Q = pfma(pmul(rho, pset(C(-4) / C(6))), pfma(zx, zx, pmul(zy, zy)), drho);
     out[0] = TAU1 ? pmul(k.omw[0], Q) : pfma(k.omw[0], Q, pmul(k.omm, h[0]));
-    C2 T[2], K[2];
+    C2 T[2], K[2], rho2;
     if (TAU1) {
         T[0] = pmul(k.omw[1], Q);
         T[1] = pmul(k.omw[2], Q);
-        K[0] = pmul(k.omw[1], rho);
-        K[1] = pmul(k.omw[2], rho);
+        K[0] = pmul(k.omw2[0], rho);
+        K[1] = pmul(k.omw2[1], rho);
+    } else {
+        rho2 = padd(rho, rho);
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        const int i = q == 0 ? 1 : (q == 1 ? 2 : (q == 2 ? 5 : 6));   // c.v = vx, vy, vx+vy, vy-vx
+        const int i = q == 0 ? 1 : (q == 1 ? 2 : (q == 2 ? 5 : 6));   // c.z = zx, zy, zx+zy, zy-zx
         const int j = opp(i);
-        const C2 cv = q == 0 ? vx : (q == 1 ? vy : (q == 2 ? padd(vx, vy) : psub(vy, vx)));
+        const C2 cz = q == 0 ? zx : (q == 1 ? zy : (q == 2 ? padd(zx, zy) : psub(zy, zx)));
         if (TAU1) {
-            const C2 kv = pmul(K[q >> 1], cv);
-            const C2 E = pfma(kv, pmul(cv, pset(C(0.5))), T[q >> 1]);
+            const C2 kv = pmul(K[q >> 1], cz);
+            const C2 E = pfma(kv, cz, T[q >> 1]);
             out[i] = padd(E, kv);
             out[j] = psub(E, kv);
         } else {
             const C2 ow = k.omw[q < 2 ? 1 : 2];
-            const C2 rv = pmul(rho, cv);
-            const C2 g = pfma(rv, pmul(cv, pset(C(0.5))), Q);
+            const C2 rv = pmul(rho2, cz);
+            const C2 g = pfma(rv, cz, Q);
             out[i] = pfma(ow, padd(g, rv), pmul(k.omm, h[i]));
             out[j] = pfma(ow, psub(g, rv), pmul(k.omm, h[j]));
         }
@@ -436,6 +463,53 @@ __device__ __forceinline__ void force_sums(const C2* ps, const C2* rr, const Coe
     }
 }
 
+// FP64: the stencil sums of a warp's row of sites, taken column by column.
+// The FP64 step is bound by its FP64 operations (two lanes per SM and clock),
+// while shuffles and shared-memory loads are nearly free beside them, so the
+// sums over a window column are taken once, by the lane that holds the
+// column, and shared along the row by shuffles: with v_k = q(+k) + q(-k) and
+// w_k = q(+k) - q(-k) of a column (k rows above and below),
+//   sum_d K d_x q: A(+1) - A(-1) + B(+2) - B(-2),
+//     A = K(1) q + K(2) v_1 + K(5) v_2,  B = 2K(4) q + 2K(5) v_1 + 2K(8) v_2,
+//   sum_d K d_y q: C_0 + C_1(+1) + C_1(-1) + C_2(+2) + C_2(-2),
+//     C_0 = K(1) w_1 + 2K(4) w_2,  C_1 = K(2) w_1 + 2K(5) w_2,  C_2 = K(5) w_1 + 2K(8) w_2
+// (arguments: columns right or left of the site), 23 FP64 operations per
+// species against 41 row by row; the cross sums likewise in 6 against 13.
+// ps, rr: the Psi and rho window rows (row stride RXS) at window column
+// `lane`, starting two rows above the sites; a lane's site is two columns to
+// the right of its window column.  All lanes of the warp call it.
+__device__ __forceinline__ double2 shfl_down2(double2 v, int n) {
+    return make_double2(__shfl_down_sync(0xffffffffu, v.x, n), __shfl_down_sync(0xffffffffu, v.y, n));
+}
+template <int RXS>
+__device__ __forceinline__ void force_sums_warp(const double2* ps, const double2* rr,
+                                                const Coef<double>& k, double2& fx, double2& fy,
+                                                double2& qx, double2& qy, double2& dpsi,
+                                                double2& drho) {
+    {
+        const double2 q0 = ps[2 * RXS];
+        const double2 v1 = padd(ps[3 * RXS], ps[RXS]), w1 = psub(ps[3 * RXS], ps[RXS]);
+        const double2 v2 = padd(ps[4 * RXS], ps[0]), w2 = psub(ps[4 * RXS], ps[0]);
+        const double2 A = pfma(k.KC[2], v2, pfma(k.KC[1], v1, pmul(k.KC[0], q0)));
+        const double2 B = pfma(k.KC[5], v2, pfma(k.KC[4], v1, pmul(k.KC[3], q0)));
+        fx = padd(psub(shfl_down2(A, 3), shfl_down2(A, 1)), psub(shfl_down2(B, 4), B));
+        const double2 C0 = pfma(k.KC[3], w2, pmul(k.KC[0], w1));
+        const double2 C1 = pfma(k.KC[4], w2, pmul(k.KC[1], w1));
+        const double2 C2 = pfma(k.KC[5], w2, pmul(k.KC[2], w1));
+        fy = padd(padd(shfl_down2(C0, 2), padd(shfl_down2(C1, 3), shfl_down2(C1, 1))),
+                  padd(shfl_down2(C2, 4), C2));
+        dpsi = shfl_down2(q0, 2);
+    }
+    {
+        const double2 r0 = rr[2 * RXS];
+        const double2 A = pfma(k.WC[0], r0, padd(rr[3 * RXS], rr[RXS]));   // weights 4, 1
+        const double2 w = psub(rr[3 * RXS], rr[RXS]);
+        qx = psub(shfl_down2(A, 3), shfl_down2(A, 1));
+        qy = pfma(k.WC[0], shfl_down2(w, 2), padd(shfl_down2(w, 3), shfl_down2(w, 1)));
+        drho = shfl_down2(r0, 2);
+    }
+}
+
 // Plain global stores of a stored pair, with an L2 cache policy.
 __device__ __forceinline__ void st_pair(float2* p, float2 v, uint64_t pol) {
     asm volatile("st.global.L2::cache_hint.v2.f32 [%0], {%1, %2}, %3;" ::"l"(p), "f"(v.x), "f"(v.y),
@@ -519,13 +593,13 @@ __device__ __forceinline__ void site_update(
     if constexpr (OBS) {
         if (o.valid && !(isfinite(rho.x) && isfinite(rho.y))) bad = true;
     } else if (o.valid) {
-        *nf = pfma(rho, pset(C(0)), *nf);   // stays zero unless a density is inf or NaN
+        note_nonfinite(rho, *nf);   // stays zero unless a density is inf or NaN
     }
 
     // Eq. (2): F_s = -Psi_s(r) sum_d K_s(d) d Psi_s(r + d)
     //               - (G_X/rho0) rho_s(r) sum_d w(d) d rho_s'(r + d);
     // species A feels rho_B, so the cross sums are used swapped.
-    const C2 npc = psub(pset(-v.psi_ref), dpsi);          // -Psi_s(r)
+    const C2 npc = neg_psi(dpsi, v);                       // -Psi_s(r)
     const C2 ng = pmul(pset(-v.gx_rho0), rho);             // -(G_X/rho0) rho_s
     C2 Fx = pfma(npc, fxl, pmul(ng, pair(qx.y, qx.x)));
     C2 Fy = pfma(npc, fyl, pmul(ng, pair(qy.y, qy.x)));
@@ -565,30 +639,30 @@ __device__ __forceinline__ void site_update(
 
     // Eq. (1): forced BGK relaxation.  Common velocity
     // u' = sum_s (j_s/tau_s) / sum_s (rho_s/tau_s); shift u_s = u' + tau_s F_s/rho_s;
-    // carried as v = 3u.  (Selects, not branches: an empty site has u' = 0
+    // carried as z = 1.5u.  (Selects, not branches: an empty site has u' = 0
     // and no shift.)
     // (TAU1: omega = 1 exactly, and the products are the values themselves)
     const C2 om = pair(k.omega[0], k.omega[1]);
     const C2 ro = TAU1 ? rho : pmul(rho, om), jxo = TAU1 ? jx : pmul(jx, om),
              jyo = TAU1 ? jy : pmul(jy, om);
     const C den = ro.x + ro.y;
-    // 3 / den, times the storage scale's inverse where j is taken in the
+    // 1.5 / den, times the storage scale's inverse where j is taken in the
     // storage scale (TAU1; both factors exact powers of two apart)
-    const C inv3 = den != C(0) ? (TAU1 ? C(3) * inv_scale_of<P>() : C(3)) * recip(den) : C(0);
-    const C2 vp = pair((jxo.x + jxo.y) * inv3, (jyo.x + jyo.y) * inv3);
+    const C inv = den != C(0) ? (TAU1 ? C(1.5) * inv_scale_of<P>() : C(1.5)) * recip(den) : C(0);
+    const C2 zp = pair((jxo.x + jxo.y) * inv, (jyo.x + jyo.y) * inv);
     const bool source = GEN && k.source;
-    C2 vx = pset(vp.x), vy = pset(vp.y);
+    C2 zx = pset(zp.x), zy = pset(zp.y);
     if (!source) {
-        const C2 tr = pair(rho.x != C(0) ? k.tau3[0] * recip(rho.x) : C(0),
-                           rho.y != C(0) ? k.tau3[1] * recip(rho.y) : C(0));
-        vx = pfma(tr, Fx, vx);
-        vy = pfma(tr, Fy, vy);
+        const C2 tr = pair(rho.x != C(0) ? k.tau15[0] * recip(rho.x) : C(0),
+                           rho.y != C(0) ? k.tau15[1] * recip(rho.y) : C(0));
+        zx = pfma(tr, Fx, zx);
+        zy = pfma(tr, Fy, zy);
     }
     C2 hs[9];
     if (source)
-        collide<C, C2, true, TAU1>(h, hs, drho, rho, vx, vy, k, Fx, Fy, scale_of<P>());
+        collide<C, C2, true, TAU1>(h, hs, drho, rho, zx, zy, k, Fx, Fy, scale_of<P>());
     else
-        collide<C, C2, false, TAU1>(h, hs, drho, rho, vx, vy, k, Fx, Fy, scale_of<P>());
+        collide<C, C2, false, TAU1>(h, hs, drho, rho, zx, zy, k, Fx, Fy, scale_of<P>());
     T2 e[9];
     if constexpr (sizeof(T2) == 4) {
         if (k.sr) {   // half formats: random bits from (site, step), one word per pair
@@ -878,6 +952,7 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
     // window column and block row of this thread (both phases)
     const int t_lx = tid % L::RX, t_j = tid / L::RX;
     static_assert(L::NT == L::RX * L::TYB && L::TY >= 4, "one window column per thread and block row");
+    static_assert(P != LB_FP64 || (L::RX == 32 && SPT == 1), "FP64: a warp is a row of a tile");
     // Rows of the density phase: thread row t_j computes the new window rows
     // 4 + SPT t_m + c, c < SPT, which hold its own sites (window rows
     // 2 + SPT t_j + c) for t_j >= 2 / SPT; the first 2 / SPT thread rows,
@@ -898,6 +973,11 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
     const int t_w = (t_lx + 2) % L::RX;
     // TAU1: momenta (jx, jy) of the first thread rows' new cells, kept for
     // the next tile, whose first sites they are; jc: this thread's entries
+    // FP64: the exponential table, copied while the previous step drains
+    double2* s_tab = reinterpret_cast<double2*>(smem + L::TAB_OFF);
+#if LB_PREC == 0
+    for (int i = tid; i < kExpN; i += L::NT) s_tab[i] = g_exp_tab[i];
+#endif
     __shared__ __align__(16) C2 s_jcarry[kCarry * L::RX * SPT * 2];
     C2* const jc = s_jcarry + ((t_carry ? t_j : 0) * L::RX + t_lx) * (SPT * 2);
     auto slot = [&](int pos) { return reinterpret_cast<T2*>(smem + (pos % L::NB) * L::SLOT_BYTES); };
@@ -1041,7 +1121,7 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
                             if (ty == ty_a) {
                                 C2 r, p, jt[2];
                                 cell_dev<P, PS, TAU1>(brow(kk, bc), brow(kk + 1, bc), brow(kk + 2, bc),
-                                                      y0 - 2 + kk, per, pull, g, v, r, p, jt);
+                                                      y0 - 2 + kk, per, pull, g, v, r, p, s_tab, jt);
                                 win_r[kk * L::RX + t_w] = r;
                                 win_p[kk * L::RX + t_w] = p;
                                 if (TAU1 && t_carry) {   // rows 2 and 3: this thread's sites
@@ -1064,7 +1144,7 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
                         const int k = 4 + SPT * t_m + c;
                         C2 r, p;
                         cell_dev<P, PS, TAU1>(brow(k, bc), brow(k + 1, bc), brow(k + 2, bc), y0 - 2 + k,
-                                              per, pull, g, v, r, p, jn[c]);
+                                              per, pull, g, v, r, p, s_tab, jn[c]);
                         win_r[k * L::RX + t_w] = r;
                         win_p[k * L::RX + t_w] = p;
                     }
@@ -1114,10 +1194,16 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
                 {
                     const int lx = t_lx, ly = SPT * t_j;
                     const int x = x0 + lx, y = y0 + ly;
+                    C2 fx[SPT], fy[SPT], qx[SPT], qy[SPT], dp[SPT], dr[SPT];
+                    if constexpr (P == LB_FP64) {   // a warp is a row (RX = 32)
+                        if (y < g.ny)
+                            force_sums_warp<L::RX>(win_p + ly * L::RX + lx, win_r + ly * L::RX + lx, a.k,
+                                                   fx[0], fy[0], qx[0], qy[0], dp[0], dr[0]);
+                    }
                     if (lx < L::TX && x < g.nx && y < g.ny) {
-                        C2 fx[SPT], fy[SPT], qx[SPT], qy[SPT], dp[SPT], dr[SPT];
-                        force_sums<SPT, L::RX>(win_p + ly * L::RX + lx + 2,
-                                               win_r + ly * L::RX + lx + 2, a.k, fx, fy, qx, qy, dp, dr);
+                        if constexpr (P != LB_FP64)
+                            force_sums<SPT, L::RX>(win_p + ly * L::RX + lx + 2,
+                                                   win_r + ly * L::RX + lx + 2, a.k, fx, fy, qx, qy, dp, dr);
                         SiteOut<T2> o;
                         o.rbits = 0u;
                         [[maybe_unused]] uint32_t srh = 0u;   // the shared hash of this thread's sites
@@ -1277,14 +1363,11 @@ __global__ void __launch_bounds__(Layout<P>::NT)
     const int x0 = blockIdx.x * L::TX, y0 = blockIdx.y * L::TY;
     const Geom& g = a.g;
     const bool per = g.periodic != 0;
-    LatVals<C> v;
-    v.rho_ref = a.k.rho_ref;
-    v.psi_ref = a.k.psi_ref;
-    v.psi_scale = a.k.psi_scale;
-    v.inv_rho0 = a.k.inv_rho0;
-    v.gx_rho0 = a.k.gx_rho0;
-    v.u_wall = a.k.u_wall;
-    v.kolmo_w = a.k.kolmo_w;
+    const LatVals<C> v = vals_of(a.k);
+    const double2* tab = nullptr;
+#if LB_PREC == 0
+    tab = g_exp_tab;
+#endif
     if (tid == 0) {
         s_fail = 0;
         mbar_init(&bar, 1);
@@ -1305,7 +1388,7 @@ __global__ void __launch_bounds__(Layout<P>::NT)
             if (!per && (y < 0 || y >= g.ny)) continue;
             const T2* b0 = box + (ly + 1) * L::BX + lx - 2 + L::GX;
             C2 r, p;
-            cell_dev<P, PS>(b0 - L::BX, b0, b0 + L::BX, y, per, a.pull, g, v, r, p);
+            cell_dev<P, PS>(b0 - L::BX, b0, b0 + L::BX, y, per, a.pull, g, v, r, p, tab);
             srho[ly * L::RX + lx] = r;
             spsi[ly * L::RX + lx] = p;
         }

@@ -6,6 +6,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include "lb_exp_table.h"
 #include "lb_internal.h"
 
 namespace lbgb {
@@ -158,17 +159,63 @@ __device__ __forceinline__ double2 pset(double v) { return make_double2(v, v); }
 __device__ __forceinline__ float2 pair(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ double2 pair(double a, double b) { return make_double2(a, b); }
 
-// Reciprocal: correctly rounded in FP64; in FP32 the hardware approximation
+// Reciprocal, for normal arguments.  FP64: the hardware's gross approximation
+// (rcp.approx.ftz.f64, 20 bits or more) and one third-order step
+// y (1 + e + e^2), e = 1 - v y, which leaves e^3 < 2^-60: three FP64
+// operations, within about an ulp.  FP32: the hardware approximation
 // (rcp.approx.ftz, within 1 ulp), which has no slow path or branch.
-__device__ __forceinline__ double recip(double v) { return 1.0 / v; }
+__device__ __forceinline__ double recip(double v) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
+    const double e = fma(-v, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
 __device__ __forceinline__ float recip(float v) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
     return r;
 }
 
-// exp(x) - 1 of a pair.  FP64: the library function.  FP32: branch-free, by the
-// Cody-Waite reduction x = k ln2 + r (|r| <= ln2 / 2, ln2 split into a
+// E = exp(-d / rho0) - 1 of a pair in FP64, c = -64 / (ln2 rho0), inv_rho0 =
+// 1 / rho0: table-driven after P. T. P. Tang ("Table-driven implementation of
+// the expm1 function", ACM TOMS 18, 1992).  n = the integer nearest d c,
+// r = d c - n by one fused operation (|r| <= 1/2, in units of ln2 / 64), and
+// E = (T - 1) + T p with T = 2^(n/64) and T - 1 from the table and p =
+// exp(r ln2 / 64) - 1 from its Taylor polynomial of degree 6 (truncation below
+// 2^-57 relative).  Ten FP64 operations a value: GB300 runs two FP64 lanes
+// per SM and clock, and the FP64 step is bound by them (310 per site with the
+// library's expm1 and divisions and row-by-row stencil sums, its FP64 pipe
+// 80 % busy; 512^2 took 205 us a step, with this and the column sums of
+// force_sums_warp 144 us).  Outside the table
+// (-d / rho0 beyond [-3.4, 2.0]) and for non-finite d the library's expm1.
+__device__ __noinline__ double expm1_slow(double x);
+__device__ __forceinline__ double2 pexpm1_scaled(double2 d, double c, double inv_rho0,
+                                                 const double2* tab) {
+    double2 r;
+    int k[2];
+    bool ok = true;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        const double x = s ? d.y : d.x;
+        const double t = fma(x, c, 6755399441055744.0);   // 1.5 2^52: rounds to an integer
+        const double n = t - 6755399441055744.0;
+        (s ? r.y : r.x) = fma(x, c, -n);
+        k[s] = __double2loint(t) + kExpLo;
+        // |n| < 2^31 (the high word of 1.5 2^52, or one less), n in the table
+        ok = ok && (unsigned)(__double2hiint(t) - 0x4337ffff) <= 1u && (unsigned)k[s] < (unsigned)kExpN;
+    }
+    if (!ok) return make_double2(expm1_slow(-d.x * inv_rho0), expm1_slow(-d.y * inv_rho0));
+    double2 p = pset(0x1.430912f86c787p-49);              // (ln2/64)^j / j!, j = 6 .. 1
+    p = pfma(p, r, pset(0x1.5d87fe78a6731p-40));
+    p = pfma(p, r, pset(0x1.3b2ab6fba4e77p-31));
+    p = pfma(p, r, pset(0x1.c6b08d704a0c0p-23));
+    p = pfma(p, r, pset(0x1.ebfbdff82c58fp-15));
+    p = pfma(p, r, pset(0x1.62e42fefa39efp-7));
+    p = pmul(p, r);
+    const double2 ta = tab[k[0]], tb = tab[k[1]];
+    return make_double2(fma(ta.x, p.x, ta.y), fma(tb.x, p.y, tb.y));
+}
+// exp(x) - 1 of a pair in FP32: branch-free, by the Cody-Waite reduction x = k ln2 + r (|r| <= ln2 / 2, ln2 split into a
 // 16-bit head and a tail so that k * head is exact) and
 // expm1(x) = 2^k expm1(r) + (2^k - 1), with expm1(r) from its Taylor series
 // through r^7 / 7! (truncation below 1.6e-8 relative on |r| <= ln2 / 2).
@@ -177,7 +224,6 @@ __device__ __forceinline__ float recip(float v) {
 // number, k in [-126, 127]): adding 1.5 2^23 to x log2(e) rounds it to an
 // integer held in the low mantissa bits, which also give 2^k's exponent
 // field by one shift.
-__device__ __forceinline__ double2 pexpm1(double2 v) { return make_double2(expm1(v.x), expm1(v.y)); }
 __device__ __forceinline__ float2 pexpm1(float2 x) {
     const float2 xc = make_float2(fminf(fmaxf(x.x, -87.0f), 88.0f), fminf(fmaxf(x.y, -87.0f), 88.0f));
     const float2 kt = pfma(xc, pset(1.44269504088896341f), pset(12582912.0f));
@@ -237,7 +283,10 @@ struct Layout {
     static constexpr int STAGE_FULL = 9 * TY * TX * (int)sizeof(T2);
     static constexpr bool STAGED = STAGE_OFF + STAGE_FULL + 128 <= 227 * 1024 - 1024;
     static constexpr int STAGE_BYTES = STAGED ? STAGE_FULL : 0;
-    static constexpr int SMEM = STAGE_OFF + STAGE_BYTES + 128;
+    // FP64: the exponential table (pexpm1_scaled)
+    static constexpr int TAB_OFF = STAGE_OFF + STAGE_BYTES;
+    static constexpr int TAB_BYTES = P == LB_FP64 ? kExpN * (int)sizeof(double2) : 0;
+    static constexpr int SMEM = TAB_OFF + TAB_BYTES + 128;
     // staging slot (plane 0) of tile row ly, column lx: planes of a half are
     // 8 TX pairs apart
     static __host__ __device__ constexpr int stage_off(int ly, int lx) {

@@ -319,7 +319,7 @@ lb_status lb_plan_partition(const lb_params* ps, int32_t nlat, int32_t seg, int3
  * not call cudaMalloc -- for instance code that runs inside a fixed device
  * arena it cannot grow, or inside a framework that forbids allocation on its
  * hot path.  It is the mass/momentum reduction of lb_stress (FP64 warp sums,
- * one slot per CTA, the last CTA adds the slots in a fixed order) run on
+ * one slot per CTA, added in a fixed order) run on
  * fields the caller passes in.
  *
  * Inputs: device arrays rho_A, rho_B, ux, uy of nx * ny FP64 values each
@@ -329,14 +329,13 @@ lb_status lb_plan_partition(const lb_params* ps, int32_t nlat, int32_t seg, int3
  * (a cudaStream_t, NULL = default stream).  Returns LB_ERR_INVALID for a NULL
  * pointer, nx or ny < 1, or nx * ny > LB_NOALLOC_MAX_SITES.
  *
- * Scratch: the per-CTA slots and the arrival counter live in one static
- * device array of 128 KB + 256 B that every GPU which loads the library keeps
- * until the process exits.  The first call on a device looks up that array's
- * device address (cudaGetSymbolAddress); make that first call before any
- * stream capture.  The address is kept per device and context: after a
- * cudaDeviceReset the next call on the new context looks it up again (and is
- * then again a first call).  Each call clears the counter with cudaMemsetAsync on
- * `stream` and overwrites the slots it uses.  All calls on a device share the
+ * Scratch: the per-CTA slots live in one static device array of 19 KB that
+ * every GPU which loads the library keeps until the process exits.  The first
+ * call on a device looks up that array's device address
+ * (cudaGetSymbolAddress); make that first call before any stream capture.  The
+ * address is kept per device and context: after a cudaDeviceReset the next
+ * call on the new context looks it up again (and is then again a first call).
+ * Each call overwrites the slots it uses.  All calls on a device share the
  * array, so calls whose kernels may overlap on the GPU (different streams with
  * no ordering between them) race: order them on one stream or with events. */
 lb_status lb_totals_noalloc(int32_t nx, int32_t ny, const double* rho_A, const double* rho_B,

@@ -174,9 +174,11 @@ lb_status lb_step(lb_handle* h, int64_t n) {
     if (!h->lat.inited) return LB_ERR_STATE;
     nvtxRangePushA("lb_step");   // a profiler range around the launches (free without a tool)
     lb_status s = LB_OK;
-    for (int64_t k = 0; k < n && s == LB_OK; ++k) {
-        s = launch_run(h->launch, h->stream);
-        if (s == LB_OK) lattice_advanced(h->lat, 1);
+    while (n > 0 && s == LB_OK) {
+        const int w = n < (1 << 20) ? (int)n : 1 << 20;
+        s = launch_window(h->launch, w, h->stream);
+        if (s == LB_OK) lattice_advanced(h->lat, w);
+        n -= w;
     }
     nvtxRangePop();
     return s;

@@ -333,8 +333,6 @@ static void fill_desc(LatDesc<C>& d, const Lattice& L, const Coef<C>& k, int nti
     d.nstrips = L.nstrips;
     d.ntiles_y = ntiles;
     d.stress_every = L.p.stress_every;
-    d.stress_t0 = L.p.stress_t0;
-    d.inv_nx = 1.0 / L.p.nx;
 }
 
 size_t launch_area_doubles(size_t tiles, size_t strips, int sms) {
@@ -643,9 +641,17 @@ lb_status launch_build(Launch& Ln, Lattice* const* lats, int nlat, void* descs, 
     return LB_OK;
 }
 
-lb_status launch_run(const Launch& Ln, cudaStream_t s) {
+lb_status launch_run(Launch& Ln, int step_k, int advance, cudaStream_t s) {
+    Ln.ad.step_k = Ln.af.step_k = step_k;
+    Ln.ad.advance = Ln.af.advance = advance;
     const void* args = Ln.precision == LB_FP64 ? (const void*)&Ln.ad : (const void*)&Ln.af;
     return cuda_status(launch_step(Ln.precision, args, Ln.variant, Ln.spt, Ln.grid, s));
+}
+
+lb_status launch_window(Launch& Ln, int n, cudaStream_t s) {
+    lb_status st = LB_OK;
+    for (int k = 0; k < n && st == LB_OK; ++k) st = launch_run(Ln, k, k == n - 1 ? n : 0, s);
+    return st;
 }
 
 static lb_status lattice_observe_pull(Lattice& L, int obs, double* out, int q0, int q1, int pull,
@@ -671,6 +677,8 @@ static lb_status lattice_observe_pull(Lattice& L, int obs, double* out, int q0, 
         a.obs_out = out;
         a.q0 = q0;
         a.q1 = q1;
+        a.wsum = L.wsum;
+        a.nstrips = L.nstrips;
         e = launch_observe(L.p.precision, &L.tobs[L.cur], &a, grid, s);
     } else {
         StepArgs<float> a;
@@ -684,6 +692,8 @@ static lb_status lattice_observe_pull(Lattice& L, int obs, double* out, int q0, 
         a.obs_out = out;
         a.q0 = q0;
         a.q1 = q1;
+        a.wsum = L.wsum;
+        a.nstrips = L.nstrips;
         e = launch_observe(L.p.precision, &L.tobs[L.cur], &a, grid, s);
     }
     return cuda_status(e);
@@ -709,6 +719,8 @@ static long long first_sample(const lb_params& p, long long t) {
 
 static lb_status lattice_reset(Lattice& L, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(L.st, 0, sizeof(DevStats), s);   // t = 0, cur = 0, pull = 0
+    if (e == cudaSuccess && !L.g.periodic)   // the wall momentum totals restart
+        e = cudaMemsetAsync(L.wsum, 0, 2 * sizeof(double) * (size_t)L.nstrips, s);
     L.next_sample = first_sample(L.p, 0);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(&L.st->next_sample, &L.next_sample, sizeof(long long), cudaMemcpyHostToDevice, s);

@@ -19,7 +19,7 @@ struct Lattice {
     DevStats* st;
     double* slots;           // observe partial sums, 4 per tile
     char* wallx;             // the step's wall-momentum pairs: [2][nx] (bottom, top), compute type
-    double* wsum;            // their per-strip sums: [2][nstrips]
+    double* wsum;            // their sums per strip and over the sampled steps: [2][nstrips]
     char* fbuf[2];
     size_t fbytes;
     CUtensorMap tblock[2];   // step kernel: 8-row block loads of buffer b
@@ -83,7 +83,12 @@ lb_status launch_build(Launch& Ln, Lattice* const* lats, int nlat, void* descs, 
                        unsigned int* ticket, int sms, cudaStream_t stream, void* host_scratch,
                        int seg = 0, int spt = 1);
 size_t launch_area_doubles(size_t tiles, size_t strips, int sms);
-lb_status launch_run(const Launch& Ln, cudaStream_t s);
+// Enqueue step step_k of a window of consecutive steps (0-based); advance: the
+// window's steps on its last launch, else 0.  The device's step counters move
+// with the window's last launch only.
+lb_status launch_run(Launch& Ln, int step_k, int advance, cudaStream_t s);
+// Enqueue n steps as one window (n < 2^30).
+lb_status launch_window(Launch& Ln, int n, cudaStream_t s);
 
 lb_status lattice_init_seeded(Lattice& L, uint64_t seed, cudaStream_t s);
 lb_status lattice_init_fields(Lattice& L, const double* rho_A, const double* rho_B,

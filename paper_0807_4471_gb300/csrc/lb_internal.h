@@ -17,15 +17,15 @@ struct DevStats {
     unsigned int err;       // bit 0: non-finite density, bit 1: TMA wait timeout
     unsigned int ticket;    // CTA arrival counter of the observe reductions
     long long t;            // completed time steps
-    double sum_bot;         // sum of per-step bottom-wall samples
-    double sum_top;         // sum of per-step top-wall samples
+    double sum_bot;         // sum of the bottom-wall samples, as of the last observe pass
+    double sum_top;         // sum of the top-wall samples
     long long samples;      // number of samples in the sums
     double totals[4];       // last observe pass: mass_A, mass_B, mom_x, mom_y
     int cur;                // buffer holding the current state (0 or 1)
     int pull;               // 1: it holds post-collision f*(t-1); 0: f(t) in place
     long long next_sample;  // the next step whose wall momentum is sampled
                             // (stress_t0 + k stress_every >= t; set by the host
-                            // with t, advanced by the kernel)
+                            // with t, advanced by the kernel with t)
     double pad_[5];
 };
 static_assert(sizeof(DevStats) == 128, "DevStats is one 128-byte line");
@@ -135,12 +135,11 @@ struct alignas(128) LatDesc {
     DevStats* st;
     void* wallx;           // [2][nx] compute-type pairs: x-momentum handed to the bottom
                            // (then top) wall by the links leaving site x, this step
-    double* wsum;          // [2][nstrips]: those summed per strip (bottom, then top)
+    double* wsum;          // [2][nstrips]: those summed per strip (bottom, then top) and
+                           // over the sampled steps
     int nstrips;           // ceil(nx / TX)
     int ntiles_y;          // tile rows of the launch's tile shape
     int stress_every;
-    long long stress_t0;
-    double inv_nx;         // 1 / nx: the wall samples are momentum per unit length
 };
 
 // Arguments of the (multi-lattice) step kernel.
@@ -155,6 +154,10 @@ struct BatchArgs {
     const int4* items;
     const int* cta_items;
     unsigned int* ticket;       // CTA arrival counter of the launch (zero between launches)
+    // Launches come in windows of consecutive steps: this one takes step
+    // DevStats::t + step_k, and the window's last one has advance = the
+    // window's steps (else 0), by which it moves the lattices' counters.
+    int step_k, advance;
     int l2_resident;            // one buffer of all lattices fits in L2: cache-policy hints
     int early_release;          // kernel variant bit 2 only: a tile's ring slots are refilled
                                 // after its density phase (else after its site phase)
@@ -174,8 +177,8 @@ struct StepArgs {
     int obs;               // ObsKind; OBS_NONE = a time step
     double* obs_out;       // observe output base
     int q0, q1;            // OBS_POPS: planes [q0, q1) written
-    long long stress_t0;
-    int stress_every;
+    const double* wsum;    // Couette: the strips' wall momentum totals, [2][nstrips]
+    int nstrips;
 };
 
 // Host-side launch helpers (lb_dispatch.cu).

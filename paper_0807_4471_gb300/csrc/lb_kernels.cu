@@ -24,7 +24,7 @@
 //     (staging tile + TMA bulk tensor store, or direct stores) and the
 //     periodic ghost copies.
 //  4. Couette: the wall sites' momentum exchange, summed per strip in FP64
-//     after the tile loop; the last CTA takes the wall samples.
+//     after the tile loop and, at sampled steps, added to the strip's total.
 // There is no dense contraction anywhere, so no tensor cores are used.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -57,6 +57,9 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
                  "r"(bytes)
                  : "memory");
+}
+__device__ __forceinline__ void tma_prefetch_map(const CUtensorMap* map) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int x, int y,
                                             int z, uint64_t* bar) {
@@ -727,15 +730,18 @@ __device__ __forceinline__ void site_update(
     }
 }
 
-// Wall momentum of one CTA's items that hold a wall row, in FP64: the
-// wall-site values the site phase left in the lattice's wall columns, summed
-// over the item's strip in a fixed order (lane l takes columns l, l + 32,
-// ..., then the butterfly), one warp per item -- so the sums do not depend
-// on the partition or the tile shape.
-template <int P, int SPT>
+// Wall momentum of one CTA's items that hold a wall row, in FP64, at the
+// lattices' sampled steps: the wall-site values the site phase left in the
+// lattice's wall columns, summed over the item's strip in a fixed order (lane l
+// takes columns l, l + 32, ..., then the butterfly), one warp per item, and
+// added to the strip's running total -- so the totals do not depend on the
+// partition or the tile shape, and no CTA has to wait for the others' sums.
+// Sampled steps: stress_t0 + k stress_every; DevStats::next_sample is the
+// first one from the window's start on (32-bit remainder: a window is short,
+// and a 64-bit one would compile to a call).
+template <int P, class L>
 __device__ __forceinline__ void wall_sums(const BatchArgs<typename Prec<P>::C>& a, int it0, int it_end,
                                        int tid) {
-    typedef Layout<P, SPT> L;
     typedef typename L::C C;
     typedef typename L::C2 C2;
     const int lane = tid & 31, warp = tid >> 5;
@@ -746,6 +752,8 @@ __device__ __forceinline__ void wall_sums(const BatchArgs<typename Prec<P>::C>& 
         const bool bot = w.z == 0, top = w.w == d->ntiles_y;
         if (d->g.periodic || !(bot || top)) continue;
         if (n++ % (L::NT / 32) != warp) continue;
+        const long long since = d->st->t + a.step_k - d->st->next_sample;
+        if (since < 0 || (unsigned)since % (unsigned)d->stress_every != 0u) continue;
         const int nx = d->g.nx;
         const int xe = min(w.y * L::TX + L::TX, nx);
         const C2* wx = reinterpret_cast<const C2*>(d->wallx);
@@ -757,58 +765,28 @@ __device__ __forceinline__ void wall_sums(const BatchArgs<typename Prec<P>::C>& 
         sb = warp_sum(sb);
         st = warp_sum(st);
         if (lane == 0) {
-            if (bot) d->wsum[w.y] = sb;
-            if (top) d->wsum[d->nstrips + w.y] = st;
+            if (bot) d->wsum[w.y] += sb;
+            if (top) d->wsum[d->nstrips + w.y] += st;
         }
     }
 }
 
-// The last CTA of a step launch: the Couette wall samples, one warp per
-// lattice, then every lattice's step counter and buffer parity, one thread
-// per lattice.  t0, cur0: the step counter and buffer of lattice tid,
-// loaded by every CTA before its arrival (they change only between
-// launches), so the counters take no load on the launch's tail.
-template <int P, bool ALLPER, int NT>
-__device__ __forceinline__ void advance_lattices(const BatchArgs<typename Prec<P>::C>& a, int tid,
-                                                 long long t0, int cur0) {
-    typedef typename Prec<P>::C C;
-    if constexpr (!ALLPER) {
-        // Strip sums in a fixed order -- lane l adds strips l, l + 32, ...,
-        // then a butterfly over the lanes -- so they do not depend on the
-        // partition; FP64 has a long latency on this GPU, so no serial chain
-        // runs over the strips.  Sampled steps: stress_t0 + k stress_every,
-        // tracked by next_sample (no 64-bit remainder: it would compile to a
-        // call, which burdens the whole kernel's register allocation).
-        const int lane = tid & 31;
-        for (int l = tid >> 5; l < a.nlat; l += NT / 32) {
-            const LatDesc<C>* d = &a.lat[l];
-            if (d->g.periodic) continue;
-            DevStats* st = d->st;
-            const int ns = d->nstrips;
-            const volatile double* ws = d->wsum;
-            double sb = 0.0, stp = 0.0;
-            for (int i = lane; i < ns; i += 32) {
-                sb += ws[i];
-                stp += ws[ns + i];
-            }
-            sb = warp_sum(sb);
-            stp = warp_sum(stp);
-            const long long t = st->t;
-            if (lane == 0 && t == st->next_sample) {
-                st->sum_bot += sb * d->inv_nx;
-                st->sum_top += stp * d->inv_nx;
-                st->samples += 1;
-                st->next_sample = t + (d->stress_every > 0 ? d->stress_every : 1);
-            }
-        }
-        __syncthreads();   // the samples have read the step counters
-    }
+// The last CTA of a window's last launch: every lattice's step counter, buffer
+// parity and wall-sample schedule, one thread per lattice.
+template <int NT, typename C>
+__device__ __forceinline__ void advance_lattices(const BatchArgs<C>& a, int tid) {
     for (int l = tid; l < a.nlat; l += NT) {
-        DevStats* st = a.lat[l].st;
-        const long long t = l == tid ? t0 : st->t;
-        const int cur = l == tid ? cur0 : st->cur;
-        st->t = t + 1;
-        st->cur = cur ^ 1;
+        const LatDesc<C>* d = &a.lat[l];
+        DevStats* st = d->st;
+        const long long t = st->t + a.advance, next = st->next_sample;
+        if (!d->g.periodic && t > next) {   // samples taken in the window
+            const unsigned every = (unsigned)d->stress_every;
+            const unsigned m = ((unsigned)(t - next) + every - 1u) / every;
+            st->samples += m;
+            st->next_sample = next + (long long)m * every;
+        }
+        st->t = t;
+        st->cur ^= a.advance & 1;
         st->pull = 1;
     }
 }
@@ -909,8 +887,8 @@ __device__ __forceinline__ void block_sum4(double red[4], double (*s_red)[4]) {
 // lattice edge, and tiles near an edge then write the periodic ghost
 // copies; where the staging tile does not fit beside the ring (FP32 with
 // 16-row tiles) the threads store their sites and ghost copies to global
-// memory themselves.  The last CTA to finish advances every lattice's step
-// counter and buffer parity and takes the Couette wall samples.
+// memory themselves.  The last CTA of a window's last launch advances every
+// lattice's step counter and buffer parity.
 // V: bit 0 = every lattice periodic (no wall code); bit 1 = general forcing;
 // bit 2 = omega = 1 for both species (the site phase reads no populations).
 template <int P, int V, int SPT>
@@ -991,12 +969,14 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
         s_pol[1] = a.l2_resident ? policy_evict_last() : policy_evict_normal();
     }
     __syncthreads();
-    // Up to here only shared memory and the host-built item tables were
-    // touched; the lattice state (DevStats, populations) written by the
-    // previous step is read after the wait.  The next step's CTAs may then
-    // take each SM as soon as this CTA leaves it (one CTA fills an SM).
-    griddep_wait();
-    griddep_launch_dependents();
+    // Before the wait only shared memory, the host-built tables and, after a
+    // window's first launch, the lattices' counters are read: the previous
+    // launch of the window leaves the counters alone, and the launch before it
+    // has completed.  Everything else of the lattice state is read after the
+    // wait.  The next step's CTAs may then take each SM as soon as this CTA
+    // leaves it (one CTA fills an SM).
+    const int step_k = a.step_k;
+    if (step_k == 0) griddep_wait();
 
     // Producer (thread 0): the blocks of this CTA's items, in order.  Item
     // tiles [ty_a, ty_b) need blocks SPT ty_a .. SPT ty_b (block j = padded
@@ -1012,7 +992,8 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
         p_x0 = w.y * L::TX;
         p_ty_a = w.z;
         p_nblk = SPT * (w.w - w.z) + 1;
-        p_map = &d->tin[*((volatile int*)&d->st->cur)];
+        p_map = &d->tin[*((volatile int*)&d->st->cur) ^ (step_k & 1)];
+        tma_prefetch_map(p_map);
     };
     auto issue_next = [&]() -> bool {
         if (p_item >= it_end) return false;
@@ -1030,6 +1011,8 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
         return true;
     };
     if (tid == 0) p_load();
+    if (step_k != 0) griddep_wait();
+    griddep_launch_dependents();
     if (tid == 0)
         while (p_pos < L::NB && issue_next()) {}
     int ty_b = 0, ty = 0;   // the consumer's item end and tile (read by release)
@@ -1053,10 +1036,11 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
         const Geom g = d->g;
         const LatVals<C> v = d->v;
         const bool per_lat = ALLPER || g.periodic;
-        const int cur = *((volatile int*)&d->st->cur);
-        const int pull = *((volatile int*)&d->st->pull);
-        // the step counter advances only after every CTA of the launch is done
-        const uint32_t key = hash32((uint32_t)*((volatile long long*)&d->st->t) * 0x9e3779b9u);
+        // the counters advance only after every CTA of a window's last launch is done
+        const int cur = *((volatile int*)&d->st->cur) ^ (step_k & 1);
+        const int pull = step_k != 0 ? 1 : *((volatile int*)&d->st->pull);
+        const uint32_t key =
+            hash32(((uint32_t)*((volatile long long*)&d->st->t) + (uint32_t)step_k) * 0x9e3779b9u);
         T2* fout = reinterpret_cast<T2*>(d->fbuf[cur ^ 1]);
         C2 nf = pset(C(0));   // 0 * rho over the item's sites: NaN at a non-finite density
         // ring slot and phase parity of the tile's first block, kept as the
@@ -1304,8 +1288,8 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
     // the generic variant 1-4 % even on periodic lattices, which skip it.
     if constexpr (!ALLPER) {
         __syncthreads();   // this CTA's wall-site values are written
-        if (!s_fail) wall_sums<P, SPT>(a, a.cta_items[blockIdx.x], it_end, tid);
-    }   // (the barrier before the arrival orders the sums before it)
+        if (!s_fail) wall_sums<P, L>(a, a.cta_items[blockIdx.x], it_end, tid);
+    }
     if (STAGED && tid == kStoreThread) bulk_wait_all();
     if (s_fail && tid == 0) {
         // Let copies in flight land before the CTA exits.  No slot is
@@ -1319,20 +1303,18 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
     if (s_fail && tid == 0)   // report on every lattice of the launch
         for (int l = 0; l < a.nlat; ++l) atomicOr(&a.lat[l].st->err, ERR_TIMEOUT);
 
-    // The last CTA advances every lattice and takes the wall samples.  Its
-    // step counters are loaded by every CTA now, off the launch's tail.
-    long long t0 = 0;
-    int cur0 = 0;
-    if (tid < a.nlat) {
-        const DevStats* st = a.lat[tid].st;
-        t0 = *((volatile const long long*)&st->t);
-        cur0 = *((volatile const int*)&st->cur);
-    }
+    // A window's last launch advances the lattices, by its last CTA; the other
+    // launches need no arrival counter.  That and the set-up ahead of the wait
+    // took a step of one 128^2 FP32 lattice from 8.2 to 6.1 us (its counter's
+    // round trip, the last CTA's work and four dependent loads before the first
+    // block load), 300 x 211 Couette from 11.8 to 9.0, the 5 x 512^2 sweep from
+    // 35.0 to 33.3.
+    if (!a.advance) return;
     __syncthreads();   // this CTA's writes (wall sums, timeout flags) precede its arrival
     if (tid == 0) s_last = ticket_arrive(a.ticket) == (unsigned int)(G - 1);
     __syncthreads();
     if (!s_last) return;
-    advance_lattices<P, ALLPER, L::NT>(a, tid, t0, cur0);
+    advance_lattices<L::NT>(a, tid);
     // no other CTA of the launch touches the ticket again; the next launch
     // reads it after this one has completed
     if (tid == 0) *a.ticket = 0u;
@@ -1452,6 +1434,21 @@ __global__ void __launch_bounds__(Layout<P>::NT)
 #pragma unroll
     for (int q = 0; q < 4; ++q) red[q] = w[q];
     block_sum4<L::NT>(red, s_red);
+    // the wall momentum totals: the strips' running totals, in a fixed order
+    // (lane l adds strips l, l + 32, ..., then the butterfly)
+    if (tid < 32 && !a.g.periodic) {
+        double sb = 0.0, st = 0.0;
+        for (int i = tid; i < a.nstrips; i += 32) {
+            sb += a.wsum[i];
+            st += a.wsum[a.nstrips + i];
+        }
+        sb = warp_sum(sb);
+        st = warp_sum(st);
+        if (tid == 0) {
+            a.st->sum_bot = sb * (1.0 / a.g.nx);
+            a.st->sum_top = st * (1.0 / a.g.nx);
+        }
+    }
     if (tid == 0) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) a.st->totals[q] = red[q];

@@ -177,8 +177,7 @@ lb_status capture_graph(lb_pool* P) {
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(P->stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_status(e);
-    lb_status s = LB_OK;
-    for (int i = 0; i < kGraphChunk && s == LB_OK; ++i) s = launch_run(P->launch, P->stream);
+    lb_status s = launch_window(P->launch, kGraphChunk, P->stream);
     e = cudaStreamEndCapture(P->stream, &g);
     if (s != LB_OK) {
         if (g) cudaGraphDestroy(g);
@@ -202,11 +201,7 @@ lb_status run_steps(lb_pool* P, long long k) {
         if (e != cudaSuccess) return cuda_status(e);
         k -= kGraphChunk;
     }
-    for (long long i = 0; i < k; ++i) {
-        lb_status s = launch_run(P->launch, P->stream);
-        if (s != LB_OK) return s;
-    }
-    return LB_OK;
+    return launch_window(P->launch, (int)k, P->stream);
 }
 
 void advanced(lb_pool* P, long long k) {

@@ -63,12 +63,13 @@ lb_status create_common(const lb_params* p, void* stream, void* ws, size_t bytes
     if (s == LB_OK) {
         Lattice* one = &h->lat;
         alignas(128) unsigned char scratch[sizeof(LatDesc<double>)];
-        const int spt = p->tile_rows == 0 ? default_spt(p->precision)
-                                           : p->tile_rows / kernel_tile_y(p->precision);
+        const int sms = device_sms(h->device);
+        const int shape = shape_of_rows(p->precision, p->tile_rows,
+                                        (long long)one->nstrips * one->ntiles_y, sms);
         s = launch_build(h->launch, &one, 1, h->ws + H.desc,
                          reinterpret_cast<double*>(h->ws + H.slots),
-                         reinterpret_cast<unsigned int*>(h->ws + H.ticket), device_sms(h->device),
-                         h->stream, scratch, 0, spt);
+                         reinterpret_cast<unsigned int*>(h->ws + H.ticket), sms, h->stream, scratch,
+                         0, shape);
     }
     if (s != LB_OK) {
         if (owns) cudaFree(ws);

@@ -22,16 +22,16 @@ int kernel_smem_obs_bytes(int p) { LB_SWITCH(p, return Layout<P>::SMEM_OBS) retu
 int kernel_block_rows(int p) { LB_SWITCH(p, return Layout<P>::TYB) return 0; }
 int kernel_scale_log2(int p) { LB_SWITCH(p, return Prec<P>::SCALE_LOG2) return 0; }
 template <int P>
-static int staged_of(int spt) {
-    if constexpr (Prec<P>::NB2 > 0)
-        if (spt == 2) return Layout<P, 2>::STAGED ? 1 : 0;
-    return Layout<P, 1>::STAGED ? 1 : 0;
+static int staged_of(int shape) {
+    if constexpr (has_shape(P, SHAPE_16))
+        if (shape == SHAPE_16) return Layout<P, SHAPE_16>::STAGED ? 1 : 0;
+    return 1;
 }
-int kernel_staged(int p, int spt) { LB_SWITCH(p, return staged_of<P>(spt)) return 1; }
+int kernel_staged(int p, int shape) { LB_SWITCH(p, return staged_of<P>(shape)) return 1; }
 
-cudaError_t launch_step(int precision, const void* args, int variant, int spt, dim3 grid,
+cudaError_t launch_step(int precision, const void* args, int variant, int shape, dim3 grid,
                         cudaStream_t s) {
-    LB_SWITCH(precision, return launch_step_prec<P>(args, variant, spt, grid, s))
+    LB_SWITCH(precision, return launch_step_prec<P>(args, variant, shape, grid, s))
     return cudaErrorInvalidValue;
 }
 

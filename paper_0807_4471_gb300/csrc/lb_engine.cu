@@ -291,17 +291,22 @@ int choose_seg(const int* nstrips, const int* ntiles_y, int nlat, int G) {
         for (int l = 0; l < nlat; ++l) items += (long long)nstrips[l] * ((ntiles_y[l] + seg - 1) / seg);
         const int g = items < G ? (int)items : G;
         if (g <= 0) continue;
+        // equal items go round the CTAs: whole rounds count once, for all
         cost.assign((size_t)g, 0.0);
+        double all = 0.0;
         long long it = 0;
+        auto deal = [&](long long n, double c) {
+            all += (double)(n / g) * c;
+            for (long long k = 0; k < n % g; ++k) cost[(size_t)((it + k) % g)] += c;
+            it += n;
+        };
         for (int l = 0; l < nlat; ++l) {
-            const int nseg = (ntiles_y[l] + seg - 1) / seg;
-            for (int sg = 0; sg < nseg; ++sg) {
-                const int size = (sg + 1) * seg <= ntiles_y[l] ? seg : ntiles_y[l] - sg * seg;
-                for (int sx = 0; sx < nstrips[l]; ++sx, ++it) cost[(size_t)(it % g)] += size + 0.25;
-            }
+            deal((long long)nstrips[l] * (ntiles_y[l] / seg), seg + 0.25);
+            if (ntiles_y[l] % seg) deal(nstrips[l], ntiles_y[l] % seg + 0.25);
         }
         double mx = 0.0;
         for (double c : cost) mx = c > mx ? c : mx;
+        mx += all;
         if (mx <= best) {
             best = mx;
             best_seg = seg;
@@ -310,11 +315,26 @@ int choose_seg(const int* nstrips, const int* ntiles_y, int nlat, int G) {
     return best_seg;
 }
 
-int max_spt(int precision) { return precision == LB_FP64 ? 1 : 2; }
-int default_spt(int precision) { return max_spt(precision); }
-int tiles_y(const Lattice& L, int spt) {
-    const int ty = kernel_tile_y(L.p.precision) * spt;
+int tiles_y(const Lattice& L, int shape) {
+    const int ty = shape_rows(shape);
     return (L.p.ny + ty - 1) / ty;
+}
+// Default tile shape of a lattice set with `tiles8` 8-row tiles.  The 16-bit
+// formats: two CTAs per SM, except where the tiles do not even fill one CTA
+// per SM one and a half times over; a thread's single site then finishes a
+// tile sooner (256^2 FP16, 160 tiles: 6.3 us a step against 6.9; 512^2, 576
+// tiles: 11.0 against 9.7).  FP32: the 16-row tile beyond the same line
+// (256^2: 6.5 us with 8 rows, 7.3 with 16; 512^2: 11.2 and 10.2).
+int default_shape(int precision, long long tiles8, int sms) {
+    if (precision == LB_FP64 || 2 * tiles8 <= 3LL * sms) return SHAPE_8;
+    return has_shape(precision, SHAPE_8X2) ? SHAPE_8X2 : SHAPE_16;
+}
+int shape_of_rows(int precision, int rows, long long tiles8, int sms) {
+    if (rows == 0) return default_shape(precision, tiles8, sms);
+    if (rows == 16) return has_shape(precision, SHAPE_16) ? SHAPE_16 : 0;
+    if (rows != 8) return 0;
+    const int d = default_shape(precision, tiles8, sms);
+    return d == SHAPE_8X2 ? d : SHAPE_8;
 }
 
 template <typename C>
@@ -336,8 +356,8 @@ static void fill_desc(LatDesc<C>& d, const Lattice& L, const Coef<C>& k, int nti
 }
 
 size_t launch_area_doubles(size_t tiles, size_t strips, int sms) {
-    // items (int4, at most one per tile and strip) | CTA offsets
-    return 2 * (tiles + strips) + ((size_t)sms + 2) / 2 + 8;
+    // items (int4, at most one per 8-row tile and strip) | CTA offsets
+    return 2 * (tiles + strips) + (2 * (size_t)sms + 2) / 2 + 8;   // at most two CTAs per SM
 }
 
 namespace {
@@ -351,14 +371,14 @@ struct Item {
 // seg < 0: the tiles of all lattices in strip order (lattice, strip, tile
 // row) cut into G contiguous runs of equal estimated cost, each run cut
 // again at strip boundaries: every CTA walks one or two strips.
-void partition(Lattice* const* lats, int nlat, int seg, int spt, int sms, std::vector<Item>& items,
+void partition(Lattice* const* lats, int nlat, int seg, int shape, int sms, std::vector<Item>& items,
                std::vector<int>& cta, int* grid) {
     items.clear();
     cta.clear();
     std::vector<int> nty((size_t)nlat);
     long long tiles = 0;
     for (int l = 0; l < nlat; ++l) {
-        nty[(size_t)l] = tiles_y(*lats[l], spt);
+        nty[(size_t)l] = tiles_y(*lats[l], shape);
         tiles += (long long)lats[l]->nstrips * nty[(size_t)l];
     }
     // Tile costs relative to a full interior tile, fitted on GB300 to the
@@ -371,7 +391,7 @@ void partition(Lattice* const* lats, int nlat, int seg, int spt, int sms, std::v
     // rows) 0.8 of a tile.
     auto cost = [&](int l, int sx, int ty) {
         const Lattice& L = *lats[l];
-        const int tx = kernel_tile_x(L.p.precision), tyy = kernel_tile_y(L.p.precision) * spt;
+        const int tx = kernel_tile_x(L.p.precision), tyy = shape_rows(shape);
         const int x0 = sx * tx, y0 = ty * tyy;
         const bool full = x0 + tx <= L.p.nx && y0 + tyy <= L.p.ny;
         if (!full) return 1.07;
@@ -379,7 +399,7 @@ void partition(Lattice* const* lats, int nlat, int seg, int spt, int sms, std::v
         if (!per && (y0 == 0 || y0 + tyy >= L.p.ny)) return 1.38;
         double c = 1.0;
         if (x0 < 3 || x0 + tx > L.p.nx - 3) c += 0.21;
-        if (per && (y0 < 3 || y0 + tyy > L.p.ny - 3)) c += kernel_staged(L.p.precision, spt) ? 0.25 : 0.02;
+        if (per && (y0 < 3 || y0 + tyy > L.p.ny - 3)) c += kernel_staged(L.p.precision, shape) ? 0.25 : 0.02;
         return c;
     };
     const double kItemStart = 0.8;
@@ -493,9 +513,10 @@ void partition(Lattice* const* lats, int nlat, int seg, int spt, int sms, std::v
 // ~40 tiles of 8 rows (measured faster on 512^2-1024^2 lattices), the
 // load-balance model's dealt segments beyond (their CTAs sweep a band of
 // rows together, which keeps the halo columns in L2 on large lattices);
-// `tiles` counts tiles of 8 spt rows.
-static int default_seg(long long tiles, int spt, const int* ns, const int* nt, int nlat, int sms) {
-    return tiles * spt <= 40LL * sms ? -1 : choose_seg(ns, nt, nlat, sms);
+// `tiles` counts tiles of the shape, `ctas` the launch's CTAs.
+static int default_seg(long long tiles, int shape, const int* ns, const int* nt, int nlat, int sms,
+                       int ctas) {
+    return tiles * shape_rows(shape) <= 8LL * 40 * sms ? -1 : choose_seg(ns, nt, nlat, ctas);
 }
 
 // Host-only plan of a launch's work items (lb_plan_partition).
@@ -507,10 +528,9 @@ lb_status plan_partition(const lb_params* ps, int nlat, int seg, int tile_rows, 
     std::vector<Lattice*> lp((size_t)nlat);
     std::vector<int> ns((size_t)nlat), nt((size_t)nlat);
     if (validate_params(&ps[0]) != LB_OK) return LB_ERR_INVALID;
-    const int ty8 = kernel_tile_y(ps[0].precision);
-    if (tile_rows != 0 && tile_rows != ty8 && tile_rows != 2 * ty8) return LB_ERR_INVALID;
-    const int spt = tile_rows == 0 ? 1 : tile_rows / ty8;
-    if (spt > max_spt(ps[0].precision)) return LB_ERR_INVALID;
+    if (tile_rows != 0 && tile_rows != 8 && tile_rows != 16) return LB_ERR_INVALID;
+    const int shape = tile_rows == 16 ? SHAPE_16 : SHAPE_8;
+    if (!has_shape(ps[0].precision, shape)) return LB_ERR_INVALID;
     long long tiles = 0;
     for (int l = 0; l < nlat; ++l) {
         if (validate_params(&ps[l]) != LB_OK || ps[l].precision != ps[0].precision)
@@ -520,17 +540,17 @@ lb_status plan_partition(const lb_params* ps, int nlat, int seg, int tile_rows, 
         L.g = make_geom(&ps[l]);
         const int tx = kernel_tile_x(ps[l].precision);
         L.nstrips = (ps[l].nx + tx - 1) / tx;
-        L.ntiles_y = tiles_y(L, 1);
+        L.ntiles_y = tiles_y(L, SHAPE_8);
         lp[(size_t)l] = &L;
         ns[(size_t)l] = L.nstrips;
-        nt[(size_t)l] = tiles_y(L, spt);
+        nt[(size_t)l] = tiles_y(L, shape);
         tiles += (long long)L.nstrips * nt[(size_t)l];
     }
-    const int s = seg != 0 ? seg : default_seg(tiles, spt, ns.data(), nt.data(), nlat, sms);
+    const int s = seg != 0 ? seg : default_seg(tiles, shape, ns.data(), nt.data(), nlat, sms, sms);
     std::vector<Item> it;
     std::vector<int> c;
     int G = 0;
-    partition(lp.data(), nlat, s, spt, sms, it, c, &G);
+    partition(lp.data(), nlat, s, shape, sms, it, c, &G);
     const int cap_items = *nitems, cap_cta = *grid;
     *nitems = (int32_t)it.size();
     *grid = G;
@@ -548,16 +568,16 @@ lb_status plan_partition(const lb_params* ps, int nlat, int seg, int tile_rows, 
 
 lb_status launch_build(Launch& Ln, Lattice* const* lats, int nlat, void* descs, double* slots,
                        unsigned int* ticket, int sms, cudaStream_t stream, void* host_scratch,
-                       int forced_seg, int spt) {
+                       int forced_seg, int shape) {
     if (nlat < 1) return LB_ERR_INVALID;
     const int prec = lats[0]->p.precision;
-    if (spt < 1 || spt > max_spt(prec)) return LB_ERR_INVALID;
+    if (!has_shape(prec, shape)) return LB_ERR_INVALID;
     std::vector<int> ns((size_t)nlat), nt((size_t)nlat);
     bool allper = true, gen = false, tau1 = true;
     long long tiles = 0, strips = 0;
     for (int l = 0; l < nlat; ++l) {
         ns[(size_t)l] = lats[l]->nstrips;
-        nt[(size_t)l] = tiles_y(*lats[l], spt);
+        nt[(size_t)l] = tiles_y(*lats[l], shape);
         allper = allper && lats[l]->g.periodic;
         gen = gen || lats[l]->kd.source || lats[l]->kd.has_accel;
         // 1 - omega rounds to zero in the compute precision for both species:
@@ -568,11 +588,13 @@ lb_status launch_build(Launch& Ln, Lattice* const* lats, int nlat, void* descs, 
         tiles += (long long)lats[l]->nstrips * nt[(size_t)l];
         strips += lats[l]->nstrips;
     }
-    const int seg = forced_seg != 0 ? forced_seg : default_seg(tiles, spt, ns.data(), nt.data(), nlat, sms);
+    const int ctas = sms * shape_ctas(shape);
+    const int seg = forced_seg != 0 ? forced_seg
+                                    : default_seg(tiles, shape, ns.data(), nt.data(), nlat, sms, ctas);
     std::vector<Item> items;
     std::vector<int> cta;
     int grid = 0;
-    partition(lats, nlat, seg, spt, sms, items, cta, &grid);
+    partition(lats, nlat, seg, shape, ctas, items, cta, &grid);
     const int nitems = (int)items.size();
     const size_t dsz = prec == LB_FP64 ? sizeof(LatDesc<double>) : sizeof(LatDesc<float>);
     char* hs = reinterpret_cast<char*>(host_scratch);
@@ -598,7 +620,7 @@ lb_status launch_build(Launch& Ln, Lattice* const* lats, int nlat, void* descs, 
     if (e != cudaSuccess) return cuda_status(e);
     Ln.precision = prec;
     Ln.variant = (allper ? 1 : 0) | (gen ? 2 : 0) | (tau1 ? 4 : 0);
-    Ln.spt = spt;
+    Ln.shape = shape;
     Ln.grid = dim3((unsigned)grid, 1, 1);
     Ln.nitems = nitems;
     Ln.seg = seg;
@@ -645,7 +667,7 @@ lb_status launch_run(Launch& Ln, int step_k, int advance, cudaStream_t s) {
     Ln.ad.step_k = Ln.af.step_k = step_k;
     Ln.ad.advance = Ln.af.advance = advance;
     const void* args = Ln.precision == LB_FP64 ? (const void*)&Ln.ad : (const void*)&Ln.af;
-    return cuda_status(launch_step(Ln.precision, args, Ln.variant, Ln.spt, Ln.grid, s));
+    return cuda_status(launch_step(Ln.precision, args, Ln.variant, Ln.shape, Ln.grid, s));
 }
 
 lb_status launch_window(Launch& Ln, int n, cudaStream_t s) {

@@ -40,7 +40,7 @@ struct Lattice {
 struct Launch {
     int precision;
     int variant;             // bit 0: all periodic; bit 1: general forcing; bit 2: 1 - omega = 0
-    int spt;                 // sites per thread: tiles of 8 spt rows
+    int shape;               // tile shape (Shape)
     dim3 grid;
     int nitems, seg;
     BatchArgs<double> ad;
@@ -64,11 +64,12 @@ lb_status plan_partition(const lb_params* ps, int nlat, int seg, int tile_rows, 
 // Segment length (tiles per work item) minimising the most loaded CTA.
 int choose_seg(const int* nstrips, const int* ntiles_y, int nlat, int G);
 
-// Sites per thread of the step kernel: the tile shapes a precision has
-// (tiles of 8 spt rows), the library's default, and a lattice's tile rows.
-int max_spt(int precision);
-int default_spt(int precision);
-int tiles_y(const Lattice& L, int spt);
+// Tile rows of a lattice in a shape; the library's default shape for a set of
+// lattices with tiles8 8-row tiles in all; and the shape for a requested tile
+// height (0: the default; result 0: the precision has no such tile).
+int tiles_y(const Lattice& L, int shape);
+int default_shape(int precision, long long tiles8, int sms);
+int shape_of_rows(int precision, int rows, long long tiles8, int sms);
 
 // Write the lattices' descriptors to `descs` (device, 128-byte aligned, room
 // for nlat LatDesc<double>) through `host_scratch` (as large, host) and fill
@@ -78,10 +79,9 @@ int tiles_y(const Lattice& L, int spt);
 // into one contiguous run per CTA.  `slots` holds launch_area_doubles(tiles,
 // strips, sms) doubles for the lattices' total tiles and strips: the item
 // tables.
-// spt: sites per thread of the launch's kernel (1 or 2, see max_spt).
 lb_status launch_build(Launch& Ln, Lattice* const* lats, int nlat, void* descs, double* slots,
                        unsigned int* ticket, int sms, cudaStream_t stream, void* host_scratch,
-                       int seg = 0, int spt = 1);
+                       int seg = 0, int shape = SHAPE_8);
 size_t launch_area_doubles(size_t tiles, size_t strips, int sms);
 // Enqueue step step_k of a window of consecutive steps (0-based); advance: the
 // window's steps on its last launch, else 0.  The device's step counters move

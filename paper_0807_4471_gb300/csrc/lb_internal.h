@@ -181,6 +181,19 @@ struct StepArgs {
     int nstrips;
 };
 
+// Tile shapes of the step kernel (see Layout).
+//  SHAPE_8    8-row tiles, one site per thread, one CTA per SM;
+//  SHAPE_16   16-row tiles, two sites per thread, one CTA per SM;
+//  SHAPE_8X2  8-row tiles, two sites per thread, two CTAs of half the threads
+//             per SM (16-bit formats: their shared memory holds two).
+enum Shape : int { SHAPE_8 = 1, SHAPE_16 = 2, SHAPE_8X2 = 3 };
+constexpr bool has_shape(int precision, int shape) {
+    return shape == SHAPE_8 || (shape == SHAPE_16 && precision != LB_FP64) ||
+           (shape == SHAPE_8X2 && (precision == LB_FP16_OFFSET || precision == LB_BF16_OFFSET));
+}
+constexpr int shape_rows(int shape) { return shape == SHAPE_16 ? 16 : 8; }
+constexpr int shape_ctas(int shape) { return shape == SHAPE_8X2 ? 2 : 1; }   // per SM
+
 // Host-side launch helpers (lb_dispatch.cu).
 int kernel_smem_bytes(int precision);
 int kernel_tile_x(int precision);
@@ -190,16 +203,16 @@ int kernel_elem_bytes(int precision);
 int kernel_smem_obs_bytes(int precision);
 int kernel_block_rows(int precision);
 int kernel_scale_log2(int precision);
-// 1 if the step kernel with spt sites per thread leaves through a staging
-// tile (its periodic ghost copies are then separate stores after the tile)
-int kernel_staged(int precision, int spt);
+// 1 if the step kernel of a shape leaves through a staging tile (its periodic
+// ghost copies are then separate stores after the tile)
+int kernel_staged(int precision, int shape);
 
 // Step: the persistent multi-lattice kernel (args: BatchArgs<C>), variant
 // bit 0 = every lattice periodic, bit 1 = general forcing, bit 2 = 1 - omega
-// rounds to zero for both species (the collision reads no populations), spt sites per
-// thread (tiles of 8 spt rows).  Observe: one lattice, one CTA per 8-row
+// rounds to zero for both species (the collision reads no populations), in one of the
+// precision's tile shapes.  Observe: one lattice, one CTA per 8-row
 // tile (args: StepArgs<C>, tin: tile-box load map).
-cudaError_t launch_step(int precision, const void* args, int variant, int spt, dim3 grid,
+cudaError_t launch_step(int precision, const void* args, int variant, int shape, dim3 grid,
                         cudaStream_t s);
 // Opt the kernels of a precision into their shared memory (once per device;
 // call before capturing launches into a graph).
@@ -221,7 +234,7 @@ cudaError_t launch_load_pops(int precision, const Geom& g, const void* coef, voi
 template <int P>
 cudaError_t configure_prec();
 template <int P>
-cudaError_t launch_step_prec(const void* args, int variant, int spt, dim3 grid, cudaStream_t s);
+cudaError_t launch_step_prec(const void* args, int variant, int shape, dim3 grid, cudaStream_t s);
 template <int P>
 cudaError_t launch_observe_prec(const CUtensorMap* tin, const void* args, dim3 grid,
                                 cudaStream_t s);

@@ -891,10 +891,11 @@ __device__ __forceinline__ void block_sum4(double red[4], double (*s_red)[4]) {
 // lattice's step counter and buffer parity.
 // V: bit 0 = every lattice periodic (no wall code); bit 1 = general forcing;
 // bit 2 = omega = 1 for both species (the site phase reads no populations).
-template <int P, int V, int SPT>
-__global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
+template <int P, int V, int SH>
+__global__ void __launch_bounds__(Layout<P, SH>::NT, Layout<P, SH>::CTAS)
     k_step(const __grid_constant__ BatchArgs<typename Prec<P>::C> a) {
-    typedef Layout<P, SPT> L;
+    typedef Layout<P, SH> L;
+    constexpr int SPT = L::SPT, ADV = L::ADV, NBT = L::NBT;
     typedef typename L::T2 T2;
     typedef typename L::C C;
     typedef typename L::C2 C2;
@@ -929,7 +930,7 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
     // cost the large lattices 1-3 %).
     // window column and block row of this thread (both phases)
     const int t_lx = tid % L::RX, t_j = tid / L::RX;
-    static_assert(L::NT == L::RX * L::TYB && L::TY >= 4, "one window column per thread and block row");
+    static_assert(L::NT == L::RX * L::TR && L::TY >= 4, "one window column per thread and block row");
     static_assert(P != LB_FP64 || (L::RX == 32 && SPT == 1), "FP64: a warp is a row of a tile");
     // Rows of the density phase: thread row t_j computes the new window rows
     // 4 + SPT t_m + c, c < SPT, which hold its own sites (window rows
@@ -942,7 +943,7 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
     // tile boundary in a small shared buffer of their own.
     constexpr int kCarry = 2 / SPT;   // thread rows whose sites are carried rows
     static_assert(2 % SPT == 0, "two carried rows per tile");
-    const int t_m = (t_j + L::TYB - kCarry) % L::TYB;
+    const int t_m = (t_j + L::TR - kCarry) % L::TR;
     const bool t_carry = t_j < kCarry;
     // Columns likewise: window column w holds lattice column x0 - 2 + w and
     // site column lx is window column lx + 2, so thread t_lx computes window
@@ -991,7 +992,7 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
         const LatDesc<C>* d = &a.lat[w.x];
         p_x0 = w.y * L::TX;
         p_ty_a = w.z;
-        p_nblk = SPT * (w.w - w.z) + 1;
+        p_nblk = ADV * (w.w - w.z) + 1;
         p_map = &d->tin[*((volatile int*)&d->st->cur) ^ (step_k & 1)];
         tma_prefetch_map(p_map);
     };
@@ -1000,7 +1001,7 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
         uint64_t* bar = &bars[p_pos % L::NB];
         mbar_expect_tx(bar, (uint32_t)L::SLOT_BYTES);
         // box origin: pair column x0 (= x0 - gx + gx) -> element 2 x0; padded row 8j
-        tma_load_3d_hint(slot(p_pos), p_map, 2 * p_x0, L::TYB * (SPT * p_ty_a + p_j), 0, bar,
+        tma_load_3d_hint(slot(p_pos), p_map, 2 * p_x0, L::TYB * (ADV * p_ty_a + p_j), 0, bar,
                          s_pol[0]);
         ++p_pos;
         if (++p_j == p_nblk) {
@@ -1020,7 +1021,7 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
     // its blocks before the next tile's first one (all of them at an item's
     // last tile): refill those slots.
     auto release = [&](int q) {
-        const int released = (ty + 1 < ty_b) ? q + SPT : q + SPT + 1;
+        const int released = (ty + 1 < ty_b) ? q + ADV : q + NBT;
         fence_proxy_async();   // generic reads of freed slots before async writes
         while (p_pos < released + L::NB && issue_next()) {}
     };
@@ -1047,14 +1048,14 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
         // tiles advance
         int qm = c_pos % L::NB, qph = (c_pos / L::NB) & 1;
         for (ty = ty_a; ty < ty_b; ++ty) {
-            const int q = c_pos + SPT * (ty - ty_a);   // this tile uses blocks q .. q + SPT
+            const int q = c_pos + ADV * (ty - ty_a);   // this tile uses blocks q .. q + ADV
             // Each thread sees the blocks land itself (the first block of a
             // tile after an item's first was seen as the previous tile's
             // last); a timeout is acted on after the next barrier (garbage
             // read meanwhile is harmless).
-            int sl[SPT + 1];
+            int sl[NBT];
 #pragma unroll
-            for (int b = 0; b <= SPT; ++b) {
+            for (int b = 0; b < NBT; ++b) {
                 int sb = qm + b, ph = qph;
                 if (sb >= L::NB) {
                     sb -= L::NB;
@@ -1068,9 +1069,9 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
             // q + SPT; brow(r, c): padded row y0 + r, pair column c, plane 0.
             const T2* s0 = reinterpret_cast<const T2*>(smem + sl[0] * L::SLOT_BYTES);
             const T2* s1 = reinterpret_cast<const T2*>(smem + sl[1] * L::SLOT_BYTES);
-            const T2* s2 = reinterpret_cast<const T2*>(smem + sl[SPT] * L::SLOT_BYTES);
+            const T2* s2 = reinterpret_cast<const T2*>(smem + sl[ADV] * L::SLOT_BYTES);
             auto brow = [&](int r, int c) {
-                const T2* base = r < L::TYB ? s0 : (SPT == 1 || r < 2 * L::TYB ? s1 : s2);
+                const T2* base = r < L::TYB ? s0 : (ADV == 1 || r < 2 * L::TYB ? s1 : s2);
                 return base + (r & (L::TYB - 1)) * L::BX + c;
             };
 
@@ -1254,7 +1255,7 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
                     // x0 + gx, row y0 + 8h + kGY; a ragged tile's store is
                     // clipped at x = nx, y = ny (no box starts below the lattice)
 #pragma unroll
-                    for (int h = 0; h < SPT; ++h)
+                    for (int h = 0; h < ADV; ++h)
                         if (h == 0 || y0 + h * L::TYB < g.ny)
                             tma_store_3d_hint(&d->tout[cur ^ 1], stage + L::stage_off(h * L::TYB, 0),
                                               2 * (x0 + L::GX), y0 + h * L::TYB + kGY, 0, s_pol[1]);
@@ -1268,7 +1269,7 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
                                   (per_lat && (y0 < 3 || y0 + L::TY > g.ny - 3));
                 if (edge) write_edges<P, L>(stage, fout, g, x0, y0, per_lat, tid);
             }
-            qm += SPT;
+            qm += ADV;
             if (qm >= L::NB) {
                 qm -= L::NB;
                 qph ^= 1;
@@ -1277,7 +1278,7 @@ __global__ void __launch_bounds__(Layout<P, SPT>::NT, 1)
         if (!(nf.x == C(0) && nf.y == C(0)))   // a density of this lattice went non-finite
             atomicOr(&d->st->err, ERR_NONFINITE);
         if (s_fail) break;
-        c_pos += SPT * (ty_b - ty_a) + 1;
+        c_pos += ADV * (ty_b - ty_a) + 1;
     }
     // Wall momentum of this CTA's items that hold a wall row, in FP64: the
     // wall-site values the site phase left in the lattice's wall columns,
@@ -1559,34 +1560,35 @@ __global__ void k_wait_selftest(unsigned int* err, int limit) {
 #endif
 
 // ------------------------------------------------------------- launchers
-// Step kernels of precision P (8-row tiles; 16-row tiles where the
-// precision has them) and the observe kernels, variant by variant.
+// Step kernels of precision P in its tile shapes and the observe kernels,
+// variant by variant.
 template <int P>
 static cudaError_t configure_all() {
     typedef Layout<P> L;
     cudaError_t e = cudaSuccess;
     auto opt = [&](auto kern, int bytes) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e == cudaSuccess)   // room for the shape's resident CTAs
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                     cudaSharedmemCarveoutMaxShared);
     };
-    opt(k_step<P, 0, 1>, L::SMEM);
-    opt(k_step<P, 1, 1>, L::SMEM);
-    opt(k_step<P, 2, 1>, L::SMEM);
-    opt(k_step<P, 3, 1>, L::SMEM);
-    opt(k_step<P, 4, 1>, L::SMEM);
-    opt(k_step<P, 5, 1>, L::SMEM);
-    opt(k_step<P, 6, 1>, L::SMEM);
-    opt(k_step<P, 7, 1>, L::SMEM);
-    if constexpr (Prec<P>::NB2 > 0) {
-        typedef Layout<P, 2> L2;
-        opt(k_step<P, 0, 2>, L2::SMEM);
-        opt(k_step<P, 1, 2>, L2::SMEM);
-        opt(k_step<P, 2, 2>, L2::SMEM);
-        opt(k_step<P, 3, 2>, L2::SMEM);
-        opt(k_step<P, 4, 2>, L2::SMEM);
-        opt(k_step<P, 5, 2>, L2::SMEM);
-        opt(k_step<P, 6, 2>, L2::SMEM);
-        opt(k_step<P, 7, 2>, L2::SMEM);
-    }
+    auto opt_shape = [&](auto tag) {
+        constexpr int SH = decltype(tag)::value;
+        if constexpr (has_shape(P, SH)) {
+            constexpr int bytes = Layout<P, SH>::SMEM;
+            opt(k_step<P, 0, SH>, bytes);
+            opt(k_step<P, 1, SH>, bytes);
+            opt(k_step<P, 2, SH>, bytes);
+            opt(k_step<P, 3, SH>, bytes);
+            opt(k_step<P, 4, SH>, bytes);
+            opt(k_step<P, 5, SH>, bytes);
+            opt(k_step<P, 6, SH>, bytes);
+            opt(k_step<P, 7, SH>, bytes);
+        }
+    };
+    opt_shape(std::integral_constant<int, SHAPE_8>{});
+    opt_shape(std::integral_constant<int, SHAPE_16>{});
+    opt_shape(std::integral_constant<int, SHAPE_8X2>{});
     opt(k_observe<P, 2>, L::SMEM_OBS);
     opt(k_observe<P, 3>, L::SMEM_OBS);
     return e;
@@ -1615,10 +1617,10 @@ static bool pdl_enabled() {
     return on;
 }
 
-template <int P, int SPT>
+template <int P, int SH>
 static cudaError_t launch_step_shape(const BatchArgs<typename Prec<P>::C>& a, int variant, dim3 grid,
                                      cudaStream_t s) {
-    typedef Layout<P, SPT> L;
+    typedef Layout<P, SH> L;
     // Consecutive steps on a stream overlap the next launch's set-up with the
     // previous launch's last CTAs (programmatic stream serialization); the
     // kernel waits for the previous grid before it reads the lattice state.
@@ -1634,27 +1636,29 @@ static cudaError_t launch_step_shape(const BatchArgs<typename Prec<P>::C>& a, in
     cfg.numAttrs = pdl_enabled() ? 1 : 0;
     cudaError_t e;
     switch (variant & 7) {
-        case 0: e = cudaLaunchKernelEx(&cfg, k_step<P, 0, SPT>, a); break;
-        case 1: e = cudaLaunchKernelEx(&cfg, k_step<P, 1, SPT>, a); break;
-        case 2: e = cudaLaunchKernelEx(&cfg, k_step<P, 2, SPT>, a); break;
-        case 3: e = cudaLaunchKernelEx(&cfg, k_step<P, 3, SPT>, a); break;
-        case 4: e = cudaLaunchKernelEx(&cfg, k_step<P, 4, SPT>, a); break;
-        case 5: e = cudaLaunchKernelEx(&cfg, k_step<P, 5, SPT>, a); break;
-        case 6: e = cudaLaunchKernelEx(&cfg, k_step<P, 6, SPT>, a); break;
-        default: e = cudaLaunchKernelEx(&cfg, k_step<P, 7, SPT>, a); break;
+        case 0: e = cudaLaunchKernelEx(&cfg, k_step<P, 0, SH>, a); break;
+        case 1: e = cudaLaunchKernelEx(&cfg, k_step<P, 1, SH>, a); break;
+        case 2: e = cudaLaunchKernelEx(&cfg, k_step<P, 2, SH>, a); break;
+        case 3: e = cudaLaunchKernelEx(&cfg, k_step<P, 3, SH>, a); break;
+        case 4: e = cudaLaunchKernelEx(&cfg, k_step<P, 4, SH>, a); break;
+        case 5: e = cudaLaunchKernelEx(&cfg, k_step<P, 5, SH>, a); break;
+        case 6: e = cudaLaunchKernelEx(&cfg, k_step<P, 6, SH>, a); break;
+        default: e = cudaLaunchKernelEx(&cfg, k_step<P, 7, SH>, a); break;
     }
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <int P>
-cudaError_t launch_step_prec(const void* args, int variant, int spt, dim3 grid, cudaStream_t s) {
+cudaError_t launch_step_prec(const void* args, int variant, int shape, dim3 grid, cudaStream_t s) {
     typedef typename Prec<P>::C C;
     cudaError_t e = ensure_configured<P>();
     if (e != cudaSuccess) return e;
     const BatchArgs<C>& a = *reinterpret_cast<const BatchArgs<C>*>(args);
-    if (spt == 1) return launch_step_shape<P, 1>(a, variant, grid, s);
-    if constexpr (Prec<P>::NB2 > 0)
-        if (spt == 2) return launch_step_shape<P, 2>(a, variant, grid, s);
+    if (shape == SHAPE_8) return launch_step_shape<P, SHAPE_8>(a, variant, grid, s);
+    if constexpr (has_shape(P, SHAPE_16))
+        if (shape == SHAPE_16) return launch_step_shape<P, SHAPE_16>(a, variant, grid, s);
+    if constexpr (has_shape(P, SHAPE_8X2))
+        if (shape == SHAPE_8X2) return launch_step_shape<P, SHAPE_8X2>(a, variant, grid, s);
     return cudaErrorInvalidValue;
 }
 

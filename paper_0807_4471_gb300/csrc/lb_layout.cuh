@@ -248,12 +248,16 @@ __device__ __forceinline__ double csin(double v) { return sin(v); }
 __device__ __forceinline__ float csin(float v) { return sinf(v); }
 
 // Shared-memory layout and thread mapping of the step kernel for precision P
-// and SPT sites per thread: SPT = 1, tiles of TX x 8 sites, one site per
-// thread, leaving through a staging tile and a TMA bulk store; SPT = 2,
-// tiles of TX x 16 sites, each thread updating two vertically adjacent
-// sites (sharing their stencil rows) and storing them to global memory
-// directly.  Both walk the same 8-row population blocks.
-template <int P, int SPT = 1>
+// and tile shape SH: SHAPE_8, tiles of TX x 8 sites, one site per thread;
+// SHAPE_16, tiles of TX x 16 sites, each thread updating two vertically
+// adjacent sites (sharing their stencil rows); SHAPE_8X2, the same two sites
+// per thread on TX x 8 tiles by CTAs of half the threads, two of them resident
+// on an SM: a CTA's two barriers per tile stall all its warps together, and
+// while one CTA drains into a barrier the other keeps the pipes busy (FP16,
+// 4096^2: 288 us a step with SHAPE_16, 267 with SHAPE_8X2).  All walk the same 8-row
+// population blocks; tiles leave through a staging tile and a TMA bulk store
+// where it fits, else the threads store to global memory directly.
+template <int P, int SH = SHAPE_8>
 struct Layout {
     typedef typename Prec<P>::T T;
     typedef typename Prec<P>::T2 T2;
@@ -261,15 +265,20 @@ struct Layout {
     typedef typename Prec<P>::C2 C2;
     static constexpr int TX = Prec<P>::TX;
     static constexpr int TYB = Prec<P>::TY;           // rows of a population block (8)
-    static constexpr int TY = TYB * SPT;              // tile rows
+    static constexpr int SPT = SH == SHAPE_8 ? 1 : 2; // sites per thread
+    static constexpr int CTAS = shape_ctas(SH);       // resident CTAs per SM
+    static constexpr int TR = 8 / CTAS;               // thread rows
+    static constexpr int TY = TR * SPT;               // tile rows
+    static constexpr int ADV = TY / TYB;              // blocks a tile advances by
+    static constexpr int NBT = ADV + 1;               // blocks a tile reads (TY + 6 rows)
     static constexpr int GX = Prec<P>::GX;
     static constexpr int BX = TX + 2 * GX;            // box columns (sites)
     static constexpr int BY = TYB + 2 * kGY;          // observe box rows
     static constexpr int RX = TX + 4, RY = TYB + 4;   // rho/Psi tile (2-cell halo), observe
     // threads: one per deviation column and block row; in the site phase
     // thread (lx, j) = (tid % RX, tid / RX) updates sites (lx, SPT j + s), lx < TX
-    static constexpr int NT = RX * TYB;
-    static constexpr int NB = SPT == 1 ? Prec<P>::NB : Prec<P>::NB2;   // ring slots of blocks
+    static constexpr int NT = RX * TR;
+    static constexpr int NB = SH == SHAPE_8 ? Prec<P>::NB : SH == SHAPE_16 ? Prec<P>::NB2 : 3;   // ring slots of blocks
     // rho/Psi deviation window of a tile: rows y0 - 2 .. y0 + TY + 1
     static constexpr int WIN = TY + 4;
     // step kernel: NB block slots, the rho and Psi windows, and -- where it
@@ -297,9 +306,8 @@ struct Layout {
     static constexpr int BOX_STRIDE = (BOX_BYTES + 127) / 128 * 128;
     static constexpr int RHOPSI = (2 * RX * RY * (int)sizeof(C2) + 127) / 128 * 128;
     static constexpr int SMEM_OBS = BOX_STRIDE + RHOPSI + 128;
-    static_assert(SPT == 1 || SPT == 2, "one or two sites per thread");
     static_assert(SPT == 1 || STAGED || sizeof(T2) == 8, "direct stores: FP32 pairs only");
-    static_assert(NB >= SPT + 2, "the ring holds a tile's blocks and at least one more");
+    static_assert(NB >= NBT + 1, "the ring holds a tile's blocks and at least one more");
     static_assert(RX % 32 == 0, "deviation rows are whole warps");
     static_assert((2 * TX * sizeof(T)) % 16 == 0 && (2 * (TX + GX) * sizeof(T)) % 16 == 0,
                   "TMA x coordinates of tiles stay 16-byte aligned");
@@ -308,6 +316,7 @@ struct Layout {
     static_assert((BX * sizeof(T2)) % 16 == 0, "TMA box rows must be 16-byte multiples");
     static_assert(2 * BX <= 256 && 2 * TX <= 256 && BY <= 256, "TMA box extent");
     static_assert(GX >= 3 && (GX * sizeof(T)) % 16 == 0, "ghost width");
+    static_assert(CTAS * (SMEM + 4096) <= 228 * 1024, "resident CTAs");
     static_assert(SMEM <= 227 * 1024 - 1024 && SMEM_OBS <= 227 * 1024, "shared memory");
 };
 

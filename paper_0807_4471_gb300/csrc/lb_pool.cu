@@ -84,13 +84,13 @@ struct Member {
 // A launch configuration the tuner chooses: work partition and tile shape.
 struct Choice {
     int seg;                 // > 0 segments of seg tiles; -1 contiguous runs; 0 the model's
-    int spt;                 // sites per thread (tiles of 8 spt rows)
+    int shape;               // tile shape
 };
 
 struct lb_pool {
     lb_params shared;
     int forced_seg;          // 0: autotune; else the partition to use (-1: contiguous runs)
-    int forced_spt;          // 0: autotune; else the sites per thread to use
+    int forced_rows;         // 0: autotune; else the tile height to use
     cudaStream_t stream;
     bool own_stream;
     int device, sms;
@@ -165,7 +165,7 @@ lb_status build(lb_pool* P, Choice c) {
     cudaError_t ce = kernels_configure(P->shared.precision);   // before any graph capture
     if (ce != cudaSuccess) return cuda_status(ce);
     lb_status s = launch_build(P->launch, lats.data(), nlat, P->desc_mem, P->slots, P->ticket,
-                               P->sms, P->stream, P->host_desc, c.seg, c.spt);
+                               P->sms, P->stream, P->host_desc, c.seg, c.shape);
     P->built = s == LB_OK;
     return s;
 }
@@ -216,11 +216,11 @@ void advanced(lb_pool* P, long long k) {
 // and lb_pool_set_tile_rows kept), and the untuned default.
 std::vector<Choice> candidates(lb_pool* P) {
     const int prec = P->shared.precision;
-    std::vector<int> spts;
-    if (P->forced_spt != 0) spts.push_back(P->forced_spt);
-    else for (int k = 1; k <= max_spt(prec); ++k) spts.push_back(k);
     std::vector<Choice> out;
-    for (int spt : spts) {
+    for (int shape : {SHAPE_8, SHAPE_16, SHAPE_8X2}) {
+        if (!has_shape(prec, shape) || (P->forced_rows != 0 && shape_rows(shape) != P->forced_rows)) continue;
+        // (where two CTAs fit an SM the 16-row tile runs only when asked for)
+        if (shape == SHAPE_16 && has_shape(prec, SHAPE_8X2) && P->forced_rows == 0) continue;
         std::vector<int> segs;
         if (P->forced_seg != 0) {
             segs.push_back(P->forced_seg);
@@ -231,22 +231,27 @@ std::vector<Choice> candidates(lb_pool* P) {
             for (int j : P->active) {
                 const Lattice& L = P->members[(size_t)j].lat;
                 ns.push_back(L.nstrips);
-                nt.push_back(tiles_y(L, spt));
+                nt.push_back(tiles_y(L, shape));
                 tiles = std::max(tiles, nt.back());
             }
-            segs = {-1, choose_seg(ns.data(), nt.data(), (int)ns.size(), P->sms)};
+            segs = {-1, choose_seg(ns.data(), nt.data(), (int)ns.size(), P->sms * shape_ctas(shape))};
             for (int c : {1, 2, 4, 8, 16, 32, 64})
                 if (c <= tiles && std::find(segs.begin(), segs.end(), c) == segs.end()) segs.push_back(c);
         }
-        for (int seg : segs) out.push_back({seg, spt});
+        for (int seg : segs) out.push_back({seg, shape});
     }
     return out;
 }
 Choice untuned(lb_pool* P) {
-    return {P->forced_seg, P->forced_spt != 0 ? P->forced_spt : default_spt(P->shared.precision)};
+    long long tiles8 = 0;
+    for (int j : P->active) {
+        const Lattice& L = P->members[(size_t)j].lat;
+        tiles8 += (long long)L.nstrips * L.ntiles_y;
+    }
+    return {P->forced_seg, shape_of_rows(P->shared.precision, P->forced_rows, tiles8, P->sms)};
 }
 std::string cache_key(lb_pool* P) {
-    return signature(P) + "|" + std::to_string(P->forced_seg) + "|" + std::to_string(P->forced_spt);
+    return signature(P) + "|" + std::to_string(P->forced_seg) + "|" + std::to_string(P->forced_rows);
 }
 
 // Time kTuneSteps real steps for each candidate (tile shape, partition) and
@@ -515,18 +520,15 @@ lb_status lb_pool_set_partition(lb_pool* P, int32_t seg) {
 
 lb_status lb_pool_set_tile_rows(lb_pool* P, int32_t rows) {
     if (!P) return LB_ERR_INVALID;
-    const int ty = kernel_tile_y(P->shared.precision);
-    if (rows != 0 && rows != ty && rows != 2 * ty) return LB_ERR_INVALID;
-    const int spt = rows / ty;
-    if (spt > max_spt(P->shared.precision)) return LB_ERR_INVALID;
-    P->forced_spt = spt;
+    if (shape_of_rows(P->shared.precision, rows, 0, P->sms) == 0) return LB_ERR_INVALID;
+    P->forced_rows = rows;
     P->built = false;
     drop_graph(P);
     return LB_OK;
 }
 
 int32_t lb_pool_tile_rows(const lb_pool* P) {
-    return P && P->built ? P->launch.spt * kernel_tile_y(P->shared.precision) : 0;
+    return P && P->built ? shape_rows(P->launch.shape) : 0;
 }
 
 lb_status lb_pool_destroy(lb_pool* P) {

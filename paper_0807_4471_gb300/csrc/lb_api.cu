@@ -64,7 +64,7 @@ lb_status create_common(const lb_params* p, void* stream, void* ws, size_t bytes
         Lattice* one = &h->lat;
         alignas(128) unsigned char scratch[sizeof(LatDesc<double>)];
         const int sms = device_sms(h->device);
-        const int shape = shape_of_rows(p->precision, p->tile_rows,
+        const int shape = shape_of_rows(p->precision, moments_ok(*one), p->tile_rows,
                                         (long long)one->nstrips * one->ntiles_y, sms);
         s = launch_build(h->launch, &one, 1, h->ws + H.desc,
                          reinterpret_cast<double*>(h->ws + H.slots),
@@ -178,7 +178,7 @@ lb_status lb_step(lb_handle* h, int64_t n) {
     while (n > 0 && s == LB_OK) {
         const int w = n < (1 << 20) ? (int)n : 1 << 20;
         s = launch_window(h->launch, w, h->stream);
-        if (s == LB_OK) lattice_advanced(h->lat, w);
+        if (s == LB_OK) lattice_advanced(h->lat, w, h->launch.shape);
         n -= w;
     }
     nvtxRangePop();

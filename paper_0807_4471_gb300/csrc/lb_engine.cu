@@ -251,6 +251,7 @@ lb_status lattice_setup(Lattice& L, const lb_params* p, char* region) {
     L.fbytes = r.fbytes;
     L.cur = 0;
     L.pull = 0;
+    L.mom = false;
     L.inited = false;
     L.t = 0;
     L.err_latched = 0;
@@ -319,21 +320,27 @@ int tiles_y(const Lattice& L, int shape) {
     const int ty = shape_rows(shape);
     return (L.p.ny + ty - 1) / ty;
 }
+// The moment kernel: FP32, omega = 1 for both species in FP32, no source term.
+bool moments_ok(const Lattice& L) {
+    return L.p.precision == LB_FP32 && L.kf.omm.x == 0.0f && L.kf.omm.y == 0.0f && !L.kf.source;
+}
 // Default tile shape of a lattice set with `tiles8` 8-row tiles.  The 16-bit
-// formats: two CTAs per SM, except where the tiles do not even fill one CTA
-// per SM one and a half times over; a thread's single site then finishes a
-// tile sooner (256^2 FP16, 160 tiles: 6.3 us a step against 6.9; 512^2, 576
-// tiles: 11.0 against 9.7).  FP32: the 16-row tile beyond the same line
-// (256^2: 6.5 us with 8 rows, 7.3 with 16; 512^2: 11.2 and 10.2).
-int default_shape(int precision, long long tiles8, int sms) {
-    if (precision == LB_FP64 || 2 * tiles8 <= 3LL * sms) return SHAPE_8;
+// formats and the moment kernel: two CTAs per SM, except where the tiles do
+// not even fill one CTA per SM one and a half times over; a thread's single
+// site then finishes a tile sooner (256^2 FP16, 160 tiles: 6.3 us a step against
+// 6.9; 512^2, 576 tiles: 11.0 against 9.7).  Other FP32: the 16-row tile beyond
+// the same line (256^2: 6.5 us with 8 rows, 7.3 with 16; 512^2: 11.2 and 10.2).
+int default_shape(int precision, bool moments, long long tiles8, int sms) {
+    const bool few = 2 * tiles8 <= 3LL * sms;
+    if (moments) return few ? SHAPE_M8 : SHAPE_M8X2;
+    if (precision == LB_FP64 || few) return SHAPE_8;
     return has_shape(precision, SHAPE_8X2) ? SHAPE_8X2 : SHAPE_16;
 }
-int shape_of_rows(int precision, int rows, long long tiles8, int sms) {
-    if (rows == 0) return default_shape(precision, tiles8, sms);
+int shape_of_rows(int precision, bool moments, int rows, long long tiles8, int sms) {
+    if (rows == 0) return default_shape(precision, moments, tiles8, sms);
     if (rows == 16) return has_shape(precision, SHAPE_16) ? SHAPE_16 : 0;
     if (rows != 8) return 0;
-    const int d = default_shape(precision, tiles8, sms);
+    const int d = default_shape(precision, false, tiles8, sms);
     return d == SHAPE_8X2 ? d : SHAPE_8;
 }
 
@@ -398,6 +405,7 @@ void partition(Lattice* const* lats, int nlat, int seg, int shape, int sms, std:
         const bool per = L.g.periodic != 0;
         if (!per && (y0 == 0 || y0 + tyy >= L.p.ny)) return 1.38;
         double c = 1.0;
+        if (shape_moments(shape)) return c;   // no ghost copies
         if (x0 < 3 || x0 + tx > L.p.nx - 3) c += 0.21;
         if (per && (y0 < 3 || y0 + tyy > L.p.ny - 3)) c += kernel_staged(L.p.precision, shape) ? 0.25 : 0.02;
         return c;
@@ -471,14 +479,18 @@ void partition(Lattice* const* lats, int nlat, int seg, int shape, int sms, std:
         }
         return n;
     };
-    double lo = cmax + kItemStart, hi = sum + kItemStart * (double)sms;
-    if (runs_for(lo, nullptr) > sms)
-        for (int it = 0; it < 60 && hi - lo > 1e-6 * hi; ++it) {
+    // (from just above the mean run; costs are multiples of 0.01, so a bound
+    // known to 0.002 gives the optimal runs)
+    double lo = std::max(cmax + kItemStart, sum / sms), hi = lo;
+    if (runs_for(lo, nullptr) > sms) {
+        do {
+            hi += cmax + 2.0 * kItemStart;
+        } while (runs_for(hi, nullptr) > sms);
+        while (hi - lo > 0.002) {
             const double mid = 0.5 * (lo + hi);
             if (runs_for(mid, nullptr) <= sms) hi = mid; else lo = mid;
         }
-    else
-        hi = lo;
+    }
     std::vector<long long> starts;
     runs_for(hi, &starts);
     const int G = (int)starts.size();
@@ -513,10 +525,12 @@ void partition(Lattice* const* lats, int nlat, int seg, int shape, int sms, std:
 // ~40 tiles of 8 rows (measured faster on 512^2-1024^2 lattices), the
 // load-balance model's dealt segments beyond (their CTAs sweep a band of
 // rows together, which keeps the halo columns in L2 on large lattices);
-// `tiles` counts tiles of the shape, `ctas` the launch's CTAs.
+// `tiles` counts tiles of the shape, `ctas` the launch's CTAs.  The moment kernel
+// moves a third of the bytes and takes contiguous runs at every size (4096^2:
+// 304 us a step, the best dealt segments 310; 4 x 1024^2: 84 and 84).
 static int default_seg(long long tiles, int shape, const int* ns, const int* nt, int nlat, int sms,
                        int ctas) {
-    return tiles * shape_rows(shape) <= 8LL * 40 * sms ? -1 : choose_seg(ns, nt, nlat, ctas);
+    return shape_moments(shape) || tiles * shape_rows(shape) <= 8LL * 40 * sms ? -1 : choose_seg(ns, nt, nlat, ctas);
 }
 
 // Host-only plan of a launch's work items (lb_plan_partition).
@@ -627,7 +641,8 @@ lb_status launch_build(Launch& Ln, Lattice* const* lats, int nlat, void* descs, 
     // One buffer of every lattice within 80 % of L2: the step's output can
     // stay in L2 for the next step, next to the input streaming through.
     long long buf = 0;
-    for (int l = 0; l < nlat; ++l) buf += (long long)lats[l]->fbytes;
+    for (int l = 0; l < nlat; ++l)
+        buf += shape_moments(shape) ? 24LL * lats[l]->p.nx * lats[l]->p.ny : (long long)lats[l]->fbytes;
     const int l2_resident = buf * 5 <= device_l2_bytes() * 4 ? 1 : 0;
     // With the collision free of the populations (tau = 1), a tile's ring
     // slots can be refilled as soon as its density phase is done.  Measured
@@ -716,6 +731,7 @@ static lb_status lattice_observe_pull(Lattice& L, int obs, double* out, int q0, 
         a.q1 = q1;
         a.wsum = L.wsum;
         a.nstrips = L.nstrips;
+        a.mom = L.mom ? reinterpret_cast<const float2*>(L.fbuf[L.cur]) : nullptr;
         e = launch_observe(L.p.precision, &L.tobs[L.cur], &a, grid, s);
     }
     return cuda_status(e);
@@ -750,6 +766,7 @@ static lb_status lattice_reset(Lattice& L, cudaStream_t s) {
     L.t = 0;
     L.cur = 0;
     L.pull = 0;
+    L.mom = false;
     L.inited = true;
     L.err_latched = 0;
     return LB_OK;
@@ -822,11 +839,25 @@ lb_status lattice_load_populations(Lattice& L, const double* f, long long t, int
     return LB_OK;
 }
 
-void lattice_advanced(Lattice& L, long long n) {
+void lattice_advanced(Lattice& L, long long n, int shape) {
     if (n <= 0) return;
     L.t += n;
     L.cur ^= (int)(n & 1);
     L.pull = 1;
+    L.mom = shape_moments(shape);
+}
+
+lb_status lattice_to_populations(Lattice& L, cudaStream_t s) {
+    if (!L.mom) return LB_OK;
+    cudaError_t e = launch_expand(L.g, L.kf, reinterpret_cast<const float2*>(L.fbuf[L.cur]),
+                                  L.fbuf[1 - L.cur], s);
+    L.cur ^= 1;
+    L.mom = false;
+    const int state[2] = {L.cur, 1};   // DevStats::cur, pull
+    static_assert(offsetof(DevStats, pull) == offsetof(DevStats, cur) + sizeof(int), "cur, pull");
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&L.st->cur, state, sizeof(state), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // `state` is on this stack
+    return cuda_status(e);
 }
 
 lb_status lattice_fields(Lattice& L, double* rho_A, double* rho_B, double* ux, double* uy,

@@ -28,7 +28,8 @@ struct Lattice {
     Coef<double> kd;
     Coef<float> kf;
     int nstrips, ntiles_y, seg;
-    int cur, pull;           // host mirror of DevStats::cur / pull
+    int cur, pull;           // host mirror of DevStats::cur, and of pull != 0
+    bool mom;                // host mirror of DevStats::pull == 2: held by its moments
     bool inited;
     long long t;             // host mirror of the step count
     unsigned int err_latched;
@@ -64,12 +65,14 @@ lb_status plan_partition(const lb_params* ps, int nlat, int seg, int tile_rows, 
 // Segment length (tiles per work item) minimising the most loaded CTA.
 int choose_seg(const int* nstrips, const int* ntiles_y, int nlat, int G);
 
-// Tile rows of a lattice in a shape; the library's default shape for a set of
-// lattices with tiles8 8-row tiles in all; and the shape for a requested tile
-// height (0: the default; result 0: the precision has no such tile).
+// Tile rows of a lattice in a shape; whether its steps may take the moment
+// kernel; the library's default shape for a set of lattices with tiles8 8-row
+// tiles in all; and the shape for a requested tile height (0: the default;
+// 8 or 16: a population kernel; result 0: the precision has no such tile).
 int tiles_y(const Lattice& L, int shape);
-int default_shape(int precision, long long tiles8, int sms);
-int shape_of_rows(int precision, int rows, long long tiles8, int sms);
+bool moments_ok(const Lattice& L);
+int default_shape(int precision, bool moments, long long tiles8, int sms);
+int shape_of_rows(int precision, bool moments, int rows, long long tiles8, int sms);
 
 // Write the lattices' descriptors to `descs` (device, 128-byte aligned, room
 // for nlat LatDesc<double>) through `host_scratch` (as large, host) and fill
@@ -99,7 +102,10 @@ lb_status lattice_init_fields(Lattice& L, const double* rho_A, const double* rho
 // checkpoint); 0: the populations f(t) before collision.
 lb_status lattice_load_populations(Lattice& L, const double* f, long long t, int pulled,
                                    cudaStream_t s);
-void lattice_advanced(Lattice& L, long long n);
+// n steps of a launch with tile shape `shape` were enqueued.
+void lattice_advanced(Lattice& L, long long n, int shape);
+// Make a state that is held by its moments a population state (f*).
+lb_status lattice_to_populations(Lattice& L, cudaStream_t s);
 lb_status lattice_observe(Lattice& L, int obs, double* out, int q0, int q1, cudaStream_t s);
 lb_status lattice_fields(Lattice& L, double* rho_A, double* rho_B, double* ux, double* uy,
                          cudaStream_t s);

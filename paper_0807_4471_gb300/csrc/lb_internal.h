@@ -22,7 +22,8 @@ struct DevStats {
     long long samples;      // number of samples in the sums
     double totals[4];       // last observe pass: mass_A, mass_B, mom_x, mom_y
     int cur;                // buffer holding the current state (0 or 1)
-    int pull;               // 1: it holds post-collision f*(t-1); 0: f(t) in place
+    int pull;               // what it holds, 0: f(t) in place; 1: post-collision f*(t-1);
+                            // 2: the moments that f*(t-1) is the equilibrium of (k_step_m)
     long long next_sample;  // the next step whose wall momentum is sampled
                             // (stress_t0 + k stress_every >= t; set by the host
                             // with t, advanced by the kernel with t)
@@ -174,6 +175,7 @@ struct StepArgs {
     DevStats* st;
     double* slots;         // per-CTA partial sums
     int pull;              // 1: input holds post-collision f*(t-1); 0: f(t) in place
+    const float2* mom;     // FP32: the state's moments [3][ny][nx] where it is held by them, else null
     int obs;               // ObsKind; OBS_NONE = a time step
     double* obs_out;       // observe output base
     int q0, q1;            // OBS_POPS: planes [q0, q1) written
@@ -181,18 +183,24 @@ struct StepArgs {
     int nstrips;
 };
 
-// Tile shapes of the step kernel (see Layout).
+// Tile shapes of the step kernels (see Layout and MLayout).
 //  SHAPE_8    8-row tiles, one site per thread, one CTA per SM;
 //  SHAPE_16   16-row tiles, two sites per thread, one CTA per SM;
 //  SHAPE_8X2  8-row tiles, two sites per thread, two CTAs of half the threads
-//             per SM (16-bit formats: their shared memory holds two).
-enum Shape : int { SHAPE_8 = 1, SHAPE_16 = 2, SHAPE_8X2 = 3 };
+//             per SM (16-bit formats: their shared memory holds two);
+//  SHAPE_M8, SHAPE_M8X2  the same two 8-row forms of the moment kernel (FP32,
+//             tau = 1, velocity shift: see k_step_m).
+enum Shape : int { SHAPE_8 = 1, SHAPE_16 = 2, SHAPE_8X2 = 3, SHAPE_M8 = 4, SHAPE_M8X2 = 5 };
+constexpr bool shape_moments(int shape) { return shape >= SHAPE_M8; }
 constexpr bool has_shape(int precision, int shape) {
     return shape == SHAPE_8 || (shape == SHAPE_16 && precision != LB_FP64) ||
-           (shape == SHAPE_8X2 && (precision == LB_FP16_OFFSET || precision == LB_BF16_OFFSET));
+           (shape == SHAPE_8X2 && (precision == LB_FP16_OFFSET || precision == LB_BF16_OFFSET)) ||
+           (shape_moments(shape) && precision == LB_FP32);
 }
 constexpr int shape_rows(int shape) { return shape == SHAPE_16 ? 16 : 8; }
-constexpr int shape_ctas(int shape) { return shape == SHAPE_8X2 ? 2 : 1; }   // per SM
+constexpr int shape_ctas(int shape) {   // per SM
+    return shape == SHAPE_8X2 || shape == SHAPE_M8X2 ? 2 : 1;
+}
 
 // Host-side launch helpers (lb_dispatch.cu).
 int kernel_smem_bytes(int precision);
@@ -224,6 +232,11 @@ cudaError_t launch_init_seeded(int precision, const Geom& g, const void* coef, v
                                unsigned long long seed, cudaStream_t s);
 cudaError_t launch_init_fields(int precision, const Geom& g, const void* coef, void* fout,
                                const double* fields, cudaStream_t s);
+
+// FP32: the populations f* of a state held by its moments, into a population
+// buffer (with its ghost copies).
+cudaError_t launch_expand(const Geom& g, const Coef<float>& k, const float2* mom, void* fout,
+                          cudaStream_t s);
 
 // Restore directions [i0, i1) from FP64 populations [i1 - i0][2][ny][nx].
 cudaError_t launch_load_pops(int precision, const Geom& g, const void* coef, void* fout,

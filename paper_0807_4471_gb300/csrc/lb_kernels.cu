@@ -561,6 +561,65 @@ struct SiteOut {
     int q0, q1;
 };
 
+// Body acceleration along x at lattice row y.
+template <typename C>
+__device__ __forceinline__ C body_accel(const Coef<C>& k, const LatVals<C>& v, int y) {
+    C acc = k.g_x;
+    if (k.kolmo_amp != C(0)) acc += k.kolmo_amp * csin(v.kolmo_w * C(y));
+    return acc;
+}
+// Eq. (2): F_s = -Psi_s(r) sum_d K_s(d) d Psi_s(r + d)
+//               - (G_X/rho0) rho_s(r) sum_d w(d) d rho_s'(r + d);
+// species A feels rho_B, so the cross sums are used swapped.
+template <bool GEN, typename C, typename C2>
+__device__ __forceinline__ void site_force(C2 fxl, C2 fyl, C2 qx, C2 qy, C2 dpsi, C2 rho, int y,
+                                           const LatVals<C>& v, const Coef<C>& k, C2& Fx, C2& Fy) {
+    const C2 npc = neg_psi(dpsi, v);                       // -Psi_s(r)
+    const C2 ng = pmul(pset(-v.gx_rho0), rho);             // -(G_X/rho0) rho_s
+    Fx = pfma(npc, fxl, pmul(ng, pair(qx.y, qx.x)));
+    Fy = pfma(npc, fyl, pmul(ng, pair(qy.y, qy.x)));
+    if (GEN && k.has_accel) Fx = pfma(rho, pset(body_accel(k, v, y)), Fx);
+}
+// Velocities of the forced BGK relaxation (Eq. (1)), as z = 1.5u: the common
+// velocity u' = sum_s (j_s/tau_s) / sum_s (rho_s/tau_s) and, unless `source`,
+// the shift u_s = u' + tau_s F_s/rho_s.  (Selects, not branches: an empty site
+// has u' = 0 and no shift.)  TAU1: omega = 1 exactly, and the products are the
+// values themselves; j is taken in the storage scale of precision P, whose
+// inverse the factor 1.5 / den takes up (both exact powers of two apart).
+template <int P, bool TAU1, typename C, typename C2>
+__device__ __forceinline__ void site_velocity(C2 rho, C2 jx, C2 jy, C2 Fx, C2 Fy, bool source,
+                                              const Coef<C>& k, C2& zx, C2& zy) {
+    const C2 om = pair(k.omega[0], k.omega[1]);
+    const C2 ro = TAU1 ? rho : pmul(rho, om), jxo = TAU1 ? jx : pmul(jx, om),
+             jyo = TAU1 ? jy : pmul(jy, om);
+    const C den = ro.x + ro.y;
+    const C inv = den != C(0) ? (TAU1 ? C(1.5) * inv_scale_of<P>() : C(1.5)) * recip(den) : C(0);
+    zx = pset((jxo.x + jxo.y) * inv);
+    zy = pset((jyo.x + jyo.y) * inv);
+    if (!source) {
+        const C2 tr = pair(rho.x != C(0) ? k.tau15[0] * recip(rho.x) : C(0),
+                           rho.y != C(0) ? k.tau15[1] * recip(rho.y) : C(0));
+        zx = pfma(tr, Fx, zx);
+        zy = pfma(tr, Fy, zy);
+    }
+}
+// x-momentum handed to the wall by the links that will bounce back at the next
+// streaming, from the stored (rounded) values sv (storage scale of P):
+// sum_i c_ix (f*_i + f_opp), f_opp = f*_i - 6 w_i rho_w (c_i . u_w),
+// over the three links i leaving through the wall, which is
+// 2 (f*_a - f*_b) - 6 rho_w u_w (w_a + w_b) = 2 (f*_a - f*_b) - rho_w u_w / 3
+// with (a, b) = (8, 7) at the bottom wall and (5, 6) at the top
+// (c_ax = 1, c_bx = -1; w_a = w_b, so the offsets' difference is the
+// populations').  One compute-type value per site and species, kept
+// in the lattice's wall columns for the sums after the tile loop.
+template <int P, typename C, typename C2>
+__device__ __forceinline__ C2 wall_momentum(const C2 sv[9], bool down, const LatVals<C>& v) {
+    const C uw = down ? -v.u_wall : v.u_wall;
+    const C2 rw2 = pfma(sum9(sv), pset(inv_scale_of<P>()), pset(v.rho_ref));
+    const C2 dd = pmul(down ? psub(sv[8], sv[7]) : psub(sv[5], sv[6]), pset(inv_scale_of<P>()));
+    return psub(pmul(pset(C(2)), dd), pmul(rw2, pset(uw * (C(1) / C(3)))));
+}
+
 // One lattice site, given its force sums: moments from its pulled
 // populations, the force of Eq. (2), and either the forced BGK collision and
 // write-back (OBS = false) or the observables (OBS = true).  Both species are
@@ -599,18 +658,8 @@ __device__ __forceinline__ void site_update(
         note_nonfinite(rho, *nf);   // stays zero unless a density is inf or NaN
     }
 
-    // Eq. (2): F_s = -Psi_s(r) sum_d K_s(d) d Psi_s(r + d)
-    //               - (G_X/rho0) rho_s(r) sum_d w(d) d rho_s'(r + d);
-    // species A feels rho_B, so the cross sums are used swapped.
-    const C2 npc = neg_psi(dpsi, v);                       // -Psi_s(r)
-    const C2 ng = pmul(pset(-v.gx_rho0), rho);             // -(G_X/rho0) rho_s
-    C2 Fx = pfma(npc, fxl, pmul(ng, pair(qx.y, qx.x)));
-    C2 Fy = pfma(npc, fyl, pmul(ng, pair(qy.y, qy.x)));
-    if (GEN && k.has_accel) {
-        C acc = k.g_x;
-        if (k.kolmo_amp != C(0)) acc += k.kolmo_amp * csin(v.kolmo_w * C(y));
-        Fx = pfma(rho, pset(acc), Fx);
-    }
+    C2 Fx, Fy;
+    site_force<GEN>(fxl, fyl, qx, qy, dpsi, rho, y, v, k, Fx, Fy);
 
     if (OBS) {
         const long long N = (long long)g.nx * g.ny;
@@ -640,27 +689,10 @@ __device__ __forceinline__ void site_update(
         return;
     }
 
-    // Eq. (1): forced BGK relaxation.  Common velocity
-    // u' = sum_s (j_s/tau_s) / sum_s (rho_s/tau_s); shift u_s = u' + tau_s F_s/rho_s;
-    // carried as z = 1.5u.  (Selects, not branches: an empty site has u' = 0
-    // and no shift.)
-    // (TAU1: omega = 1 exactly, and the products are the values themselves)
-    const C2 om = pair(k.omega[0], k.omega[1]);
-    const C2 ro = TAU1 ? rho : pmul(rho, om), jxo = TAU1 ? jx : pmul(jx, om),
-             jyo = TAU1 ? jy : pmul(jy, om);
-    const C den = ro.x + ro.y;
-    // 1.5 / den, times the storage scale's inverse where j is taken in the
-    // storage scale (TAU1; both factors exact powers of two apart)
-    const C inv = den != C(0) ? (TAU1 ? C(1.5) * inv_scale_of<P>() : C(1.5)) * recip(den) : C(0);
-    const C2 zp = pair((jxo.x + jxo.y) * inv, (jyo.x + jyo.y) * inv);
+    // Eq. (1): forced BGK relaxation.
     const bool source = GEN && k.source;
-    C2 zx = pset(zp.x), zy = pset(zp.y);
-    if (!source) {
-        const C2 tr = pair(rho.x != C(0) ? k.tau15[0] * recip(rho.x) : C(0),
-                           rho.y != C(0) ? k.tau15[1] * recip(rho.y) : C(0));
-        zx = pfma(tr, Fx, zx);
-        zy = pfma(tr, Fy, zy);
-    }
+    C2 zx, zy;
+    site_velocity<P, TAU1>(rho, jx, jy, Fx, Fy, source, k, zx, zy);
     C2 hs[9];
     if (source)
         collide<C, C2, true, TAU1>(h, hs, drho, rho, zx, zy, k, Fx, Fy, scale_of<P>());
@@ -709,23 +741,11 @@ __device__ __forceinline__ void site_update(
         }
     }
     if (!per && (y == 0 || y == g.ny - 1)) {
-        // x-momentum handed to the wall by the links that will bounce back
-        // at the next streaming, from the stored (rounded) values:
-        // sum_i c_ix (f*_i + f_opp), f_opp = f*_i - 6 w_i rho_w (c_i . u_w),
-        // over the three links i leaving through the wall, which is
-        // 2 (f*_a - f*_b) - 6 rho_w u_w (w_a + w_b) = 2 (f*_a - f*_b) - rho_w u_w / 3
-        // with (a, b) = (8, 7) at the bottom wall and (5, 6) at the top
-        // (c_ax = 1, c_bx = -1; w_a = w_b, so the offsets' difference is the
-        // populations').  One compute-type value per site and species, kept
-        // in the lattice's wall columns for the sums after the tile loop.
-        const int down = (y == 0);
-        const C uw = down ? -v.u_wall : v.u_wall;
+        const bool down = y == 0;
         C2 sv[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) sv[i] = dec2(e[i]);
-        const C2 rw2 = pfma(sum9(sv), pset(inv_scale_of<P>()), pset(v.rho_ref));
-        const C2 dd = pmul(down ? psub(sv[8], sv[7]) : psub(sv[5], sv[6]), pset(inv_scale_of<P>()));
-        const C2 m = psub(pmul(pset(C(2)), dd), pmul(rw2, pset(uw * (C(1) / C(3)))));
+        const C2 m = wall_momentum<P>(sv, down, v);
         if (o.valid) reinterpret_cast<C2*>(o.wallx)[(down ? 0 : g.nx) + x] = m;
     }
 }
@@ -772,9 +792,10 @@ __device__ __forceinline__ void wall_sums(const BatchArgs<typename Prec<P>::C>& 
 }
 
 // The last CTA of a window's last launch: every lattice's step counter, buffer
-// parity and wall-sample schedule, one thread per lattice.
+// parity, state form (DevStats::pull) and wall-sample schedule, one thread per
+// lattice.
 template <int NT, typename C>
-__device__ __forceinline__ void advance_lattices(const BatchArgs<C>& a, int tid) {
+__device__ __forceinline__ void advance_lattices(const BatchArgs<C>& a, int tid, int pull) {
     for (int l = tid; l < a.nlat; l += NT) {
         const LatDesc<C>* d = &a.lat[l];
         DevStats* st = d->st;
@@ -787,7 +808,7 @@ __device__ __forceinline__ void advance_lattices(const BatchArgs<C>& a, int tid)
         }
         st->t = t;
         st->cur ^= a.advance & 1;
-        st->pull = 1;
+        st->pull = pull;
     }
 }
 
@@ -1315,11 +1336,315 @@ __global__ void __launch_bounds__(Layout<P, SH>::NT, Layout<P, SH>::CTAS)
     if (tid == 0) s_last = ticket_arrive(a.ticket) == (unsigned int)(G - 1);
     __syncthreads();
     if (!s_last) return;
-    advance_lattices<L::NT>(a, tid);
+    advance_lattices<L::NT>(a, tid, 1);
     // no other CTA of the launch touches the ticket again; the next launch
     // reads it after this one has completed
     if (tid == 0) *a.ticket = 0u;
 }
+
+// ------------------------------------------------- moment kernel (FP32)
+// The step of FP32 lattices with tau = 1 for both species and the velocity
+// shift.  There the post-collision populations are the equilibrium of six
+// numbers per site -- (drho, z_x, z_y) per species, see collide -- so a step
+// stores those instead of 18 populations: 24 bytes a site written and read
+// instead of 72, and the next step evaluates the populations where it needs
+// them, by the same operations on the same values (the results are the same
+// to the bit; the first step reads the initial populations themselves).
+// Bound: the population form ran at 90 % of the DRAM copy rate on 4096^2; this
+// one moves 57 bytes a site through DRAM there and is bound by instruction
+// issue (44 % busy, two barriers a tile) and the shared-memory pipe (62 %), as
+// the 16-bit kernels are.  Measured, populations -> moments: 4096^2 391 -> 304
+// us a step, 2048^2 107 -> 83, 1024^2 26.1 -> 22.1, 5 x 512^2 33.3 -> 27.3 (both
+// buffers of all five lattices now fit in L2), 128^2 5.0 -> 3.9, 512^2 Couette
+// 12.5 -> 10.1.
+//
+// The moments of a lattice are three unpadded planes [ny][nx] of (A, B) pairs;
+// loads wrap around the lattice, so no ghost copies are written.  Per tile:
+//  1. expand: the tile's 8 new rows of moments (loaded into registers during
+//     the previous tile) become populations in the ring, columns x0 - 3 ..
+//     x0 + 62 (thread column t_lx takes window column t_w; 16 threads of the
+//     first warp the two outermost columns),
+//  2. density phase and 3. site phase as in k_step, the ring in place of the
+//     block slots; the site's moments go straight to global memory.
+// Two barriers per tile: after the expansion, and before the site phase.  The
+// site phase reads no populations, so the next tile's expansion follows it
+// without one.
+#if LB_PREC == 1
+template <int V, int SH>
+__global__ void __launch_bounds__(MLayout<SH>::NT, MLayout<SH>::CTAS)
+    k_step_m(const __grid_constant__ BatchArgs<float> a) {
+    typedef MLayout<SH> L;
+    constexpr int P = LB_FP32;
+    constexpr bool ALLPER = (V & 1) != 0;
+    constexpr bool GEN = (V & 2) != 0;
+    constexpr int SPT = L::SPT, TY = L::TY, TX = L::TX, RX = L::RX, NR = L::NR, BX = L::BX, PS = L::PS;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
+    float2* ring = reinterpret_cast<float2*>(smem);                  // [9][NR][BX]
+    float2* win_r = reinterpret_cast<float2*>(smem + L::WIN_OFF);    // [WIN][RX]
+    float2* win_p = win_r + L::WIN * RX;                             // [WIN][RX]
+    constexpr int kCarry = 2 / SPT;
+    __shared__ __align__(16) float2 s_jcarry[kCarry * RX * SPT * 2];
+    __shared__ int s_last;
+    const int tid = threadIdx.x;
+    const int t_lx = tid % RX, t_j = tid / RX;
+    // window rows and column of this thread, as in k_step
+    const int t_m = (t_j + L::TR - kCarry) % L::TR;
+    const bool t_carry = t_j < kCarry;
+    const int t_w = (t_lx + 2) % RX;
+    float2* const jc = s_jcarry + ((t_carry ? t_j : 0) * RX + t_lx) * (SPT * 2);
+    const int it0 = a.cta_items[blockIdx.x], it_end = a.cta_items[blockIdx.x + 1];
+    const int step_k = a.step_k;
+    // The first item's tables are read ahead of the wait (as in k_step).
+    int4 w = make_int4(0, 0, 0, 0);
+    const LatDesc<float>* d = nullptr;
+    Geom g = {};
+    LatVals<float> v = {};
+    auto load_item = [&](int it) {
+        w = a.items[it];
+        d = &a.lat[w.x];
+        g = d->g;
+        v = d->v;
+    };
+    if (it0 < it_end) load_item(it0);
+    griddep_wait();
+    griddep_launch_dependents();
+    const uint64_t pol = a.l2_resident ? policy_evict_last() : policy_evict_normal();
+
+    for (int it = it0; it < it_end; ++it) {
+        if (it != it0) load_item(it);
+        const int x0 = w.y * TX, nx = g.nx, ny = g.ny;
+        const bool per_lat = ALLPER || g.periodic;
+        const int cur = *((volatile int*)&d->st->cur) ^ (step_k & 1);
+        const int form = step_k != 0 ? 2 : *((volatile int*)&d->st->pull);
+        const bool mom = form == 2;
+        const int pull = form != 0;
+        const size_t N = (size_t)nx * ny;
+        const float2* const m_in = reinterpret_cast<const float2*>(d->fbuf[cur]);
+        float2* const m_out = reinterpret_cast<float2*>(d->fbuf[cur ^ 1]);
+        float2 nf = pset(0.0f);
+        // The lattice column of ring column c (0 .. BX - 1), wrapped around the
+        // lattice, and the row of y, wrapped (periodic) or clamped to the
+        // lattice (walls: no site reads what lies beyond).
+        auto column = [&](int c) {
+            const int x = (x0 - 3 + c) % nx;
+            return x < 0 ? x + nx : x;
+        };
+        auto row = [&](int y) {
+            if (!per_lat) return min(max(y, 0), ny - 1);
+            y = y < 0 ? y + ny : y;
+            y = y >= ny ? y - ny : y;
+            return y >= ny ? y - ny : y;   // (ny = 8, 9 below a ragged tile)
+        };
+        const int xw = column(t_w + 1);
+        const int xe = column(tid & 1 ? BX - 1 : 0);   // outermost columns
+        struct Mom {
+            float2 r, zx, zy;
+        };
+        auto load_mom = [&](int y, int x) {
+            const size_t o = (size_t)row(y) * nx + x;
+            Mom m;
+            m.r = __ldcg(m_in + o);
+            m.zx = __ldcg(m_in + N + o);
+            m.zy = __ldcg(m_in + 2 * N + o);
+            return m;
+        };
+        // populations of a cell into ring slot row s, ring column c
+        auto put_mom = [&](const Mom& m, int s, int c) {
+            float2 h[9];
+            collide<float, float2, false, true>(nullptr, h, m.r, padd(pset(v.rho_ref), m.r), m.zx, m.zy, a.k,
+                                                m.r, m.r, 1.0f);
+            float2* o = ring + s * BX + c;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) o[i * PS] = h[i];
+        };
+        // the same from the population planes (the state before the first step)
+        auto put_pops = [&](int y, int x, int s, int c) {
+            const float2* f = m_in + (size_t)(row(y) + kGY) * g.pitch + (x + g.gx);
+            float2* o = ring + s * BX + c;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) o[i * PS] = __ldcg(f + i * g.plane);
+        };
+        const int ty_a = w.z, ty_b = w.w;
+        const int ya = ty_a * TY;
+        // the item's first NR rows, y = ya - 3 .. ya + 10
+        for (int r = t_j; r < NR; r += L::TR) {
+            if (mom) put_mom(load_mom(ya - 3 + r, xw), r, t_w + 1);
+            else put_pops(ya - 3 + r, xw, r, t_w + 1);
+        }
+        if (tid < 2 * NR) {
+            const int r = tid >> 1, c = tid & 1 ? BX - 1 : 0;
+            if (mom) put_mom(load_mom(ya - 3 + r, xe), r, c);
+            else put_pops(ya - 3 + r, xe, r, c);
+        }
+        Mom pf[SPT], pfe;   // the next tile's new rows (and outermost columns)
+        int base = 0;       // ring slot of row y0 - 3
+        auto slot_of = [&](int r) { return base + r >= NR ? base + r - NR : base + r; };
+        for (int ty = ty_a; ty < ty_b; ++ty) {
+            const int y0 = ty * TY;
+            if (ty > ty_a) {   // expand rows y0 + 3 .. y0 + 10
+#pragma unroll
+                for (int c = 0; c < SPT; ++c) {
+                    const int m = SPT * t_j + c;
+                    if (mom) put_mom(pf[c], slot_of(6 + m), t_w + 1);
+                    else put_pops(y0 + 3 + m, xw, slot_of(6 + m), t_w + 1);
+                }
+                if (tid < 2 * TY) {
+                    const int m = tid >> 1, c = tid & 1 ? BX - 1 : 0;
+                    if (mom) put_mom(pfe, slot_of(6 + m), c);
+                    else put_pops(y0 + 3 + m, xe, slot_of(6 + m), c);
+                }
+            }
+            if (mom && ty + 1 < ty_b) {
+#pragma unroll
+                for (int c = 0; c < SPT; ++c) pf[c] = load_mom(y0 + TY + 3 + SPT * t_j + c, xw);
+                if (tid < 2 * TY) pfe = load_mom(y0 + TY + 3 + (tid >> 1), xe);
+            }
+            __syncthreads();   // the ring's rows are there; the previous site phase is over
+            auto tile_body = [&](auto wall_tag) {
+                constexpr bool W = decltype(wall_tag)::value;
+                const bool per = !W || per_lat;
+                float2 jn[SPT][2];
+                // Density phase: window rows as in k_step; row k pulls from the
+                // ring rows k, k + 1, k + 2 above y0 - 3.
+                {
+                    const float2* rc = ring + t_w + 1;
+                    auto cell = [&](int k, float2& r, float2& q, float2* j) {
+                        cell_dev<P, PS, true>(rc + slot_of(k) * BX, rc + slot_of(k + 1) * BX,
+                                              rc + slot_of(k + 2) * BX, y0 - 2 + k, per, pull, g, v, r, q,
+                                              nullptr, j);
+                    };
+#pragma unroll
+                    for (int c = 0; c < SPT; ++c) {
+                        const int k = 4 + SPT * t_m + c;
+                        const int kk = k - TY;
+                        if (kk >= 0) {
+                            if (ty == ty_a) {
+                                float2 r, q, jt[2];
+                                cell(kk, r, q, jt);
+                                win_r[kk * RX + t_w] = r;
+                                win_p[kk * RX + t_w] = q;
+                                if (t_carry) {
+                                    jc[2 * c] = jt[0];
+                                    jc[2 * c + 1] = jt[1];
+                                }
+                            } else {
+                                win_r[kk * RX + t_w] = win_r[k * RX + t_w];
+                                win_p[kk * RX + t_w] = win_p[k * RX + t_w];
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int c = 0; c < SPT; ++c) {
+                        const int k = 4 + SPT * t_m + c;
+                        float2 r, q;
+                        cell(k, r, q, jn[c]);
+                        win_r[k * RX + t_w] = r;
+                        win_p[k * RX + t_w] = q;
+                    }
+                    if (t_carry) {
+#pragma unroll
+                        for (int c = 0; c < SPT; ++c) {
+                            const float2 px = jc[2 * c], py = jc[2 * c + 1];
+                            jc[2 * c] = jn[c][0];
+                            jc[2 * c + 1] = jn[c][1];
+                            jn[c][0] = px;
+                            jn[c][1] = py;
+                        }
+                    }
+                }
+                if (!per && (y0 < 2 || y0 + TY + 1 >= ny)) {   // mirror about the halfway walls
+                    __syncthreads();
+                    for (int c = tid; c < L::WIN * RX; c += L::NT) {
+                        const int k = c / RX, lx = c - k * RX;
+                        const int y = y0 - 2 + k;
+                        int ym;
+                        if (y < 0) ym = -1 - y;
+                        else if (y >= ny && y <= ny + 1) ym = 2 * ny - 1 - y;
+                        else continue;
+                        const int km = ym - (y0 - 2);
+                        win_r[k * RX + lx] = win_r[km * RX + lx];
+                        win_p[k * RX + lx] = win_p[km * RX + lx];
+                    }
+                }
+                __syncthreads();
+                // Site phase.
+                const int lx = t_lx, ly = SPT * t_j;
+                const int x = x0 + lx, y = y0 + ly;
+                if (lx < TX && x < nx && y < ny) {
+                    float2 fx[SPT], fy[SPT], qx[SPT], qy[SPT], dp[SPT], dr[SPT];
+                    force_sums<SPT, RX>(win_p + ly * RX + lx + 2, win_r + ly * RX + lx + 2, a.k, fx, fy, qx,
+                                        qy, dp, dr);
+                    float2* const o = m_out + (size_t)y * nx + x;
+#pragma unroll
+                    for (int s = 0; s < SPT; ++s) {
+                        const int ys = y + s;
+                        const bool valid = s == 0 || ys < ny;
+                        const float2 rho = padd(pset(v.rho_ref), dr[s]);
+                        if (valid) note_nonfinite(rho, nf);
+                        float2 Fx, Fy, zx, zy;
+                        site_force<GEN>(fx[s], fy[s], qx[s], qy[s], dp[s], rho, ys, v, a.k, Fx, Fy);
+                        site_velocity<P, true>(rho, jn[s][0], jn[s][1], Fx, Fy, false, a.k, zx, zy);
+                        if (valid) {
+                            float2* const os = o + s * nx;
+                            st_pair(os, dr[s], pol);
+                            st_pair(os + N, zx, pol);
+                            st_pair(os + 2 * N, zy, pol);
+                        }
+                        if (!per && valid && (ys == 0 || ys == ny - 1)) {
+                            float2 h[9];
+                            collide<float, float2, false, true>(nullptr, h, dr[s], rho, zx, zy, a.k, Fx, Fy,
+                                                                1.0f);
+                            // h[0] = omega w_0 Q as the next step's expansion rounds it: here it
+                            // has no use but the density's sum, into which the compiler fuses
+                            // the packed product; a scalar one it does not
+                            const float2 Q = pfma(pmul(rho, pset(-4.0f / 6.0f)), pfma(zx, zx, pmul(zy, zy)), dr[s]);
+                            h[0] = make_float2(__fmul_rn(a.k.omw[0].x, Q.x), __fmul_rn(a.k.omw[0].y, Q.y));
+                            reinterpret_cast<float2*>(d->wallx)[(ys == 0 ? 0 : nx) + x] =
+                                wall_momentum<P>(h, ys == 0, v);
+                        }
+                    }
+                }
+            };
+            if constexpr (ALLPER)
+                tile_body(std::false_type{});
+            else if (per_lat || (y0 >= 3 && y0 + TY + 3 <= ny))
+                tile_body(std::false_type{});
+            else
+                tile_body(std::true_type{});
+            base = slot_of(TY);
+        }
+        if (!(nf.x == 0.0f && nf.y == 0.0f)) atomicOr(&d->st->err, ERR_NONFINITE);
+    }
+    if constexpr (!ALLPER) {
+        __syncthreads();   // this CTA's wall-site values are written
+        wall_sums<P, L>(a, it0, it_end, tid);
+    }
+    if (!a.advance) return;
+    __syncthreads();
+    if (tid == 0) s_last = ticket_arrive(a.ticket) == (unsigned int)(gridDim.x - 1);
+    __syncthreads();
+    if (!s_last) return;
+    advance_lattices<L::NT>(a, tid, 2);
+    if (tid == 0) *a.ticket = 0u;
+}
+
+// The populations of a state held by its moments, into population planes with
+// their ghost copies.
+__global__ void k_expand(Geom g, const __grid_constant__ Coef<float> k, const float2* mom, float2* fout) {
+    const size_t N = (size_t)g.nx * g.ny;
+    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < N;
+         idx += (size_t)gridDim.x * blockDim.x) {
+        const int x = (int)(idx % g.nx), y = (int)(idx / g.nx);
+        const float2 r = mom[idx];
+        float2 h[9];
+        collide<float, float2, false, true>(nullptr, h, r, padd(pset(k.rho_ref), r), mom[N + idx],
+                                            mom[2 * N + idx], k, r, r, 1.0f);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) put2<float2>(fout, g, i, x, y, h[i]);
+    }
+}
+#endif
 
 // --------------------------------------------------------- observe kernel
 // One CTA per tile of one lattice: fields, populations or totals of the
@@ -1355,11 +1680,38 @@ __global__ void __launch_bounds__(Layout<P>::NT)
         s_fail = 0;
         mbar_init(&bar, 1);
         fence_mbar_init();
+    }
+    bool from_mom = false;
+#if LB_PREC == 1
+    from_mom = a.mom != nullptr;
+    if (from_mom) {   // the box's populations from the state's moments, wrapped (or clamped at walls)
+        const size_t N = (size_t)g.nx * g.ny;
+        for (int c = tid; c < L::BY * L::BX; c += L::NT) {
+            const int by = c / L::BX, bx = c - by * L::BX;
+            int x = (x0 - L::GX + bx) % g.nx, y = y0 - kGY + by;
+            x = x < 0 ? x + g.nx : x;
+            if (per) {
+                y %= g.ny;
+                y = y < 0 ? y + g.ny : y;
+            } else {
+                y = min(max(y, 0), g.ny - 1);
+            }
+            const float2* m = a.mom + (size_t)y * g.nx + x;
+            const float2 r = m[0];
+            float2 h[9];
+            collide<float, float2, false, true>(nullptr, h, r, padd(pset(a.k.rho_ref), r), m[N], m[2 * N], a.k,
+                                                r, r, 1.0f);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) box[i * PS + c] = h[i];
+        }
+    }
+#endif
+    if (tid == 0 && !from_mom) {
         mbar_expect_tx(&bar, (uint32_t)L::BOX_BYTES);
         tma_load_3d(box, &tin, 2 * x0, y0, 0, &bar);
     }
     __syncthreads();
-    if (!mbar_wait_bounded(&bar, 0)) s_fail = 1;
+    if (!from_mom && !mbar_wait_bounded(&bar, 0)) s_fail = 1;
     __syncthreads();
     double red[4] = {0.0, 0.0, 0.0, 0.0};
     bool bad = false;
@@ -1589,6 +1941,18 @@ static cudaError_t configure_all() {
     opt_shape(std::integral_constant<int, SHAPE_8>{});
     opt_shape(std::integral_constant<int, SHAPE_16>{});
     opt_shape(std::integral_constant<int, SHAPE_8X2>{});
+#if LB_PREC == 1
+    auto opt_moments = [&](auto tag) {
+        constexpr int SH = decltype(tag)::value;
+        constexpr int bytes = MLayout<SH>::SMEM;
+        opt(k_step_m<0, SH>, bytes);
+        opt(k_step_m<1, SH>, bytes);
+        opt(k_step_m<2, SH>, bytes);
+        opt(k_step_m<3, SH>, bytes);
+    };
+    opt_moments(std::integral_constant<int, SHAPE_M8>{});
+    opt_moments(std::integral_constant<int, SHAPE_M8X2>{});
+#endif
     opt(k_observe<P, 2>, L::SMEM_OBS);
     opt(k_observe<P, 3>, L::SMEM_OBS);
     return e;
@@ -1648,6 +2012,39 @@ static cudaError_t launch_step_shape(const BatchArgs<typename Prec<P>::C>& a, in
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+#if LB_PREC == 1
+template <int SH>
+static cudaError_t launch_moments_shape(const BatchArgs<float>& a, int variant, dim3 grid, cudaStream_t s) {
+    typedef MLayout<SH> L;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(L::NT, 1, 1);
+    cfg.dynamicSmemBytes = L::SMEM;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl_enabled() ? 1 : 0;
+    cudaError_t e;
+    switch (variant & 3) {
+        case 0: e = cudaLaunchKernelEx(&cfg, k_step_m<0, SH>, a); break;
+        case 1: e = cudaLaunchKernelEx(&cfg, k_step_m<1, SH>, a); break;
+        case 2: e = cudaLaunchKernelEx(&cfg, k_step_m<2, SH>, a); break;
+        default: e = cudaLaunchKernelEx(&cfg, k_step_m<3, SH>, a); break;
+    }
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+cudaError_t launch_expand(const Geom& g, const Coef<float>& k, const float2* mom, void* fout,
+                          cudaStream_t s) {
+    const long long N = (long long)g.nx * g.ny;
+    const long long blocks = (N + 255) / 256;
+    k_expand<<<(unsigned)(blocks < 152 * 32 ? blocks : 152 * 32), 256, 0, s>>>(
+        g, k, mom, reinterpret_cast<float2*>(fout));
+    return cudaGetLastError();
+}
+#endif
+
 template <int P>
 cudaError_t launch_step_prec(const void* args, int variant, int shape, dim3 grid, cudaStream_t s) {
     typedef typename Prec<P>::C C;
@@ -1657,6 +2054,10 @@ cudaError_t launch_step_prec(const void* args, int variant, int shape, dim3 grid
     if (shape == SHAPE_8) return launch_step_shape<P, SHAPE_8>(a, variant, grid, s);
     if constexpr (has_shape(P, SHAPE_16))
         if (shape == SHAPE_16) return launch_step_shape<P, SHAPE_16>(a, variant, grid, s);
+#if LB_PREC == 1
+    if (shape == SHAPE_M8) return launch_moments_shape<SHAPE_M8>(a, variant, grid, s);
+    if (shape == SHAPE_M8X2) return launch_moments_shape<SHAPE_M8X2>(a, variant, grid, s);
+#endif
     if constexpr (has_shape(P, SHAPE_8X2))
         if (shape == SHAPE_8X2) return launch_step_shape<P, SHAPE_8X2>(a, variant, grid, s);
     return cudaErrorInvalidValue;

@@ -320,4 +320,25 @@ struct Layout {
     static_assert(SMEM <= 227 * 1024 - 1024 && SMEM_OBS <= 227 * 1024, "shared memory");
 };
 
+// Layout of the moment kernel (k_step_m): 60 x 8 tiles; a ring of 14 rows of
+// populations (the 8 + 6 rows a tile's deviation window pulls from), columns
+// x0 - 3 .. x0 + 62, and the deviation windows.  SHAPE_M8: one site per thread,
+// 512 threads; SHAPE_M8X2: two vertically adjacent sites per thread, two CTAs
+// of 256 threads per SM.
+template <int SH>
+struct MLayout {
+    typedef float2 T2;
+    typedef float C;
+    typedef float2 C2;
+    static constexpr int SPT = SH == SHAPE_M8 ? 1 : 2;
+    static constexpr int CTAS = shape_ctas(SH);
+    static constexpr int TX = Prec<LB_FP32>::TX, TR = 8 / SPT, TY = 8, RX = TX + 4;
+    static constexpr int NT = RX * TR;
+    static constexpr int WIN = TY + 4;
+    static constexpr int NR = TY + 6, BX = TX + 6, PS = NR * BX;   // ring rows, columns, plane stride
+    static constexpr int WIN_OFF = (9 * PS * (int)sizeof(float2) + 127) / 128 * 128;
+    static constexpr int SMEM = WIN_OFF + 2 * WIN * RX * (int)sizeof(float2) + 128;
+    static_assert(CTAS * (SMEM + 4096) <= 228 * 1024, "resident CTAs");
+};
+
 }  // namespace lbgb

@@ -146,6 +146,11 @@ lb_status build(lb_pool* P, Choice c) {
     std::vector<Lattice*> lats;
     for (int j : P->active) lats.push_back(&P->members[(size_t)j].lat);
     const int nlat = (int)lats.size();
+    if (!shape_moments(c.shape))
+        for (Lattice* L : lats) {
+            lb_status s = lattice_to_populations(*L, P->stream);
+            if (s != LB_OK) return s;
+        }
     // item tables: items are most numerous for seg = 1 (one per tile)
     size_t tiles = 0, strips = 0;
     for (Lattice* L : lats) {
@@ -207,7 +212,7 @@ lb_status run_steps(lb_pool* P, long long k) {
 void advanced(lb_pool* P, long long k) {
     for (int j : P->active) {
         Member& m = P->members[(size_t)j];
-        lattice_advanced(m.lat, k);
+        lattice_advanced(m.lat, k, P->launch.shape);
         m.done += k;
     }
 }
@@ -217,7 +222,9 @@ void advanced(lb_pool* P, long long k) {
 std::vector<Choice> candidates(lb_pool* P) {
     const int prec = P->shared.precision;
     std::vector<Choice> out;
-    for (int shape : {SHAPE_8, SHAPE_16, SHAPE_8X2}) {
+    const bool moments = P->forced_rows == 0 && moments_ok(P->members[(size_t)P->active[0]].lat);
+    for (int shape : {SHAPE_8, SHAPE_16, SHAPE_8X2, SHAPE_M8, SHAPE_M8X2}) {
+        if (shape_moments(shape) != moments) continue;
         if (!has_shape(prec, shape) || (P->forced_rows != 0 && shape_rows(shape) != P->forced_rows)) continue;
         // (where two CTAs fit an SM the 16-row tile runs only when asked for)
         if (shape == SHAPE_16 && has_shape(prec, SHAPE_8X2) && P->forced_rows == 0) continue;
@@ -248,7 +255,8 @@ Choice untuned(lb_pool* P) {
         const Lattice& L = P->members[(size_t)j].lat;
         tiles8 += (long long)L.nstrips * L.ntiles_y;
     }
-    return {P->forced_seg, shape_of_rows(P->shared.precision, P->forced_rows, tiles8, P->sms)};
+    return {P->forced_seg, shape_of_rows(P->shared.precision, moments_ok(P->members[(size_t)P->active[0]].lat),
+                                        P->forced_rows, tiles8, P->sms)};
 }
 std::string cache_key(lb_pool* P) {
     return signature(P) + "|" + std::to_string(P->forced_seg) + "|" + std::to_string(P->forced_rows);
@@ -520,7 +528,7 @@ lb_status lb_pool_set_partition(lb_pool* P, int32_t seg) {
 
 lb_status lb_pool_set_tile_rows(lb_pool* P, int32_t rows) {
     if (!P) return LB_ERR_INVALID;
-    if (shape_of_rows(P->shared.precision, rows, 0, P->sms) == 0) return LB_ERR_INVALID;
+    if (shape_of_rows(P->shared.precision, false, rows, 0, P->sms) == 0) return LB_ERR_INVALID;
     P->forced_rows = rows;
     P->built = false;
     drop_graph(P);

@@ -54,9 +54,9 @@ cudaError_t launch_init_seeded(int precision, const Geom& g, const void* coef, v
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_init_fields(int precision, const Geom& g, const void* coef, void* fout,
+cudaError_t launch_init_fields(int precision, const Geom& g, const void* coef, void* fout, int mode,
                                const double* fields, cudaStream_t s) {
-    LB_SWITCH(precision, return launch_init_prec<P>(g, coef, fout, 1, fields, 0, 0, 0, 0, 0, s))
+    LB_SWITCH(precision, return launch_init_prec<P>(g, coef, fout, mode, fields, 0, 0, 0, 0, 0, s))
     return cudaErrorInvalidValue;
 }
 

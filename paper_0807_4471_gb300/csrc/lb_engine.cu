@@ -699,8 +699,13 @@ lb_status lattice_observe(Lattice& L, int obs, double* out, int q0, int q1, cuda
 
 static lb_status lattice_observe_pull(Lattice& L, int obs, double* out, int q0, int q1, int pull,
                                       cudaStream_t s) {
-    const int tx = kernel_tile_x(L.p.precision), ty = kernel_tile_y(L.p.precision);
-    dim3 grid((unsigned)((L.p.nx + tx - 1) / tx), (unsigned)((L.p.ny + ty - 1) / ty), 1);
+    // CTAs take several tiles each once every SM is full (2048 threads)
+    const long long tiles = (long long)L.nstrips * L.ntiles_y;
+    const int threads = L.p.precision == LB_FP64 ? 256 : 512;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const long long most = (long long)device_sms(dev) * (2048 / threads);
+    dim3 grid((unsigned)std::min(tiles, most), 1, 1);
     cudaError_t e;
     if (L.p.precision == LB_FP64) {
         StepArgs<double> a;
@@ -794,14 +799,10 @@ lb_status lattice_init_fields(Lattice& L, const double* rho_A, const double* rho
     double* stage = reinterpret_cast<double*>(L.fbuf[1]);
     cudaError_t e = cudaMemcpyAsync(stage, rho_A, n * 8, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(stage + n, rho_B, n * 8, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess)
-        e = ux ? cudaMemcpyAsync(stage + 2 * n, ux, n * 8, cudaMemcpyHostToDevice, s)
-               : cudaMemsetAsync(stage + 2 * n, 0, n * 8, s);
-    if (e == cudaSuccess)
-        e = uy ? cudaMemcpyAsync(stage + 3 * n, uy, n * 8, cudaMemcpyHostToDevice, s)
-               : cudaMemsetAsync(stage + 3 * n, 0, n * 8, s);
+    if (e == cudaSuccess && ux) e = cudaMemcpyAsync(stage + 2 * n, ux, n * 8, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess && uy) e = cudaMemcpyAsync(stage + 3 * n, uy, n * 8, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return cuda_status(e);
-    e = launch_init_fields(L.p.precision, L.g, coef_ptr(L), L.fbuf[0], stage, s);
+    e = launch_init_fields(L.p.precision, L.g, coef_ptr(L), L.fbuf[0], 1 | (ux ? 2 : 0) | (uy ? 4 : 0), stage, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     return cuda_status(e);
 }

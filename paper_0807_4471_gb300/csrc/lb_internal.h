@@ -218,8 +218,8 @@ int kernel_staged(int precision, int shape);
 // Step: the persistent multi-lattice kernel (args: BatchArgs<C>), variant
 // bit 0 = every lattice periodic, bit 1 = general forcing, bit 2 = 1 - omega
 // rounds to zero for both species (the collision reads no populations), in one of the
-// precision's tile shapes.  Observe: one lattice, one CTA per 8-row
-// tile (args: StepArgs<C>, tin: tile-box load map).
+// precision's tile shapes.  Observe: one lattice (args: StepArgs<C>, tin: tile-box
+// load map), at most one CTA per 8-row tile.
 cudaError_t launch_step(int precision, const void* args, int variant, int shape, dim3 grid,
                         cudaStream_t s);
 // Opt the kernels of a precision into their shared memory (once per device;
@@ -230,7 +230,8 @@ cudaError_t launch_observe(int precision, const CUtensorMap* tin, const void* ar
 cudaError_t launch_init_seeded(int precision, const Geom& g, const void* coef, void* fout,
                                double rho0, double amp, double u_wall, int init_shear,
                                unsigned long long seed, cudaStream_t s);
-cudaError_t launch_init_fields(int precision, const Geom& g, const void* coef, void* fout,
+// mode: 1, + 2 with u_x, + 4 with u_y (else zero) in fields [4][ny][nx]
+cudaError_t launch_init_fields(int precision, const Geom& g, const void* coef, void* fout, int mode,
                                const double* fields, cudaStream_t s);
 
 // FP32: the populations f* of a state held by its moments, into a population

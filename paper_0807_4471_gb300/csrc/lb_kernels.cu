@@ -555,10 +555,7 @@ struct SiteOut {
     int valid;             // 0: a site beyond the lattice, computed only to keep
                            // the site updates of a thread free of branches:
                            // its global stores and non-finite flag are dropped
-    int obs;               // ObsKind (observe kernel) or OBS_NONE
-    void* wallx;           // step: the lattice's wall-momentum pairs, [2][nx] compute type
-    double* obs_out;
-    int q0, q1;
+    void* wallx;           // the lattice's wall-momentum pairs, [2][nx] compute type
 };
 
 // Body acceleration along x at lattice row y.
@@ -621,27 +618,24 @@ __device__ __forceinline__ C2 wall_momentum(const C2 sv[9], bool down, const Lat
 }
 
 // One lattice site, given its force sums: moments from its pulled
-// populations, the force of Eq. (2), and either the forced BGK collision and
-// write-back (OBS = false) or the observables (OBS = true).  Both species are
-// carried as (A, B) pairs throughout.  TAU1 (omega = 1 for both species,
-// OBS = false): the collision needs the populations only through j, which the
-// caller passes in jg = {jx, jy} (in the storage scale); bm, b0 and bp are
-// not read.  Non-finite densities: the step (OBS = false) accumulates
-// 0 * rho into *nf, which turns NaN at an inf or NaN density and stays zero
-// otherwise; the observables set `bad`.
-template <int P, bool OBS, bool GEN, int PS, int SINK, bool TAU1 = false>
+// populations, the force of Eq. (2), the forced BGK collision and the
+// write-back.  Both species are carried as (A, B) pairs throughout.  TAU1
+// (omega = 1 for both species): the collision needs the populations only
+// through j, which the caller passes in jg = {jx, jy} (in the storage scale);
+// bm, b0 and bp are not read.  *nf accumulates 0 * rho, which turns NaN at an
+// inf or NaN density and stays zero otherwise.
+template <int P, bool GEN, int PS, int SINK, bool TAU1 = false>
 __device__ __forceinline__ void site_update(
     const typename Prec<P>::T2* bm, const typename Prec<P>::T2* b0,
     const typename Prec<P>::T2* bp, typename Prec<P>::C2 fxl, typename Prec<P>::C2 fyl,
     typename Prec<P>::C2 qx, typename Prec<P>::C2 qy, typename Prec<P>::C2 dpsi,
     typename Prec<P>::C2 drho, int x, int y, bool per, int pull, const Geom& g,
     const LatVals<typename Prec<P>::C>& v, const Coef<typename Prec<P>::C>& k,
-    const SiteOut<typename Prec<P>::T2>& o, double red[4], bool& bad,
-    typename Prec<P>::C2* nf = nullptr, const typename Prec<P>::C2* jg = nullptr) {
+    const SiteOut<typename Prec<P>::T2>& o, typename Prec<P>::C2* nf,
+    const typename Prec<P>::C2* jg = nullptr) {
     typedef typename Prec<P>::T2 T2;
     typedef typename Prec<P>::C C;
     typedef typename Prec<P>::C2 C2;
-    static_assert(!(TAU1 && OBS), "the observables read the populations");
     C2 h[9];
     C2 jx, jy;
     if constexpr (TAU1) {
@@ -652,42 +646,9 @@ __device__ __forceinline__ void site_update(
         moments<P>(h, jx, jy);
     }
     const C2 rho = padd(pset(v.rho_ref), drho);
-    if constexpr (OBS) {
-        if (o.valid && !(isfinite(rho.x) && isfinite(rho.y))) bad = true;
-    } else if (o.valid) {
-        note_nonfinite(rho, *nf);   // stays zero unless a density is inf or NaN
-    }
-
+    if (o.valid) note_nonfinite(rho, *nf);   // stays zero unless a density is inf or NaN
     C2 Fx, Fy;
     site_force<GEN>(fxl, fyl, qx, qy, dpsi, rho, y, v, k, Fx, Fy);
-
-    if (OBS) {
-        const long long N = (long long)g.nx * g.ny;
-        const long long idx = (long long)y * g.nx + x;
-        const double rA = (double)v.rho_ref + (double)drho.x;
-        const double rB = (double)v.rho_ref + (double)drho.y;
-        const double tot = rA + rB;
-        const double mx = (double)jx.x + (double)jx.y + 0.5 * ((double)Fx.x + (double)Fx.y);
-        const double my = (double)jy.x + (double)jy.y + 0.5 * ((double)Fy.x + (double)Fy.y);
-        if (o.obs == OBS_FIELDS) {
-            o.obs_out[idx] = rA;
-            o.obs_out[N + idx] = rB;
-            o.obs_out[2 * N + idx] = tot != 0.0 ? mx / tot : 0.0;
-            o.obs_out[3 * N + idx] = tot != 0.0 ? my / tot : 0.0;
-        } else if (o.obs == OBS_POPS) {
-#pragma unroll
-            for (int q = 0; q < 18; ++q)
-                if (q >= o.q0 && q < o.q1)
-                    o.obs_out[(long long)(q - o.q0) * N + idx] =
-                        (double)(q < 9 ? h[q % 9].x : h[q % 9].y) * (double)inv_scale_of<P>() +
-                        wgt<double>(q % 9) * (double)v.rho_ref;
-        }
-        red[0] += rA;
-        red[1] += rB;
-        red[2] += mx;
-        red[3] += my;
-        return;
-    }
 
     // Eq. (1): forced BGK relaxation.
     const bool source = GEN && k.source;
@@ -867,25 +828,31 @@ __device__ __forceinline__ void write_edges(const typename Prec<P>::T2* stage,
     }
 }
 
-// FP64 block reduction of red[0..3] (all threads), result valid in thread 0.
+// FP64 block sums of red[0..3] over all threads; sum k is the result of thread
+// 8 k.  The four sums share the butterfly: its first two steps hand half of the
+// lanes' values over, so a warp takes 6 FP64 additions instead of 20.
 template <int NT>
-__device__ __forceinline__ void block_sum4(double red[4], double (*s_red)[4]) {
+__device__ __forceinline__ double block_sum4(const double red[4], double (*s_red)[4]) {
+    const unsigned full = 0xffffffffu;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) red[k] = warp_sum(red[k]);
+    const bool h16 = lane & 16, h8 = lane & 8;
+    double a = (h16 ? red[2] : red[0]) + __shfl_xor_sync(full, h16 ? red[0] : red[2], 16);
+    double b = (h16 ? red[3] : red[1]) + __shfl_xor_sync(full, h16 ? red[1] : red[3], 16);
+    a = (h8 ? b : a) + __shfl_xor_sync(full, h8 ? a : b, 8);
+    a += __shfl_xor_sync(full, a, 4);
+    a += __shfl_xor_sync(full, a, 2);
+    a += __shfl_xor_sync(full, a, 1);
     __syncthreads();
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) s_red[warp][k] = red[k];
+    if ((lane & 7) == 0) s_red[warp][lane >> 3] = a;
     __syncthreads();
-    if (tid == 0) {
-        double v[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int w = 0; w < NT / 32; ++w)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) v[k] += s_red[w][k];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) red[k] = v[k];
+    if (warp == 0) {
+        a = 0.0;
+        for (int w = lane & 7; w < NT / 32; w += 8) a += s_red[w][lane >> 3];
+        a += __shfl_xor_sync(full, a, 4);
+        a += __shfl_xor_sync(full, a, 2);
+        a += __shfl_xor_sync(full, a, 1);
     }
+    return a;
 }
 
 // ------------------------------------------------------------ step kernel
@@ -1047,7 +1014,6 @@ __global__ void __launch_bounds__(Layout<P, SH>::NT, Layout<P, SH>::CTAS)
         while (p_pos < released + L::NB && issue_next()) {}
     };
 
-    bool bad_unused = false;   // (the observables' flag; the step uses nf)
     int c_pos = 0;   // ring position of the current item's first block
     for (int it = a.cta_items[blockIdx.x]; it < it_end && !s_fail; ++it) {
         const int4 w = a.items[it];
@@ -1214,7 +1180,6 @@ __global__ void __launch_bounds__(Layout<P, SH>::NT, Layout<P, SH>::CTAS)
                         o.rbits = 0u;
                         [[maybe_unused]] uint32_t srh = 0u;   // the shared hash of this thread's sites
                         if constexpr (sizeof(T2) == 4) srh = sr_hash(key, x, y, g.nx);
-                        o.obs = OBS_NONE;
                         o.valid = 1;
                         o.wallx = d->wallx;
                         if constexpr (!STAGED) {
@@ -1241,17 +1206,16 @@ __global__ void __launch_bounds__(Layout<P, SH>::NT, Layout<P, SH>::CTAS)
                                         : ys < 3 ? (long long)g.ny * g.pitch
                                         : (ys >= g.ny - 3 ? -(long long)g.ny * g.pitch : 0);
                             }
-                            double wr[4];   // (observables only)
                             if constexpr (TAU1) {
-                                site_update<P, false, GEN, PS, STAGED ? SINK_STAGE : SINK_GLOBAL, true>(
+                                site_update<P, GEN, PS, STAGED ? SINK_STAGE : SINK_GLOBAL, true>(
                                     nullptr, nullptr, nullptr, fx[s], fy[s], qx[s], qy[s], dp[s], dr[s],
-                                    x, ys, per, pull, g, v, a.k, o, wr, bad_unused, &nf, jn[s]);
+                                    x, ys, per, pull, g, v, a.k, o, &nf, jn[s]);
                             } else {
                                 const int bc = lx + L::GX;
-                                site_update<P, false, GEN, PS, STAGED ? SINK_STAGE : SINK_GLOBAL>(
+                                site_update<P, GEN, PS, STAGED ? SINK_STAGE : SINK_GLOBAL>(
                                     brow(ly + s + 2, bc), brow(ly + s + 3, bc), brow(ly + s + 4, bc),
                                     fx[s], fy[s], qx[s], qy[s], dp[s], dr[s], x, ys, per, pull, g, v,
-                                    a.k, o, wr, bad_unused, &nf);
+                                    a.k, o, &nf);
                             }
                         }
                         if constexpr (STAGED) fence_proxy_async();   // staging writes before the bulk store
@@ -1647,10 +1611,27 @@ __global__ void k_expand(Geom g, const __grid_constant__ Coef<float> k, const fl
 #endif
 
 // --------------------------------------------------------- observe kernel
-// One CTA per tile of one lattice: fields, populations or totals of the
-// current state, with the same site arithmetic as the step.
-template <int P, int V>
-__global__ void __launch_bounds__(Layout<P>::NT)
+// Fields, totals or populations of one lattice's current state, with the same
+// site arithmetic as the step; CTAs take tiles b, b + G, ...  GB300 has two FP64
+// lanes per SM and clock, and the observables' FP64 work bounded this kernel
+// (2048^2 FP16: 51 FP64-pipe operations a site for the totals, 504 us; 71 for
+// the fields, 638 us): floats are widened by integer operations, the sums are
+// reduced once per CTA instead of once per tile, one reciprocal serves both
+// velocity components, and populations take no force and no totals (2048^2 FP16:
+// 15 operations, 154 us, and 21, 222 us; FP32 from the moments about the same).
+
+// A float widened to double.  The conversion instruction runs on the FP64
+// pipe; a normal value's bits are moved by integer operations instead.
+__device__ __forceinline__ double widen(float x) {
+    const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+    return m == 0u ? __hiloint2double((int)b, 0) : (double)x;
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
+template <int P, int V, bool POPS>
+__global__ void __launch_bounds__(Layout<P>::NT, P == LB_FP64 ? 1 : 2)
     k_observe(const __grid_constant__ CUtensorMap tin,
               const __grid_constant__ StepArgs<typename Prec<P>::C> a) {
     typedef Layout<P> L;
@@ -1668,7 +1649,6 @@ __global__ void __launch_bounds__(Layout<P>::NT)
     __shared__ int s_fail, s_last;
     __shared__ double s_red[L::NT / 32][4];
     const int tid = threadIdx.x;
-    const int x0 = blockIdx.x * L::TX, y0 = blockIdx.y * L::TY;
     const Geom& g = a.g;
     const bool per = g.periodic != 0;
     const LatVals<C> v = vals_of(a.k);
@@ -1676,117 +1656,168 @@ __global__ void __launch_bounds__(Layout<P>::NT)
 #if LB_PREC == 0
     tab = g_exp_tab;
 #endif
+    bool from_mom = false;
+#if LB_PREC == 1
+    from_mom = a.mom != nullptr;
+#endif
     if (tid == 0) {
         s_fail = 0;
         mbar_init(&bar, 1);
         fence_mbar_init();
     }
-    bool from_mom = false;
-#if LB_PREC == 1
-    from_mom = a.mom != nullptr;
-    if (from_mom) {   // the box's populations from the state's moments, wrapped (or clamped at walls)
-        const size_t N = (size_t)g.nx * g.ny;
-        for (int c = tid; c < L::BY * L::BX; c += L::NT) {
-            const int by = c / L::BX, bx = c - by * L::BX;
-            int x = (x0 - L::GX + bx) % g.nx, y = y0 - kGY + by;
-            x = x < 0 ? x + g.nx : x;
-            if (per) {
-                y %= g.ny;
-                y = y < 0 ? y + g.ny : y;
-            } else {
-                y = min(max(y, 0), g.ny - 1);
-            }
-            const float2* m = a.mom + (size_t)y * g.nx + x;
-            const float2 r = m[0];
-            float2 h[9];
-            collide<float, float2, false, true>(nullptr, h, r, padd(pset(a.k.rho_ref), r), m[N], m[2 * N], a.k,
-                                                r, r, 1.0f);
-#pragma unroll
-            for (int i = 0; i < 9; ++i) box[i * PS + c] = h[i];
-        }
-    }
-#endif
-    if (tid == 0 && !from_mom) {
-        mbar_expect_tx(&bar, (uint32_t)L::BOX_BYTES);
-        tma_load_3d(box, &tin, 2 * x0, y0, 0, &bar);
-    }
     __syncthreads();
-    if (!from_mom && !mbar_wait_bounded(&bar, 0)) s_fail = 1;
-    __syncthreads();
+    const int ntx = (g.nx + L::TX - 1) / L::TX, ntiles = ntx * ((g.ny + L::TY - 1) / L::TY);
+    const size_t N = (size_t)g.nx * g.ny;
     double red[4] = {0.0, 0.0, 0.0, 0.0};
     bool bad = false;
-    if (!s_fail) {
-        // box row of lattice row y: y - y0 + kGY; deviation tile row: y - y0 + 2
-        for (int c = tid; c < L::RX * L::RY; c += L::NT) {
-            const int ly = c / L::RX, lx = c - ly * L::RX;
-            const int y = y0 - 2 + ly;
-            if (!per && (y < 0 || y >= g.ny)) continue;
-            const T2* b0 = box + (ly + 1) * L::BX + lx - 2 + L::GX;
-            C2 r, p;
-            cell_dev<P, PS>(b0 - L::BX, b0, b0 + L::BX, y, per, a.pull, g, v, r, p, tab);
-            srho[ly * L::RX + lx] = r;
-            spsi[ly * L::RX + lx] = p;
-        }
-        if (!per) {
-            __syncthreads();
-            for (int c = tid; c < L::RX * L::RY; c += L::NT) {
-                const int ly = c / L::RX, lx = c - ly * L::RX;
-                const int y = y0 - 2 + ly;
-                int ym;
-                if (y < 0) ym = -1 - y;
-                else if (y >= g.ny) ym = 2 * g.ny - 1 - y;
-                else continue;
-                const int lm = ym - (y0 - 2);
-                if (lm < 0 || lm >= L::RY) continue;
-                srho[ly * L::RX + lx] = srho[lm * L::RX + lx];
-                spsi[ly * L::RX + lx] = spsi[lm * L::RX + lx];
+    int phase = 0;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, phase ^= 1) {
+        const int x0 = (tile % ntx) * L::TX, y0 = (tile / ntx) * L::TY;
+#if LB_PREC == 1
+        if (from_mom) {   // the box's populations from the state's moments, wrapped (or clamped at walls)
+            for (int c = tid; c < L::BY * L::BX; c += L::NT) {
+                const int by = c / L::BX, bx = c - by * L::BX;
+                int x = (x0 - L::GX + bx) % g.nx, y = y0 - kGY + by;
+                x = x < 0 ? x + g.nx : x;
+                if (per) {
+                    y %= g.ny;
+                    y = y < 0 ? y + g.ny : y;
+                } else {
+                    y = min(max(y, 0), g.ny - 1);
+                }
+                const float2* m = a.mom + (size_t)y * g.nx + x;
+                const float2 r = m[0];
+                float2 h[9];
+                collide<float, float2, false, true>(nullptr, h, r, padd(pset(a.k.rho_ref), r), m[N], m[2 * N],
+                                                    a.k, r, r, 1.0f);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) box[i * PS + c] = h[i];
             }
         }
+#endif
+        if (!from_mom) {
+            if (tid == 0) {
+                fence_proxy_async();   // generic reads of the previous tile's box before async writes
+                mbar_expect_tx(&bar, (uint32_t)L::BOX_BYTES);
+                tma_load_3d(box, &tin, 2 * x0, y0, 0, &bar);
+            }
+            if (!mbar_wait_bounded(&bar, phase)) s_fail = 1;
+        }
         __syncthreads();
+        if (s_fail) break;
         const int lx = tid % L::RX, ly = tid / L::RX;
         const int x = x0 + lx, y = y0 + ly;
-        if (lx < L::TX && x < g.nx && y < g.ny) {
-            const T2* b0 = box + (ly + kGY) * L::BX + lx + L::GX;
+        const bool site = lx < L::TX && x < g.nx && y < g.ny;
+        const T2* b0 = box + (ly + kGY) * L::BX + lx + L::GX;
+        const size_t idx = (size_t)y * g.nx + x;
+        C2 h[9];
+        if constexpr (POPS) {
+            if (site) {
+                load_site<P, PS>(b0 - L::BX, b0, b0 + L::BX, y, per, a.pull, g, v, h);
+                const C2 r = sum9(h);
+                if (!(isfinite(r.x) && isfinite(r.y))) bad = true;
+                const double is = (double)inv_scale_of<P>(), rref = (double)v.rho_ref;
+#pragma unroll
+                for (int q = 0; q < 18; ++q)
+                    if (q >= a.q0 && q < a.q1)
+                        a.obs_out[(size_t)(q - a.q0) * N + idx] =
+                            widen(q < 9 ? h[q % 9].x : h[q % 9].y) * is + wgt<double>(q % 9) * rref;
+            }
+        } else {
+            // box row of lattice row y: y - y0 + kGY; deviation tile row: y - y0 + 2
+            for (int c = tid; c < L::RX * L::RY; c += L::NT) {
+                const int cy = c / L::RX, cx = c - cy * L::RX;
+                const int yc = y0 - 2 + cy;
+                if (!per && (yc < 0 || yc >= g.ny)) continue;
+                const T2* c0 = box + (cy + 1) * L::BX + cx - 2 + L::GX;
+                C2 r, p;
+                cell_dev<P, PS>(c0 - L::BX, c0, c0 + L::BX, yc, per, a.pull, g, v, r, p, tab);
+                srho[cy * L::RX + cx] = r;
+                spsi[cy * L::RX + cx] = p;
+            }
+            if (!per) {
+                __syncthreads();
+                for (int c = tid; c < L::RX * L::RY; c += L::NT) {
+                    const int cy = c / L::RX, cx = c - cy * L::RX;
+                    const int yc = y0 - 2 + cy;
+                    int ym;
+                    if (yc < 0) ym = -1 - yc;
+                    else if (yc >= g.ny) ym = 2 * g.ny - 1 - yc;
+                    else continue;
+                    const int lm = ym - (y0 - 2);
+                    if (lm < 0 || lm >= L::RY) continue;
+                    srho[cy * L::RX + cx] = srho[lm * L::RX + cx];
+                    spsi[cy * L::RX + cx] = spsi[lm * L::RX + cx];
+                }
+            }
+            __syncthreads();
             C2 fx[1], fy[1], qx[1], qy[1], dp[1], dr[1];
-            force_sums<1, L::RX>(spsi + ly * L::RX + lx + 2, srho + ly * L::RX + lx + 2, a.k, fx, fy,
-                                 qx, qy, dp, dr);
-            SiteOut<T2> o;
-            o.stage = nullptr;
-            o.rbits = 0u;
-            o.valid = 1;
-            o.obs = a.obs;
-            o.obs_out = a.obs_out;
-            o.q0 = a.q0;
-            o.q1 = a.q1;
-            site_update<P, true, GEN, PS, SINK_STAGE>(b0 - L::BX, b0, b0 + L::BX, fx[0], fy[0], qx[0],
-                                                      qy[0], dp[0], dr[0], x, y, per, a.pull, g, v,
-                                                      a.k, o, red, bad);
+            if constexpr (P == LB_FP64)   // a warp is a row (RX = 32)
+                force_sums_warp<L::RX>(spsi + ly * L::RX + lx, srho + ly * L::RX + lx, a.k, fx[0], fy[0], qx[0],
+                                       qy[0], dp[0], dr[0]);
+            if (site) {
+                if constexpr (P != LB_FP64)
+                    force_sums<1, L::RX>(spsi + ly * L::RX + lx + 2, srho + ly * L::RX + lx + 2, a.k, fx, fy,
+                                         qx, qy, dp, dr);
+                load_site<P, PS>(b0 - L::BX, b0, b0 + L::BX, y, per, a.pull, g, v, h);
+                C2 jx, jy, Fx, Fy;
+                moments<P>(h, jx, jy);
+                const C2 rho = padd(pset(v.rho_ref), dr[0]);
+                if (!(isfinite(rho.x) && isfinite(rho.y))) bad = true;
+                site_force<GEN>(fx[0], fy[0], qx[0], qy[0], dp[0], rho, y, v, a.k, Fx, Fy);
+                const double rref = (double)v.rho_ref;
+                const double rA = rref + widen(dr[0].x), rB = rref + widen(dr[0].y);
+                const double mx = widen(jx.x) + widen(jx.y) + 0.5 * (widen(Fx.x) + widen(Fx.y));
+                const double my = widen(jy.x) + widen(jy.y) + 0.5 * (widen(Fy.x) + widen(Fy.y));
+                if (a.obs == OBS_FIELDS) {
+                    const double tot = rA + rB;
+                    const unsigned e = ((unsigned)__double2hiint(tot) >> 20) & 0x7ffu;
+                    double ux, uy;
+                    if (e - 64u < 1920u) {   // well inside the normal range
+                        const double r = recip(tot);
+                        ux = mx * r;
+                        uy = my * r;
+                    } else {
+                        ux = tot != 0.0 ? mx / tot : 0.0;
+                        uy = tot != 0.0 ? my / tot : 0.0;
+                    }
+                    a.obs_out[idx] = rA;
+                    a.obs_out[N + idx] = rB;
+                    a.obs_out[2 * N + idx] = ux;
+                    a.obs_out[3 * N + idx] = uy;
+                }
+                red[0] += rA;
+                red[1] += rB;
+                red[2] += mx;
+                red[3] += my;
+            }
         }
-    } else if (tid == 0) {
+        __syncthreads();   // the box and the window have been read
+    }
+    if (s_fail && tid == 0) {
         atomicOr(&a.st->err, ERR_TIMEOUT);
-        mbar_wait_bounded(&bar, 0);
+        mbar_wait_bounded(&bar, phase);
     }
     if (bad) atomicOr(&a.st->err, ERR_NONFINITE);
-    block_sum4<L::NT>(red, s_red);
-    const int bid = blockIdx.y * gridDim.x + blockIdx.x;
+    if constexpr (POPS) return;
+    const double part = block_sum4<L::NT>(red, s_red);
+    if (tid < 32 && (tid & 7) == 0) a.slots[4 * blockIdx.x + (tid >> 3)] = part;
+    __syncthreads();
     if (tid == 0) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) a.slots[4 * bid + q] = red[q];
         __threadfence();
-        s_last = atomicAdd(&a.st->ticket, 1u) == gridDim.x * gridDim.y - 1;
+        s_last = atomicAdd(&a.st->ticket, 1u) == gridDim.x - 1;
     }
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    const int nb = gridDim.x * gridDim.y;
     const volatile double* vs = a.slots;
-    double w[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int b = tid; b < nb; b += L::NT)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) w[q] += vs[4 * b + q];
+    for (int q = 0; q < 4; ++q) red[q] = 0.0;
+    for (int b = tid; b < (int)gridDim.x; b += L::NT)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) red[q] = w[q];
-    block_sum4<L::NT>(red, s_red);
+        for (int q = 0; q < 4; ++q) red[q] += vs[4 * b + q];
+    const double total = block_sum4<L::NT>(red, s_red);
+    if (tid < 32 && (tid & 7) == 0) a.st->totals[tid >> 3] = total;
     // the wall momentum totals: the strips' running totals, in a fixed order
     // (lane l adds strips l, l + 32, ..., then the butterfly)
     if (tid < 32 && !a.g.periodic) {
@@ -1803,8 +1834,6 @@ __global__ void __launch_bounds__(Layout<P>::NT)
         }
     }
     if (tid == 0) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) a.st->totals[q] = red[q];
         a.st->ticket = 0u;
         __threadfence();
     }
@@ -1812,7 +1841,8 @@ __global__ void __launch_bounds__(Layout<P>::NT)
 
 // ------------------------------------------------------------ init kernels
 // f(r, 0) = f^eq(rho_s, u) in place (the first step reads it unshifted).
-// mode 0: rho_s from the counter generator; mode 1: FP64 fields [4][ny][nx].
+// mode 0: rho_s from the counter generator; mode 1 (+ 2, + 4): FP64 fields
+// [4][ny][nx], with (+ 2) u_x and (+ 4) u_y, else zero.
 template <int P>
 __global__ void k_init(Geom g, Coef<typename Prec<P>::C> k, typename Prec<P>::T2* fout, int mode,
                        const double* fields, double rho0, double amp, double u_wall, int init_shear,
@@ -1827,7 +1857,10 @@ __global__ void k_init(Geom g, Coef<typename Prec<P>::C> k, typename Prec<P>::T2
             for (int s = 0; s < 2; ++s) {
                 const uint64_t ctr = ((uint64_t)s * g.ny + y) * g.nx + x;
                 const uint64_t z = mix64(seed ^ mix64(ctr + 0x9E3779B97F4A7C15ULL));
-                const double u = (double)(z >> 11) * (1.0 / 9007199254740992.0);
+                // x = z >> 11 as a double: its low 52 bits as the fraction of
+                // 2^52 + (x mod 2^52), less 2^52 unless bit 52 is set (exact)
+                const double f = __hiloint2double((int)((unsigned)(z >> 43) & 0xfffffu | 0x43300000u), (int)(z >> 11));
+                const double u = ((long long)z < 0 ? f : f - 4503599627370496.0) * (1.0 / 9007199254740992.0);
                 r[s] = rho0 * (1.0 + amp * (2.0 * u - 1.0));
             }
             ux = init_shear ? u_wall * (2.0 * y + 1.0 - g.ny) / (double)g.ny : 0.0;
@@ -1835,11 +1868,22 @@ __global__ void k_init(Geom g, Coef<typename Prec<P>::C> k, typename Prec<P>::T2
         } else {
             r[0] = fields[idx];
             r[1] = fields[N + idx];
-            ux = fields[2 * N + idx];
-            uy = fields[3 * N + idx];
+            ux = mode & 2 ? fields[2 * N + idx] : 0.0;
+            uy = mode & 4 ? fields[3 * N + idx] : 0.0;
         }
         const double usq = ux * ux + uy * uy;
         const double rref = (double)k.rho_ref;
+        if (ux == 0.0 && uy == 0.0) {
+            // at rest: sc w_i (rho - rho_ref), three values per species (the
+            // terms below, which are exact zeros, bound this kernel by their
+            // FP64 operations)
+            const double sc = (double)scale_of<P>();
+            const double dA = r[0] - rref, dB = r[1] - rref;
+#pragma unroll
+            for (int i = 0; i < 9; ++i)
+                put2<T2>(fout, g, i, x, y, encd2<T2>(sc * wgt<double>(i) * dA, sc * wgt<double>(i) * dB));
+            continue;
+        }
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
             const double cu = cx(i) * ux + cy(i) * uy;
@@ -1953,8 +1997,10 @@ static cudaError_t configure_all() {
     opt_moments(std::integral_constant<int, SHAPE_M8>{});
     opt_moments(std::integral_constant<int, SHAPE_M8X2>{});
 #endif
-    opt(k_observe<P, 2>, L::SMEM_OBS);
-    opt(k_observe<P, 3>, L::SMEM_OBS);
+    opt(k_observe<P, 2, false>, L::SMEM_OBS);
+    opt(k_observe<P, 3, false>, L::SMEM_OBS);
+    opt(k_observe<P, 2, true>, L::SMEM_OBS);
+    opt(k_observe<P, 3, true>, L::SMEM_OBS);
     return e;
 }
 
@@ -2071,10 +2117,17 @@ cudaError_t launch_observe_prec(const CUtensorMap* tin, const void* args, dim3 g
     cudaError_t e = ensure_configured<P>();
     if (e != cudaSuccess) return e;
     const StepArgs<C>& a = *reinterpret_cast<const StepArgs<C>*>(args);
-    if (a.g.periodic)
-        k_observe<P, 3><<<grid, L::NT, L::SMEM_OBS, s>>>(*tin, a);
-    else
-        k_observe<P, 2><<<grid, L::NT, L::SMEM_OBS, s>>>(*tin, a);
+    if (a.obs == OBS_POPS) {
+        if (a.g.periodic)
+            k_observe<P, 3, true><<<grid, L::NT, L::SMEM_OBS, s>>>(*tin, a);
+        else
+            k_observe<P, 2, true><<<grid, L::NT, L::SMEM_OBS, s>>>(*tin, a);
+    } else {
+        if (a.g.periodic)
+            k_observe<P, 3, false><<<grid, L::NT, L::SMEM_OBS, s>>>(*tin, a);
+        else
+            k_observe<P, 2, false><<<grid, L::NT, L::SMEM_OBS, s>>>(*tin, a);
+    }
     return cudaGetLastError();
 }
 

@@ -25,7 +25,7 @@ template <int P>
 static int staged_of(int shape) {
     if constexpr (has_shape(P, SHAPE_16))
         if (shape == SHAPE_16) return Layout<P, SHAPE_16>::STAGED ? 1 : 0;
-    return 1;
+    return Layout<P>::STAGED ? 1 : 0;
 }
 int kernel_staged(int p, int shape) { LB_SWITCH(p, return staged_of<P>(shape)) return 1; }
 

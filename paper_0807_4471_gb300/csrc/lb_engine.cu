@@ -378,14 +378,16 @@ struct Item {
 // seg < 0: the tiles of all lattices in strip order (lattice, strip, tile
 // row) cut into G contiguous runs of equal estimated cost, each run cut
 // again at strip boundaries: every CTA walks one or two strips.
+// rows > 0 (FP64 launches): the units cut and dealt are groups of `rows` rows in
+// place of tiles, all of the same cost.
 void partition(Lattice* const* lats, int nlat, int seg, int shape, int sms, std::vector<Item>& items,
-               std::vector<int>& cta, int* grid) {
+               std::vector<int>& cta, int* grid, int rows = 0) {
     items.clear();
     cta.clear();
     std::vector<int> nty((size_t)nlat);
     long long tiles = 0;
     for (int l = 0; l < nlat; ++l) {
-        nty[(size_t)l] = tiles_y(*lats[l], shape);
+        nty[(size_t)l] = rows ? (lats[l]->p.ny + rows - 1) / rows : tiles_y(*lats[l], shape);
         tiles += (long long)lats[l]->nstrips * nty[(size_t)l];
     }
     // Tile costs relative to a full interior tile, fitted on GB300 to the
@@ -397,6 +399,7 @@ void partition(Lattice* const* lats, int nlat, int seg, int shape, int sms, std:
     // item's start (its block ring fills, it computes four more deviation
     // rows) 0.8 of a tile.
     auto cost = [&](int l, int sx, int ty) {
+        if (rows) return 1.0;
         const Lattice& L = *lats[l];
         const int tx = kernel_tile_x(L.p.precision), tyy = shape_rows(shape);
         const int x0 = sx * tx, y0 = ty * tyy;
@@ -410,7 +413,9 @@ void partition(Lattice* const* lats, int nlat, int seg, int shape, int sms, std:
         if (per && (y0 < 3 || y0 + tyy > L.p.ny - 3)) c += kernel_staged(L.p.precision, shape) ? 0.25 : 0.02;
         return c;
     };
-    const double kItemStart = 0.8;
+    // An FP64 item start is four more window rows at a quarter of a row's work
+    // each, and the wait for its first blocks.
+    const double kItemStart = rows ? 1.6 / rows : 0.8;
     if (seg > 0) {
         // Segments in band order (all strips of a segment row, row after row),
         // each given to the CTA with the least work so far (the lowest index
@@ -608,7 +613,21 @@ lb_status launch_build(Launch& Ln, Lattice* const* lats, int nlat, void* descs, 
     std::vector<Item> items;
     std::vector<int> cta;
     int grid = 0;
-    partition(lats, nlat, seg, shape, ctas, items, cta, &grid);
+    if (prec == LB_FP64) {
+        // Rows, in groups of 1, 2, 4 or 8, so that a CTA gets 16 to 32 of them;
+        // a requested segment is in tiles.
+        long long all = 0;
+        for (int l = 0; l < nlat; ++l) all += (long long)lats[l]->nstrips * lats[l]->p.ny;
+        int rows = seg > 0 ? shape_rows(shape) : 1;
+        while (rows < shape_rows(shape) && all > 32LL * ctas * rows) rows *= 2;
+        partition(lats, nlat, seg, shape, ctas, items, cta, &grid, rows);
+        for (Item& it : items) {
+            it.ty_a *= rows;
+            it.ty_b = std::min(it.ty_b * rows, lats[it.lat]->p.ny);
+        }
+    } else {
+        partition(lats, nlat, seg, shape, ctas, items, cta, &grid);
+    }
     const int nitems = (int)items.size();
     const size_t dsz = prec == LB_FP64 ? sizeof(LatDesc<double>) : sizeof(LatDesc<float>);
     char* hs = reinterpret_cast<char*>(host_scratch);
@@ -616,7 +635,7 @@ lb_status launch_build(Launch& Ln, Lattice* const* lats, int nlat, void* descs, 
         lats[l]->seg = seg;
         if (prec == LB_FP64)
             fill_desc(*reinterpret_cast<LatDesc<double>*>(hs + l * dsz), *lats[l], lats[l]->kd,
-                      nt[(size_t)l]);
+                      lats[l]->p.ny);   // (items in rows)
         else
             fill_desc(*reinterpret_cast<LatDesc<float>*>(hs + l * dsz), *lats[l], lats[l]->kf,
                       nt[(size_t)l]);

@@ -139,7 +139,7 @@ struct alignas(128) LatDesc {
     double* wsum;          // [2][nstrips]: those summed per strip (bottom, then top) and
                            // over the sampled steps
     int nstrips;           // ceil(nx / TX)
-    int ntiles_y;          // tile rows of the launch's tile shape
+    int ntiles_y;          // tile rows of the launch's tile shape (FP64: ny)
     int stress_every;
 };
 
@@ -150,8 +150,8 @@ struct BatchArgs {
     const LatDesc<C>* lat;      // nlat descriptors
     int nlat;
     int nitems;                 // total work items
-    // Work items (lattice, strip, first tile row, end tile row), grouped by
-    // CTA: CTA b takes items cta_items[b] .. cta_items[b + 1] - 1 in order.
+    // Work items (lattice, strip, first tile row, end tile row; FP64: first row,
+    // end row), grouped by CTA: CTA b takes items cta_items[b] .. cta_items[b + 1] - 1 in order.
     const int4* items;
     const int* cta_items;
     unsigned int* ticket;       // CTA arrival counter of the launch (zero between launches)

@@ -884,6 +884,12 @@ __global__ void __launch_bounds__(Layout<P, SH>::NT, Layout<P, SH>::CTAS)
     k_step(const __grid_constant__ BatchArgs<typename Prec<P>::C> a) {
     typedef Layout<P, SH> L;
     constexpr int SPT = L::SPT, ADV = L::ADV, NBT = L::NBT;
+    // FP64: items are runs of rows (y_a, y_b) in place of runs of tiles, cut
+    // into tiles of 8 rows from their own first row on, the last one partial.
+    // Its time is the number of rows a CTA sums (the FP64 pipe), so a lattice
+    // is spread over the SMs row by row (128^2: 80 CTAs of one 8-row tile, 20.5 us
+    // a step; 128 CTAs of 5 rows, 16.4.  512^2: 142 -> 128 us).
+    constexpr bool ROWS = P == LB_FP64;
     typedef typename L::T2 T2;
     typedef typename L::C C;
     typedef typename L::C2 C2;
@@ -973,14 +979,14 @@ __global__ void __launch_bounds__(Layout<P, SH>::NT, Layout<P, SH>::CTAS)
     int p_item = a.cta_items[blockIdx.x], p_j = 0, p_pos = 0;
     // cached geometry of the producer's current item
     const CUtensorMap* p_map = nullptr;
-    int p_x0 = 0, p_ty_a = 0, p_nblk = 0;
+    int p_x0 = 0, p_y = 0, p_nblk = 0;
     auto p_load = [&]() {
         if (p_item >= it_end) return;
         const int4 w = a.items[p_item];
         const LatDesc<C>* d = &a.lat[w.x];
         p_x0 = w.y * L::TX;
-        p_ty_a = w.z;
-        p_nblk = ADV * (w.w - w.z) + 1;
+        p_y = ROWS ? w.z : L::TY * w.z;   // padded row of the first block
+        p_nblk = ADV * (ROWS ? (w.w - w.z + L::TY - 1) / L::TY : w.w - w.z) + 1;
         p_map = &d->tin[*((volatile int*)&d->st->cur) ^ (step_k & 1)];
         tma_prefetch_map(p_map);
     };
@@ -989,7 +995,7 @@ __global__ void __launch_bounds__(Layout<P, SH>::NT, Layout<P, SH>::CTAS)
         uint64_t* bar = &bars[p_pos % L::NB];
         mbar_expect_tx(bar, (uint32_t)L::SLOT_BYTES);
         // box origin: pair column x0 (= x0 - gx + gx) -> element 2 x0; padded row 8j
-        tma_load_3d_hint(slot(p_pos), p_map, 2 * p_x0, L::TYB * (ADV * p_ty_a + p_j), 0, bar,
+        tma_load_3d_hint(slot(p_pos), p_map, 2 * p_x0, p_y + L::TYB * p_j, 0, bar,
                          s_pol[0]);
         ++p_pos;
         if (++p_j == p_nblk) {
@@ -1019,8 +1025,9 @@ __global__ void __launch_bounds__(Layout<P, SH>::NT, Layout<P, SH>::CTAS)
         const int4 w = a.items[it];
         const LatDesc<C>* d = &a.lat[w.x];
         const int x0 = w.y * L::TX;
-        const int ty_a = w.z;
-        ty_b = w.w;
+        const int ty_a = ROWS ? 0 : w.z;
+        ty_b = ROWS ? (w.w - w.z + L::TY - 1) / L::TY : w.w;
+        const int y_first = ROWS ? w.z : 0;   // lattice row of tile 0
         const Geom g = d->g;
         const LatVals<C> v = d->v;
         const bool per_lat = ALLPER || g.periodic;
@@ -1051,7 +1058,8 @@ __global__ void __launch_bounds__(Layout<P, SH>::NT, Layout<P, SH>::CTAS)
                 sl[b] = sb;
                 if ((b > 0 || ty == ty_a) && !mbar_wait_bounded(&bars[sb], ph)) s_fail = 1;
             }
-            const int y0 = ty * L::TY;
+            const int y0 = y_first + ty * L::TY;
+            const int y_end = ROWS ? w.w : g.ny;   // end of the rows this item updates
             // The tile's padded rows [y0, y0 + 8 (SPT + 1)) are blocks q ..
             // q + SPT; brow(r, c): padded row y0 + r, pair column c, plane 0.
             const T2* s0 = reinterpret_cast<const T2*>(smem + sl[0] * L::SLOT_BYTES);
@@ -1114,6 +1122,7 @@ __global__ void __launch_bounds__(Layout<P, SH>::NT, Layout<P, SH>::CTAS)
     #pragma unroll
                     for (int c = 0; c < SPT; ++c) {
                         const int k = 4 + SPT * t_m + c;
+                        if (ROWS && k >= y_end - y0 + 4) break;   // (a warp is a row)
                         C2 r, p;
                         cell_dev<P, PS, TAU1>(brow(k, bc), brow(k + 1, bc), brow(k + 2, bc), y0 - 2 + k,
                                               per, pull, g, v, r, p, s_tab, jn[c]);
@@ -1168,11 +1177,11 @@ __global__ void __launch_bounds__(Layout<P, SH>::NT, Layout<P, SH>::CTAS)
                     const int x = x0 + lx, y = y0 + ly;
                     C2 fx[SPT], fy[SPT], qx[SPT], qy[SPT], dp[SPT], dr[SPT];
                     if constexpr (P == LB_FP64) {   // a warp is a row (RX = 32)
-                        if (y < g.ny)
+                        if (y < y_end)
                             force_sums_warp<L::RX>(win_p + ly * L::RX + lx, win_r + ly * L::RX + lx, a.k,
                                                    fx[0], fy[0], qx[0], qy[0], dp[0], dr[0]);
                     }
-                    if (lx < L::TX && x < g.nx && y < g.ny) {
+                    if (lx < L::TX && x < g.nx && y < y_end) {
                         if constexpr (P != LB_FP64)
                             force_sums<SPT, L::RX>(win_p + ly * L::RX + lx + 2,
                                                    win_r + ly * L::RX + lx + 2, a.k, fx, fy, qx, qy, dp, dr);

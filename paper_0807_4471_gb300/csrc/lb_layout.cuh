@@ -290,7 +290,8 @@ struct Layout {
     static constexpr int WIN_BYTES = 2 * WIN * RX * (int)sizeof(C2);
     static constexpr int STAGE_OFF = WIN_OFF + WIN_BYTES;
     static constexpr int STAGE_FULL = 9 * TY * TX * (int)sizeof(T2);
-    static constexpr bool STAGED = STAGE_OFF + STAGE_FULL + 128 <= 227 * 1024 - 1024;
+    // (FP64 items end inside a tile: direct stores)
+    static constexpr bool STAGED = P != LB_FP64 && STAGE_OFF + STAGE_FULL + 128 <= 227 * 1024 - 1024;
     static constexpr int STAGE_BYTES = STAGED ? STAGE_FULL : 0;
     // FP64: the exponential table (pexpm1_scaled)
     static constexpr int TAB_OFF = STAGE_OFF + STAGE_BYTES;
@@ -306,7 +307,7 @@ struct Layout {
     static constexpr int BOX_STRIDE = (BOX_BYTES + 127) / 128 * 128;
     static constexpr int RHOPSI = (2 * RX * RY * (int)sizeof(C2) + 127) / 128 * 128;
     static constexpr int SMEM_OBS = BOX_STRIDE + RHOPSI + 128;
-    static_assert(SPT == 1 || STAGED || sizeof(T2) == 8, "direct stores: FP32 pairs only");
+    static_assert(STAGED || sizeof(T2) >= 8, "direct stores: FP32 and FP64 pairs only");
     static_assert(NB >= NBT + 1, "the ring holds a tile's blocks and at least one more");
     static_assert(RX % 32 == 0, "deviation rows are whole warps");
     static_assert((2 * TX * sizeof(T)) % 16 == 0 && (2 * (TX + GX) * sizeof(T)) % 16 == 0,

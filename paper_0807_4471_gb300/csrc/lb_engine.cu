@@ -533,9 +533,16 @@ void partition(Lattice* const* lats, int nlat, int seg, int shape, int sms, std:
 // `tiles` counts tiles of the shape, `ctas` the launch's CTAs.  The moment kernel
 // moves a third of the bytes and takes contiguous runs at every size (4096^2:
 // 304 us a step, the best dealt segments 310; 4 x 1024^2: 84 and 84).
+// Contiguous runs also for more tiles where every lattice's buffer takes at most
+// a third of L2 (`largest` bytes): neighbouring strips then find each other's
+// halo columns there (4 x 1024^2 FP16: 78 us a step, dealt segments 83; one
+// 2048^2, the same number of tiles: 101 and 78).
 static int default_seg(long long tiles, int shape, const int* ns, const int* nt, int nlat, int sms,
-                       int ctas) {
-    return shape_moments(shape) || tiles * shape_rows(shape) <= 8LL * 40 * sms ? -1 : choose_seg(ns, nt, nlat, ctas);
+                       int ctas, long long largest) {
+    return shape_moments(shape) || tiles * shape_rows(shape) <= 8LL * 40 * sms ||
+                   largest * 3 <= device_l2_bytes()
+               ? -1
+               : choose_seg(ns, nt, nlat, ctas);
 }
 
 // Host-only plan of a launch's work items (lb_plan_partition).
@@ -565,7 +572,8 @@ lb_status plan_partition(const lb_params* ps, int nlat, int seg, int tile_rows, 
         nt[(size_t)l] = tiles_y(L, shape);
         tiles += (long long)L.nstrips * nt[(size_t)l];
     }
-    const int s = seg != 0 ? seg : default_seg(tiles, shape, ns.data(), nt.data(), nlat, sms, sms);
+    const int s = seg != 0 ? seg : default_seg(tiles, shape, ns.data(), nt.data(), nlat, sms, sms,
+                                            1LL << 60);
     std::vector<Item> it;
     std::vector<int> c;
     int G = 0;
@@ -608,8 +616,10 @@ lb_status launch_build(Launch& Ln, Lattice* const* lats, int nlat, void* descs, 
         strips += lats[l]->nstrips;
     }
     const int ctas = sms * shape_ctas(shape);
+    long long largest = 0;
+    for (int l = 0; l < nlat; ++l) largest = std::max(largest, (long long)lats[l]->fbytes);
     const int seg = forced_seg != 0 ? forced_seg
-                                    : default_seg(tiles, shape, ns.data(), nt.data(), nlat, sms, ctas);
+                                    : default_seg(tiles, shape, ns.data(), nt.data(), nlat, sms, ctas, largest);
     std::vector<Item> items;
     std::vector<int> cta;
     int grid = 0;

@@ -1354,8 +1354,8 @@ __global__ void __launch_bounds__(MLayout<SH>::NT, MLayout<SH>::CTAS)
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
     float2* ring = reinterpret_cast<float2*>(smem);                  // [9][NR][BX]
-    float2* win_r = reinterpret_cast<float2*>(smem + L::WIN_OFF);    // [WIN][RX]
-    float2* win_p = win_r + L::WIN * RX;                             // [WIN][RX]
+    float2* const win_r0 = reinterpret_cast<float2*>(smem + L::WIN_OFF);   // [WROWS][RX]
+    float2* const win_p0 = win_r0 + L::WROWS * RX;                         // [WROWS][RX]
     constexpr int kCarry = 2 / SPT;
     __shared__ __align__(16) float2 s_jcarry[kCarry * RX * SPT * 2];
     __shared__ int s_last;
@@ -1483,6 +1483,7 @@ __global__ void __launch_bounds__(MLayout<SH>::NT, MLayout<SH>::CTAS)
         }
         Mom pf[SPT], pfe;   // the next tile's new rows (and outermost columns)
         int base = 0;       // ring slot of row y0 - 3
+        int wm = 0;         // the tile's window starts at row wm TY
         auto slot_of = [&](int r) { return base + r >= NR ? base + r - NR : base + r; };
         for (int ty = ty_a; ty < ty_b; ++ty) {
             const int y0 = ty * TY;
@@ -1504,6 +1505,8 @@ __global__ void __launch_bounds__(MLayout<SH>::NT, MLayout<SH>::CTAS)
                 for (int c = 0; c < SPT; ++c) pf[c] = load_mom(y0 + TY + 3 + SPT * t_j + c, xw);
                 if (tid < 2 * TY) pfe = load_mom(y0 + TY + 3 + (tid >> 1), xe);
             }
+            float2* const win_r = win_r0 + wm * (TY * RX);
+            float2* const win_p = win_p0 + wm * (TY * RX);
             __syncthreads();   // the ring's rows are there; the previous site phase is over
             auto tile_body = [&](auto wall_tag) {
                 constexpr bool W = decltype(wall_tag)::value;
@@ -1532,9 +1535,10 @@ __global__ void __launch_bounds__(MLayout<SH>::NT, MLayout<SH>::CTAS)
                                     jc[2 * c] = jt[0];
                                     jc[2 * c + 1] = jt[1];
                                 }
-                            } else {
-                                win_r[kk * RX + t_w] = win_r[k * RX + t_w];
-                                win_p[kk * RX + t_w] = win_p[k * RX + t_w];
+                            } else if (wm == 0) {   // from the previous tile's window
+                                constexpr int back = (L::WM - 1) * TY;
+                                win_r[kk * RX + t_w] = win_r[(back + k) * RX + t_w];
+                                win_p[kk * RX + t_w] = win_p[(back + k) * RX + t_w];
                             }
                         }
                     }
@@ -1617,6 +1621,7 @@ __global__ void __launch_bounds__(MLayout<SH>::NT, MLayout<SH>::CTAS)
             else
                 tile_body(std::true_type{});
             base = slot_of(TY);
+            wm = wm + 1 == L::WM ? 0 : wm + 1;
         }
         if (!(nf.x == 0.0f && nf.y == 0.0f)) atomicOr(&d->st->err, ERR_NONFINITE);
     }

@@ -335,10 +335,13 @@ struct MLayout {
     static constexpr int CTAS = shape_ctas(SH);
     static constexpr int TX = Prec<LB_FP32>::TX, TR = 8 / SPT, TY = 8, RX = TX + 4;
     static constexpr int NT = RX * TR;
-    static constexpr int WIN = TY + 4;
+    // the windows' rows: a tile uses TY + 4 of them, WM tiles of an item go down
+    // them before the last four rows are copied back to the top (5 x 512^2: 25.3
+    // us a step, with a copy per tile 26.0)
+    static constexpr int WIN = TY + 4, WM = 4, WROWS = WM * TY + 4;
     static constexpr int NR = TY + 6, BX = TX + 6, PS = NR * BX;   // ring rows, columns, plane stride
     static constexpr int WIN_OFF = (9 * PS * (int)sizeof(float2) + 127) / 128 * 128;
-    static constexpr int SMEM = WIN_OFF + 2 * WIN * RX * (int)sizeof(float2) + 128;
+    static constexpr int SMEM = WIN_OFF + 2 * WROWS * RX * (int)sizeof(float2) + 128;
     static_assert(CTAS * (SMEM + 4096) <= 228 * 1024, "resident CTAs");
 };
 

@@ -216,8 +216,8 @@ lb_status lb_destroy(lb_handle* h);
  * creation; members are placed in it first-fit and admission fails with
  * LB_ERR_NOMEM when a member's footprint does not fit.  Steps run on the
  * pool's stream (a private stream is created when `stream` is NULL); runs of
- * consecutive steps over an unchanged member set are captured once into a
- * CUDA graph and replayed.  The work partition (segment length of the
+ * 512 or more steps over an unchanged member set are captured once into a CUDA
+ * graph and replayed.  The work partition (segment length of the
  * column strips) is tuned by timing candidate partitions on the first steps
  * of each new member set (those steps are real steps) and cached; a member
  * set that runs fewer than 8 times the steps the timing takes (about 400 to

@@ -62,13 +62,12 @@ lb_status create_common(const lb_params* p, void* stream, void* ws, size_t bytes
     if (s == LB_OK) s = lattice_setup(h->lat, p, h->ws + H.lattice);
     if (s == LB_OK) {
         Lattice* one = &h->lat;
-        alignas(128) unsigned char scratch[sizeof(LatDesc<double>)];
         const int sms = device_sms(h->device);
         const int shape = shape_of_rows(p->precision, moments_ok(*one), p->tile_rows,
                                         (long long)one->nstrips * one->ntiles_y, sms);
         s = launch_build(h->launch, &one, 1, h->ws + H.desc,
                          reinterpret_cast<double*>(h->ws + H.slots),
-                         reinterpret_cast<unsigned int*>(h->ws + H.ticket), sms, h->stream, scratch,
+                         reinterpret_cast<unsigned int*>(h->ws + H.ticket), sms, h->stream, nullptr,
                          0, shape);
     }
     if (s != LB_OK) {

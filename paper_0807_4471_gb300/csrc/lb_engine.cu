@@ -593,8 +593,48 @@ lb_status plan_partition(const lb_params* ps, int nlat, int seg, int tile_rows, 
     return LB_OK;
 }
 
+HostStage::~HostStage() {
+    for (Buffer& b : buf_) {
+        if (b.done) {
+            if (b.busy) cudaEventSynchronize(b.done);
+            cudaEventDestroy(b.done);
+        }
+        if (b.mem) cudaFreeHost(b.mem);
+    }
+}
+
+char* HostStage::get(size_t bytes) {
+    last_ = (last_ + 1) % kBuffers;
+    Buffer& b = buf_[last_];
+    if (b.busy && cudaEventSynchronize(b.done) != cudaSuccess) return nullptr;
+    b.busy = false;
+    if (!b.done && cudaEventCreateWithFlags(&b.done, cudaEventDisableTiming) != cudaSuccess) {
+        b.done = nullptr;
+        return nullptr;
+    }
+    if (b.cap < bytes) {
+        if (b.mem) cudaFreeHost(b.mem);
+        b.mem = nullptr;
+        b.cap = 0;
+        const size_t cap = align_up(bytes + bytes / 2, 64 << 10);
+        if (cudaHostAlloc(reinterpret_cast<void**>(&b.mem), cap, cudaHostAllocDefault) != cudaSuccess) {
+            b.mem = nullptr;
+            return nullptr;
+        }
+        b.cap = cap;
+    }
+    return b.mem;
+}
+
+cudaError_t HostStage::sent(cudaStream_t s) {
+    Buffer& b = buf_[last_];
+    const cudaError_t e = cudaEventRecord(b.done, s);
+    b.busy = e == cudaSuccess;
+    return e;
+}
+
 lb_status launch_build(Launch& Ln, Lattice* const* lats, int nlat, void* descs, double* slots,
-                       unsigned int* ticket, int sms, cudaStream_t stream, void* host_scratch,
+                       unsigned int* ticket, int sms, cudaStream_t stream, HostStage* stage,
                        int forced_seg, int shape) {
     if (nlat < 1) return LB_ERR_INVALID;
     const int prec = lats[0]->p.precision;
@@ -640,7 +680,21 @@ lb_status launch_build(Launch& Ln, Lattice* const* lats, int nlat, void* descs, 
     }
     const int nitems = (int)items.size();
     const size_t dsz = prec == LB_FP64 ? sizeof(LatDesc<double>) : sizeof(LatDesc<float>);
-    char* hs = reinterpret_cast<char*>(host_scratch);
+    // descriptors | items | CTA offsets, as they go to the device
+    const size_t at_items = align_up(dsz * (size_t)nlat, 128);
+    const size_t at_cta = at_items + sizeof(Item) * (size_t)nitems;
+    const size_t bytes = at_cta + sizeof(int) * cta.size();
+    std::vector<char> own;
+    char* hs = nullptr;
+    if (stage) {
+        hs = stage->get(bytes);
+        if (!hs) return LB_ERR_CUDA;
+    } else {
+        own.resize(bytes + 128);
+        hs = own.data() + (128 - reinterpret_cast<uintptr_t>(own.data()) % 128) % 128;
+    }
+    memcpy(hs + at_items, items.data(), sizeof(Item) * (size_t)nitems);
+    memcpy(hs + at_cta, cta.data(), sizeof(int) * cta.size());
     for (int l = 0; l < nlat; ++l) {
         lats[l]->seg = seg;
         if (prec == LB_FP64)
@@ -656,10 +710,9 @@ lb_status launch_build(Launch& Ln, Lattice* const* lats, int nlat, void* descs, 
     static_assert(sizeof(Item) == sizeof(int4), "item layout");
     cudaError_t e = cudaMemcpyAsync(descs, hs, dsz * nlat, cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(d_items, items.data(), sizeof(int4) * (size_t)nitems, cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(d_cta, cta.data(), sizeof(int) * cta.size(), cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);   // host buffers are reused
+        // (the CTA offsets follow the items on both sides)
+        e = cudaMemcpyAsync(d_items, hs + at_items, bytes - at_items, cudaMemcpyHostToDevice, stream);
+    if (e == cudaSuccess) e = stage ? stage->sent(stream) : cudaStreamSynchronize(stream);
     if (e != cudaSuccess) return cuda_status(e);
     Ln.precision = prec;
     Ln.variant = (allper ? 1 : 0) | (gen ? 2 : 0) | (tau1 ? 4 : 0);

@@ -74,16 +74,39 @@ bool moments_ok(const Lattice& L);
 int default_shape(int precision, bool moments, long long tiles8, int sms);
 int shape_of_rows(int precision, bool moments, int rows, long long tiles8, int sms);
 
+// Pinned host buffers for tables on their way to the device: a few, used in
+// turn, so that a launch can be built while the device still works on the
+// steps before it.  A buffer is handed out again once its copies are done.
+class HostStage {
+public:
+    ~HostStage();
+    // `bytes` of pinned memory (128-byte aligned), or null
+    char* get(size_t bytes);
+    // the copies out of the last buffer handed out are enqueued on s
+    cudaError_t sent(cudaStream_t s);
+
+private:
+    static constexpr int kBuffers = 4;
+    struct Buffer {
+        char* mem = nullptr;
+        size_t cap = 0;
+        cudaEvent_t done = nullptr;
+        bool busy = false;
+    } buf_[kBuffers];
+    int last_ = 0;
+};
+
 // Write the lattices' descriptors to `descs` (device, 128-byte aligned, room
-// for nlat LatDesc<double>) through `host_scratch` (as large, host) and fill
-// the launch.  Synchronises the stream.  All lattices share the precision
+// for nlat LatDesc<double>) and the item tables to `slots`, and fill the
+// launch.  With a stage the copies are only enqueued; without one they go
+// through pageable memory and the stream is synchronised.  All lattices share the precision
 // and the coefficients of lats[0] (couplings, tau, forcing).  seg > 0 forces
 // the segment length; seg = 0 takes choose_seg's; seg < 0 cuts the tiles
 // into one contiguous run per CTA.  `slots` holds launch_area_doubles(tiles,
 // strips, sms) doubles for the lattices' total tiles and strips: the item
 // tables.
 lb_status launch_build(Launch& Ln, Lattice* const* lats, int nlat, void* descs, double* slots,
-                       unsigned int* ticket, int sms, cudaStream_t stream, void* host_scratch,
+                       unsigned int* ticket, int sms, cudaStream_t stream, HostStage* stage,
                        int seg = 0, int shape = SHAPE_8);
 size_t launch_area_doubles(size_t tiles, size_t strips, int sms);
 // Enqueue step step_k of a window of consecutive steps (0-based); advance: the

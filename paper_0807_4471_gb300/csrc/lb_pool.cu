@@ -23,6 +23,11 @@ namespace {
 
 constexpr size_t kAlign = 256;
 constexpr int kGraphChunk = 16;   // steps per captured graph
+// Steps of a run from which a graph is captured: a launch costs the host 2-3 us,
+// less than any step takes, while a member set's capture and instantiation
+// take 0.2 ms, during which the device has nothing to do (16 served jobs of
+// 64..200^2, quanta of 100 steps: 7.2 -> 6.5 ms with this and the staged tables).
+constexpr int kGraphLeast = 512;
 constexpr int kTuneSteps = 6;     // timed steps per candidate (tile shape, partition)
 // A new member set is tuned only if it runs at least kTuneShare times the
 // steps that timing all candidates takes: a short-lived set (a server's
@@ -103,7 +108,7 @@ struct lb_pool {
     unsigned int* ticket;
     double* slots;
     size_t slot_cap;         // doubles
-    void* host_desc;         // staging of the descriptors (128-byte aligned)
+    HostStage stage;         // descriptors and tables on their way to the device
     // current active set and its launch
     std::vector<int> active;
     bool built;
@@ -170,7 +175,7 @@ lb_status build(lb_pool* P, Choice c) {
     cudaError_t ce = kernels_configure(P->shared.precision);   // before any graph capture
     if (ce != cudaSuccess) return cuda_status(ce);
     lb_status s = launch_build(P->launch, lats.data(), nlat, P->desc_mem, P->slots, P->ticket,
-                               P->sms, P->stream, P->host_desc, c.seg, c.shape);
+                               P->sms, P->stream, &P->stage, c.seg, c.shape);
     P->built = s == LB_OK;
     return s;
 }
@@ -197,9 +202,11 @@ lb_status capture_graph(lb_pool* P) {
     return LB_OK;
 }
 
-// Run k steps of the built launch: captured chunks, then single launches.
+// Run k steps of the built launch: captured chunks (a long run, or a graph that
+// is there), then single launches.
 lb_status run_steps(lb_pool* P, long long k) {
-    while (k >= kGraphChunk) {
+    const bool graph = P->graph || k >= kGraphLeast;
+    while (graph && k >= kGraphChunk) {
         lb_status s = capture_graph(P);
         if (s != LB_OK) return s;
         cudaError_t e = cudaGraphLaunch(P->graph, P->stream);
@@ -366,7 +373,6 @@ lb_status lb_pool_create(const lb_params* shared, size_t bytes_budget, int32_t m
     P->slot_cap = 0;
     P->arena_mem = nullptr;
     P->desc_mem = nullptr;
-    P->host_desc = nullptr;
     cudaError_t e = cudaSuccess;
     if (!P->stream) {   // graphs need a capturable stream
         e = cudaStreamCreateWithFlags(&P->stream, cudaStreamNonBlocking);
@@ -378,10 +384,6 @@ lb_status lb_pool_create(const lb_params* shared, size_t bytes_budget, int32_t m
     if (e == cudaSuccess) {
         P->ticket = reinterpret_cast<unsigned int*>(P->desc_mem + dbytes);
         e = cudaMemsetAsync(P->ticket, 0, sizeof(unsigned int), P->stream);
-    }
-    if (e == cudaSuccess) {
-        P->host_desc = std::aligned_alloc(128, dbytes);
-        if (!P->host_desc) e = cudaErrorMemoryAllocation;
     }
     if (e != cudaSuccess) {
         lb_pool_destroy(P);
@@ -546,7 +548,6 @@ lb_status lb_pool_destroy(lb_pool* P) {
     if (P->slots) cudaFree(P->slots);
     if (P->desc_mem) cudaFree(P->desc_mem);
     if (P->arena_mem) cudaFree(P->arena_mem);
-    if (P->host_desc) std::free(P->host_desc);
     if (P->own_stream) cudaStreamDestroy(P->stream);
     delete P;
     return cuda_status(e);

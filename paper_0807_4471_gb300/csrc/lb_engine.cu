@@ -324,16 +324,20 @@ int tiles_y(const Lattice& L, int shape) {
 bool moments_ok(const Lattice& L) {
     return L.p.precision == LB_FP32 && L.kf.omm.x == 0.0f && L.kf.omm.y == 0.0f && !L.kf.source;
 }
-// Default tile shape of a lattice set with `tiles8` 8-row tiles.  The 16-bit
-// formats and the moment kernel: two CTAs per SM, except where the tiles do
-// not even fill one CTA per SM one and a half times over; a thread's single
-// site then finishes a tile sooner (256^2 FP16, 160 tiles: 6.3 us a step against
-// 6.9; 512^2, 576 tiles: 11.0 against 9.7).  Other FP32: the 16-row tile beyond
-// the same line (256^2: 6.5 us with 8 rows, 7.3 with 16; 512^2: 11.2 and 10.2).
+// Default tile shape of a lattice set with `tiles8` 8-row tiles.
+//  One tile per SM at most: the direct kernel, with the shortest chain (its
+//  figures are there; with two tiles on a CTA it loses: 256^2 FP16, 160 tiles,
+//  6.9 us a step against 6.3).
+//  Up to 1.5 tiles per SM: one site per thread, which finishes a tile sooner
+//  (256^2 FP16: 6.3 us with SHAPE_8, 6.9 with SHAPE_8X2; 512^2, 576 tiles: 11.0
+//  and 9.7.  FP32: 6.5 us with 8 rows, 7.3 with 16; 512^2: 11.2 and 10.2).
+//  Beyond: two sites per thread, two CTAs per SM where they fit.
 int default_shape(int precision, bool moments, long long tiles8, int sms) {
     const bool few = 2 * tiles8 <= 3LL * sms;
     if (moments) return few ? SHAPE_M8 : SHAPE_M8X2;
-    if (precision == LB_FP64 || few) return SHAPE_8;
+    if (precision == LB_FP64) return SHAPE_8;
+    if (tiles8 <= sms) return SHAPE_D8;
+    if (few) return SHAPE_8;
     return has_shape(precision, SHAPE_8X2) ? SHAPE_8X2 : SHAPE_16;
 }
 int shape_of_rows(int precision, bool moments, int rows, long long tiles8, int sms) {
@@ -341,7 +345,7 @@ int shape_of_rows(int precision, bool moments, int rows, long long tiles8, int s
     if (rows == 16) return has_shape(precision, SHAPE_16) ? SHAPE_16 : 0;
     if (rows != 8) return 0;
     const int d = default_shape(precision, false, tiles8, sms);
-    return d == SHAPE_8X2 ? d : SHAPE_8;
+    return d == SHAPE_16 ? SHAPE_8 : d;
 }
 
 template <typename C>
@@ -555,8 +559,8 @@ lb_status plan_partition(const lb_params* ps, int nlat, int seg, int tile_rows, 
     std::vector<int> ns((size_t)nlat), nt((size_t)nlat);
     if (validate_params(&ps[0]) != LB_OK) return LB_ERR_INVALID;
     if (tile_rows != 0 && tile_rows != 8 && tile_rows != 16) return LB_ERR_INVALID;
-    const int shape = tile_rows == 16 ? SHAPE_16 : SHAPE_8;
-    if (!has_shape(ps[0].precision, shape)) return LB_ERR_INVALID;
+    const int shape = tile_rows == 16 ? SHAPE_16 : SHAPE_8;   // (any 8-row shape: one CTA per SM)
+    if (shape == SHAPE_16 && !has_shape(ps[0].precision, shape)) return LB_ERR_INVALID;
     long long tiles = 0;
     for (int l = 0; l < nlat; ++l) {
         if (validate_params(&ps[l]) != LB_OK || ps[l].precision != ps[0].precision)

@@ -188,13 +188,17 @@ struct StepArgs {
 //  SHAPE_16   16-row tiles, two sites per thread, one CTA per SM;
 //  SHAPE_8X2  8-row tiles, two sites per thread, two CTAs of half the threads
 //             per SM (16-bit formats: their shared memory holds two);
-//  SHAPE_M8, SHAPE_M8X2  the same two 8-row forms of the moment kernel (FP32,
+//  SHAPE_D8   8-row tiles, one site per thread, the tile loaded by plain loads
+//             (FP32 and 16-bit populations, few tiles: see k_step_d);
+//  SHAPE_M8, SHAPE_M8X2  8-row tiles with one site per thread, and with
+//             two and two CTAs per SM, of the moment kernel (FP32,
 //             tau = 1, velocity shift: see k_step_m).
-enum Shape : int { SHAPE_8 = 1, SHAPE_16 = 2, SHAPE_8X2 = 3, SHAPE_M8 = 4, SHAPE_M8X2 = 5 };
+enum Shape : int { SHAPE_8 = 1, SHAPE_16 = 2, SHAPE_8X2 = 3, SHAPE_D8 = 4, SHAPE_M8 = 5, SHAPE_M8X2 = 6 };
 constexpr bool shape_moments(int shape) { return shape >= SHAPE_M8; }
 constexpr bool has_shape(int precision, int shape) {
     return shape == SHAPE_8 || (shape == SHAPE_16 && precision != LB_FP64) ||
            (shape == SHAPE_8X2 && (precision == LB_FP16_OFFSET || precision == LB_BF16_OFFSET)) ||
+           (shape == SHAPE_D8 && precision != LB_FP64) ||
            (shape_moments(shape) && precision == LB_FP32);
 }
 constexpr int shape_rows(int shape) { return shape == SHAPE_16 ? 16 : 8; }

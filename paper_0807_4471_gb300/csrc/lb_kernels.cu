@@ -1315,6 +1315,176 @@ __global__ void __launch_bounds__(Layout<P, SH>::NT, Layout<P, SH>::CTAS)
     if (tid == 0) *a.ticket = 0u;
 }
 
+// ------------------------------------- direct kernel (few tiles, not FP64)
+// The step for lattices whose tiles do not fill the SMs: a step then is one
+// chain of latencies, and k_step's ring, descriptors, staging tile and bulk
+// stores only lengthen it.  A CTA loads a tile's populations by plain loads (all
+// of a thread's at once) into shared memory, takes the tile's whole deviation
+// window (no rows are carried), updates one site per thread and stores it from
+// registers.  One CTA per SM; the site arithmetic is k_step's.  Measured, k_step
+// -> this: 300 x 211 FP32 Couette with tau 0.8 (135 tiles) 8.3 -> 7.4 us a step,
+// 128^2 FP16 5.25 -> 4.67, 64^2 FP16 5.18 -> 4.61.
+#if LB_PREC != 0
+template <int P, int V>
+__global__ void __launch_bounds__(DLayout<P>::NT, 1)
+    k_step_d(const __grid_constant__ BatchArgs<float> a) {
+    typedef DLayout<P> L;
+    typedef typename L::T2 T2;
+    constexpr bool ALLPER = (V & 1) != 0;
+    constexpr bool GEN = (V & 2) != 0;
+    constexpr bool TAU1 = (V & 4) != 0;
+    constexpr int TY = L::TY, TX = L::TX, RX = L::RX, NR = L::NR, BX = L::BX, PS = L::PS;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
+    T2* const box = reinterpret_cast<T2*>(smem);                     // [9][NR][BX]
+    float2* const win_r = reinterpret_cast<float2*>(smem + L::WIN_OFF);   // [WIN][RX]
+    float2* const win_p = win_r + L::WIN * RX;                            // [WIN][RX]
+    __shared__ int s_last;
+    const int tid = threadIdx.x;
+    const int t_lx = tid % RX, t_j = tid / RX;
+    const int t_w = (t_lx + 2) % RX;   // window column, the site's own for t_lx < TX
+    const int it0 = a.cta_items[blockIdx.x], it_end = a.cta_items[blockIdx.x + 1];
+    const int step_k = a.step_k;
+    // tables and counters are read ahead of the wait, as in k_step
+    int4 w = make_int4(0, 0, 0, 0);
+    const LatDesc<float>* d = nullptr;
+    Geom g = {};
+    LatVals<float> v = {};
+    int cur = 0, pull = 1;
+    uint32_t key = 0;
+    auto load_item = [&](int it) {
+        w = a.items[it];
+        d = &a.lat[w.x];
+        g = d->g;
+        v = d->v;
+    };
+    auto load_state = [&]() {
+        cur = *((volatile int*)&d->st->cur) ^ (step_k & 1);
+        if (step_k == 0) pull = *((volatile int*)&d->st->pull);
+        key = hash32(((uint32_t)*((volatile long long*)&d->st->t) + (uint32_t)step_k) * 0x9e3779b9u);
+    };
+    if (it0 < it_end) {
+        load_item(it0);
+        if (step_k != 0) load_state();
+    }
+    griddep_wait();
+    griddep_launch_dependents();
+    if (it0 < it_end && step_k == 0) load_state();
+    const uint64_t pol = a.l2_resident ? policy_evict_last() : policy_evict_normal();
+    for (int it = it0; it < it_end; ++it) {
+        if (it != it0) {
+            load_item(it);
+            load_state();
+        }
+        const int x0 = w.y * TX;
+        const bool per_lat = ALLPER || g.periodic;
+        const T2* const fin = reinterpret_cast<const T2*>(d->fbuf[cur]);
+        T2* const fout = reinterpret_cast<T2*>(d->fbuf[cur ^ 1]);
+        float2 nf = pset(0.0f);
+        for (int ty = w.z; ty < w.w; ++ty) {
+            const int y0 = ty * TY;
+            // box row r: lattice row y0 - 3 + r (the padded planes hold rows up to
+            // ny + 2 and columns up to nx + 2; beyond them no site reads)
+            auto cell = [&](int r, int c, T2 h[9]) {
+                const int y = min(y0 - 3 + r, g.ny + 2), x = min(x0 - 3 + c, g.nx + 2);
+                const T2* f = fin + (long long)(y + kGY) * g.pitch + (x + g.gx);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) h[i] = __ldcg(f + i * g.plane);
+            };
+            auto put = [&](int r, int c, const T2 h[9]) {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) box[i * PS + r * BX + c] = h[i];
+            };
+            {
+                T2 h0[9], h1[9], he[9];
+                cell(t_j, t_w + 1, h0);
+                if (t_j + 8 < NR) cell(t_j + 8, t_w + 1, h1);
+                const int r = tid >> 1, c = tid & 1 ? BX - 1 : 0;   // outermost columns
+                if (tid < 2 * NR) cell(r, c, he);
+                put(t_j, t_w + 1, h0);
+                if (t_j + 8 < NR) put(t_j + 8, t_w + 1, h1);
+                if (tid < 2 * NR) put(r, c, he);
+            }
+            __syncthreads();
+            auto tile_body = [&](auto wall_tag) {
+                constexpr bool W = decltype(wall_tag)::value;
+                const bool per = !W || per_lat;
+                // Density phase: window row k holds lattice row y0 - 2 + k, box row
+                // k + 1; the thread's own site row k = t_j + 2, and the rows 0, 1,
+                // 10, 11 by the first four thread rows.
+                float2 jn[2];
+                const T2* bc = box + t_w + 1;
+                auto window = [&](int k, float2* j) {
+                    float2 r, q;
+                    cell_dev<P, PS, TAU1>(bc + k * BX, bc + (k + 1) * BX, bc + (k + 2) * BX, y0 - 2 + k, per,
+                                          pull, g, v, r, q, nullptr, j);
+                    win_r[k * RX + t_w] = r;
+                    win_p[k * RX + t_w] = q;
+                };
+                window(t_j + 2, jn);
+                if (t_j < 4) {
+                    float2 unused[2];
+                    window(t_j < 2 ? t_j : t_j + 8, unused);
+                }
+                if (!per && (y0 < 2 || y0 + TY + 1 >= g.ny)) {   // mirror about the halfway walls
+                    __syncthreads();
+                    for (int c = tid; c < L::WIN * RX; c += L::NT) {
+                        const int k = c / RX, lx = c - k * RX;
+                        const int y = y0 - 2 + k;
+                        int ym;
+                        if (y < 0) ym = -1 - y;
+                        else if (y >= g.ny && y <= g.ny + 1) ym = 2 * g.ny - 1 - y;
+                        else continue;
+                        const int km = ym - (y0 - 2);
+                        win_r[k * RX + lx] = win_r[km * RX + lx];
+                        win_p[k * RX + lx] = win_p[km * RX + lx];
+                    }
+                }
+                __syncthreads();
+                const int x = x0 + t_lx, y = y0 + t_j;
+                if (t_lx < TX && x < g.nx && y < g.ny) {
+                    float2 fx[1], fy[1], qx[1], qy[1], dp[1], dr[1];
+                    force_sums<1, RX>(win_p + t_j * RX + t_lx + 2, win_r + t_j * RX + t_lx + 2, a.k, fx, fy, qx,
+                                      qy, dp, dr);
+                    SiteOut<T2> o;
+                    o.valid = 1;
+                    o.wallx = d->wallx;
+                    o.plane = g.plane;
+                    o.pol = pol;
+                    o.gout = fout + (long long)(y + kGY) * g.pitch + (x + g.gx);
+                    o.gdx = x < 3 ? g.nx : (x >= g.nx - 3 ? -g.nx : 0);
+                    o.gdy = !per_lat ? 0
+                            : y < 3 ? (long long)g.ny * g.pitch
+                            : (y >= g.ny - 3 ? -(long long)g.ny * g.pitch : 0);
+                    o.rbits = 0u;
+                    if constexpr (sizeof(T2) == 4) o.rbits = sr_word(sr_hash(key, x, y, g.nx), y);
+                    const T2* b0 = bc + (t_j + 3) * BX;   // (t_w is the site's column here)
+                    site_update<P, GEN, PS, SINK_GLOBAL, TAU1>(b0 - BX, b0, b0 + BX, fx[0], fy[0], qx[0], qy[0],
+                                                               dp[0], dr[0], x, y, per, pull, g, v, a.k, o, &nf,
+                                                               jn);
+                }
+            };
+            if constexpr (ALLPER)
+                tile_body(std::false_type{});
+            else if (per_lat || (y0 >= 3 && y0 + TY + 3 <= g.ny))
+                tile_body(std::false_type{});
+            else
+                tile_body(std::true_type{});
+            __syncthreads();   // the box and the windows have been read
+        }
+        if (!(nf.x == 0.0f && nf.y == 0.0f)) atomicOr(&d->st->err, ERR_NONFINITE);
+    }
+    if constexpr (!ALLPER) wall_sums<P, L>(a, it0, it_end, tid);   // (behind the tiles' last barrier)
+    if (!a.advance) return;
+    __syncthreads();
+    if (tid == 0) s_last = ticket_arrive(a.ticket) == (unsigned int)(gridDim.x - 1);
+    __syncthreads();
+    if (!s_last) return;
+    advance_lattices<L::NT>(a, tid, 1);
+    if (tid == 0) *a.ticket = 0u;
+}
+#endif
+
 // ------------------------------------------------- moment kernel (FP32)
 // The step of FP32 lattices with tau = 1 for both species and the velocity
 // shift.  There the post-collision populations are the equilibrium of six
@@ -2030,6 +2200,17 @@ static cudaError_t configure_all() {
     opt_shape(std::integral_constant<int, SHAPE_8>{});
     opt_shape(std::integral_constant<int, SHAPE_16>{});
     opt_shape(std::integral_constant<int, SHAPE_8X2>{});
+#if LB_PREC != 0
+    constexpr int dbytes = DLayout<P>::SMEM;
+    opt(k_step_d<P, 0>, dbytes);
+    opt(k_step_d<P, 1>, dbytes);
+    opt(k_step_d<P, 2>, dbytes);
+    opt(k_step_d<P, 3>, dbytes);
+    opt(k_step_d<P, 4>, dbytes);
+    opt(k_step_d<P, 5>, dbytes);
+    opt(k_step_d<P, 6>, dbytes);
+    opt(k_step_d<P, 7>, dbytes);
+#endif
 #if LB_PREC == 1
     auto opt_moments = [&](auto tag) {
         constexpr int SH = decltype(tag)::value;
@@ -2072,59 +2253,68 @@ static bool pdl_enabled() {
     return on;
 }
 
-template <int P, int SH>
-static cudaError_t launch_step_shape(const BatchArgs<typename Prec<P>::C>& a, int variant, dim3 grid,
-                                     cudaStream_t s) {
-    typedef Layout<P, SH> L;
-    // Consecutive steps on a stream overlap the next launch's set-up with the
-    // previous launch's last CTAs (programmatic stream serialization); the
-    // kernel waits for the previous grid before it reads the lattice state.
+// Consecutive steps on a stream overlap the next launch's set-up with the
+// previous launch's last CTAs (programmatic stream serialization); the kernels
+// wait for the previous grid before they read the lattice state.
+template <typename K, typename A>
+static cudaError_t launch_pdl(K kernel, const A& a, int threads, int smem, dim3 grid, cudaStream_t s) {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
-    cfg.blockDim = dim3(L::NT, 1, 1);
-    cfg.dynamicSmemBytes = L::SMEM;
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.dynamicSmemBytes = (size_t)smem;
     cfg.stream = s;
     cfg.attrs = at;
     cfg.numAttrs = pdl_enabled() ? 1 : 0;
-    cudaError_t e;
-    switch (variant & 7) {
-        case 0: e = cudaLaunchKernelEx(&cfg, k_step<P, 0, SH>, a); break;
-        case 1: e = cudaLaunchKernelEx(&cfg, k_step<P, 1, SH>, a); break;
-        case 2: e = cudaLaunchKernelEx(&cfg, k_step<P, 2, SH>, a); break;
-        case 3: e = cudaLaunchKernelEx(&cfg, k_step<P, 3, SH>, a); break;
-        case 4: e = cudaLaunchKernelEx(&cfg, k_step<P, 4, SH>, a); break;
-        case 5: e = cudaLaunchKernelEx(&cfg, k_step<P, 5, SH>, a); break;
-        case 6: e = cudaLaunchKernelEx(&cfg, k_step<P, 6, SH>, a); break;
-        default: e = cudaLaunchKernelEx(&cfg, k_step<P, 7, SH>, a); break;
-    }
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, a);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
+
+template <int P, int SH>
+static cudaError_t launch_step_shape(const BatchArgs<typename Prec<P>::C>& a, int variant, dim3 grid,
+                                     cudaStream_t s) {
+    typedef Layout<P, SH> L;
+    switch (variant & 7) {
+        case 0: return launch_pdl(k_step<P, 0, SH>, a, L::NT, L::SMEM, grid, s);
+        case 1: return launch_pdl(k_step<P, 1, SH>, a, L::NT, L::SMEM, grid, s);
+        case 2: return launch_pdl(k_step<P, 2, SH>, a, L::NT, L::SMEM, grid, s);
+        case 3: return launch_pdl(k_step<P, 3, SH>, a, L::NT, L::SMEM, grid, s);
+        case 4: return launch_pdl(k_step<P, 4, SH>, a, L::NT, L::SMEM, grid, s);
+        case 5: return launch_pdl(k_step<P, 5, SH>, a, L::NT, L::SMEM, grid, s);
+        case 6: return launch_pdl(k_step<P, 6, SH>, a, L::NT, L::SMEM, grid, s);
+        default: return launch_pdl(k_step<P, 7, SH>, a, L::NT, L::SMEM, grid, s);
+    }
+}
+
+#if LB_PREC != 0
+template <int P>
+static cudaError_t launch_direct(const BatchArgs<float>& a, int variant, dim3 grid, cudaStream_t s) {
+    typedef DLayout<P> L;
+    switch (variant & 7) {
+        case 0: return launch_pdl(k_step_d<P, 0>, a, L::NT, L::SMEM, grid, s);
+        case 1: return launch_pdl(k_step_d<P, 1>, a, L::NT, L::SMEM, grid, s);
+        case 2: return launch_pdl(k_step_d<P, 2>, a, L::NT, L::SMEM, grid, s);
+        case 3: return launch_pdl(k_step_d<P, 3>, a, L::NT, L::SMEM, grid, s);
+        case 4: return launch_pdl(k_step_d<P, 4>, a, L::NT, L::SMEM, grid, s);
+        case 5: return launch_pdl(k_step_d<P, 5>, a, L::NT, L::SMEM, grid, s);
+        case 6: return launch_pdl(k_step_d<P, 6>, a, L::NT, L::SMEM, grid, s);
+        default: return launch_pdl(k_step_d<P, 7>, a, L::NT, L::SMEM, grid, s);
+    }
+}
+#endif
 
 #if LB_PREC == 1
 template <int SH>
 static cudaError_t launch_moments_shape(const BatchArgs<float>& a, int variant, dim3 grid, cudaStream_t s) {
     typedef MLayout<SH> L;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(L::NT, 1, 1);
-    cfg.dynamicSmemBytes = L::SMEM;
-    cfg.stream = s;
-    cfg.attrs = at;
-    cfg.numAttrs = pdl_enabled() ? 1 : 0;
-    cudaError_t e;
     switch (variant & 3) {
-        case 0: e = cudaLaunchKernelEx(&cfg, k_step_m<0, SH>, a); break;
-        case 1: e = cudaLaunchKernelEx(&cfg, k_step_m<1, SH>, a); break;
-        case 2: e = cudaLaunchKernelEx(&cfg, k_step_m<2, SH>, a); break;
-        default: e = cudaLaunchKernelEx(&cfg, k_step_m<3, SH>, a); break;
+        case 0: return launch_pdl(k_step_m<0, SH>, a, L::NT, L::SMEM, grid, s);
+        case 1: return launch_pdl(k_step_m<1, SH>, a, L::NT, L::SMEM, grid, s);
+        case 2: return launch_pdl(k_step_m<2, SH>, a, L::NT, L::SMEM, grid, s);
+        default: return launch_pdl(k_step_m<3, SH>, a, L::NT, L::SMEM, grid, s);
     }
-    return e != cudaSuccess ? e : cudaGetLastError();
 }
 cudaError_t launch_expand(const Geom& g, const Coef<float>& k, const float2* mom, void* fout,
                           cudaStream_t s) {
@@ -2145,6 +2335,9 @@ cudaError_t launch_step_prec(const void* args, int variant, int shape, dim3 grid
     if (shape == SHAPE_8) return launch_step_shape<P, SHAPE_8>(a, variant, grid, s);
     if constexpr (has_shape(P, SHAPE_16))
         if (shape == SHAPE_16) return launch_step_shape<P, SHAPE_16>(a, variant, grid, s);
+#if LB_PREC != 0
+    if (shape == SHAPE_D8) return launch_direct<P>(a, variant, grid, s);
+#endif
 #if LB_PREC == 1
     if (shape == SHAPE_M8) return launch_moments_shape<SHAPE_M8>(a, variant, grid, s);
     if (shape == SHAPE_M8X2) return launch_moments_shape<SHAPE_M8X2>(a, variant, grid, s);

@@ -321,6 +321,22 @@ struct Layout {
     static_assert(SMEM <= 227 * 1024 - 1024 && SMEM_OBS <= 227 * 1024, "shared memory");
 };
 
+// Layout of the direct kernel (k_step_d): a 60 x 8 tile's populations, 14 rows
+// of columns x0 - 3 .. x0 + 62, and its deviation windows; 512 threads, one site
+// each.
+template <int P>
+struct DLayout {
+    typedef typename Prec<P>::T2 T2;
+    typedef float C;
+    typedef float2 C2;
+    static constexpr int TX = Prec<P>::TX, TR = 8, TY = 8, RX = TX + 4;
+    static constexpr int NT = RX * TR;
+    static constexpr int WIN = TY + 4;
+    static constexpr int NR = TY + 6, BX = TX + 6, PS = NR * BX;
+    static constexpr int WIN_OFF = (9 * PS * (int)sizeof(T2) + 127) / 128 * 128;
+    static constexpr int SMEM = WIN_OFF + 2 * WIN * RX * (int)sizeof(float2) + 128;
+};
+
 // Layout of the moment kernel (k_step_m): 60 x 8 tiles; a ring of 14 rows of
 // populations (the 8 + 6 rows a tile's deviation window pulls from), columns
 // x0 - 3 .. x0 + 62, and the deviation windows.  SHAPE_M8: one site per thread,

@@ -230,8 +230,17 @@ std::vector<Choice> candidates(lb_pool* P) {
     const int prec = P->shared.precision;
     std::vector<Choice> out;
     const bool moments = P->forced_rows == 0 && moments_ok(P->members[(size_t)P->active[0]].lat);
-    for (int shape : {SHAPE_8, SHAPE_16, SHAPE_8X2, SHAPE_M8, SHAPE_M8X2}) {
+    long long tiles8 = 0;
+    for (int j : P->active) {
+        const Lattice& L = P->members[(size_t)j].lat;
+        tiles8 += (long long)L.nstrips * L.ntiles_y;
+    }
+    // one-site tiles: the direct kernel for sets with few tiles, and none for
+    // the 16-bit formats where two CTAs per SM have enough
+    const int usual = default_shape(prec, false, tiles8, P->sms);
+    for (int shape : {SHAPE_8, SHAPE_D8, SHAPE_16, SHAPE_8X2, SHAPE_M8, SHAPE_M8X2}) {
         if (shape_moments(shape) != moments) continue;
+        if (shape == SHAPE_8 ? usual == SHAPE_D8 || usual == SHAPE_8X2 : shape == SHAPE_D8 && usual != SHAPE_D8) continue;
         if (!has_shape(prec, shape) || (P->forced_rows != 0 && shape_rows(shape) != P->forced_rows)) continue;
         // (where two CTAs fit an SM the 16-row tile runs only when asked for)
         if (shape == SHAPE_16 && has_shape(prec, SHAPE_8X2) && P->forced_rows == 0) continue;

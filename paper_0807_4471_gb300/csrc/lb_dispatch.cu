@@ -48,21 +48,23 @@ cudaError_t launch_observe(int precision, const CUtensorMap* tin, const void* ar
 
 cudaError_t launch_init_seeded(int precision, const Geom& g, const void* coef, void* fout,
                                double rho0, double amp, double u_wall, int init_shear,
-                               unsigned long long seed, cudaStream_t s) {
-    LB_SWITCH(precision, return launch_init_prec<P>(g, coef, fout, 0, nullptr, rho0, amp, u_wall,
-                                                    init_shear, seed, s))
+                               unsigned long long seed, const StateInit& state, cudaStream_t s) {
+    LB_SWITCH(precision, return launch_init_prec<P>(g, coef, fout, nullptr, rho0, amp, u_wall,
+                                                    init_shear, seed, state, s))
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_init_fields(int precision, const Geom& g, const void* coef, void* fout, int mode,
-                               const double* fields, cudaStream_t s) {
-    LB_SWITCH(precision, return launch_init_prec<P>(g, coef, fout, mode, fields, 0, 0, 0, 0, 0, s))
+cudaError_t launch_init_fields(int precision, const Geom& g, const void* coef, void* fout,
+                               const double* const fields[4], const StateInit& state, cudaStream_t s) {
+    LB_SWITCH(precision, return launch_init_prec<P>(g, coef, fout, fields, 0, 0, 0, 0, 0, state, s))
     return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_load_pops(int precision, const Geom& g, const void* coef, void* fout,
-                             const double* pops, int i0, int i1, cudaStream_t s) {
-    LB_SWITCH(precision, return launch_load_pops_prec<P>(g, coef, fout, pops, i0, i1, s))
+                             const double* pops, size_t species, size_t direction, int i0, int i1,
+                             const StateInit& state, cudaStream_t s) {
+    LB_SWITCH(precision,
+              return launch_load_pops_prec<P>(g, coef, fout, pops, species, direction, i0, i1, state, s))
     return cudaErrorInvalidValue;
 }
 

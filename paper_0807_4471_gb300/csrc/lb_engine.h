@@ -33,8 +33,6 @@ struct Lattice {
     bool inited;
     long long t;             // host mirror of the step count
     unsigned int err_latched;
-    long long next_sample;   // source of the device's DevStats::next_sample (lives with
-                             // the lattice, so the asynchronous copy needs no wait)
 };
 
 // One launch of the persistent step kernel over a set of lattices.
@@ -129,7 +127,8 @@ lb_status lattice_load_populations(Lattice& L, const double* f, long long t, int
 void lattice_advanced(Lattice& L, long long n, int shape);
 // Make a state that is held by its moments a population state (f*).
 lb_status lattice_to_populations(Lattice& L, cudaStream_t s);
-lb_status lattice_observe(Lattice& L, int obs, double* out, int q0, int q1, cudaStream_t s);
+// dst: the outputs of the kind (see StepArgs::obs_dst), or null.
+lb_status lattice_observe(Lattice& L, int obs, double* const dst[4], int q0, int q1, cudaStream_t s);
 lb_status lattice_fields(Lattice& L, double* rho_A, double* rho_B, double* ux, double* uy,
                          cudaStream_t s);
 // raw = 0: f(t) after streaming; raw = 1: the stored state as it is (f*(t-1)

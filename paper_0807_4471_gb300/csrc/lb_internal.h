@@ -164,6 +164,16 @@ struct BatchArgs {
                                 // after its density phase (else after its site phase)
 };
 
+// The device-side state that an initialising kernel leaves with the
+// populations: counters cleared but for these, wall momentum totals zero.
+struct StateInit {
+    DevStats* st;          // null: leave the state alone
+    long long t, next_sample;
+    int pull;
+    double* wsum;          // nwsum totals (0: none)
+    int nwsum;
+};
+
 // Observe-mode outputs (the kernel writes FP64 planes of nx*ny values).
 enum ObsKind : int { OBS_NONE = 0, OBS_FIELDS = 1, OBS_POPS = 2, OBS_TOTALS = 3 };
 
@@ -177,7 +187,9 @@ struct StepArgs {
     int pull;              // 1: input holds post-collision f*(t-1); 0: f(t) in place
     const float2* mom;     // FP32: the state's moments [3][ny][nx] where it is held by them, else null
     int obs;               // ObsKind; OBS_NONE = a time step
-    double* obs_out;       // observe output base
+    // OBS_FIELDS: rho_A, rho_B, u_x, u_y (null: not wanted), OBS_POPS: the first
+    // plane's address; device memory or pinned host memory
+    double* obs_dst[4];
     int q0, q1;            // OBS_POPS: planes [q0, q1) written
     const double* wsum;    // Couette: the strips' wall momentum totals, [2][nstrips]
     int nstrips;
@@ -231,21 +243,24 @@ cudaError_t launch_step(int precision, const void* args, int variant, int shape,
 cudaError_t kernels_configure(int precision);
 cudaError_t launch_observe(int precision, const CUtensorMap* tin, const void* args, dim3 grid,
                            cudaStream_t s);
+// Initial states (see k_init).  fields: rho_A, rho_B, u_x, u_y (velocities may
+// be null: zero), in device memory or pinned host memory.
 cudaError_t launch_init_seeded(int precision, const Geom& g, const void* coef, void* fout,
                                double rho0, double amp, double u_wall, int init_shear,
-                               unsigned long long seed, cudaStream_t s);
-// mode: 1, + 2 with u_x, + 4 with u_y (else zero) in fields [4][ny][nx]
-cudaError_t launch_init_fields(int precision, const Geom& g, const void* coef, void* fout, int mode,
-                               const double* fields, cudaStream_t s);
+                               unsigned long long seed, const StateInit& state, cudaStream_t s);
+cudaError_t launch_init_fields(int precision, const Geom& g, const void* coef, void* fout,
+                               const double* const fields[4], const StateInit& state, cudaStream_t s);
 
 // FP32: the populations f* of a state held by its moments, into a population
 // buffer (with its ghost copies).
 cudaError_t launch_expand(const Geom& g, const Coef<float>& k, const float2* mom, void* fout,
                           cudaStream_t s);
 
-// Restore directions [i0, i1) from FP64 populations [i1 - i0][2][ny][nx].
+// Restore directions [i0, i1) from FP64 populations: species s of direction i at
+// pops + s species + (i - i0) direction (device or pinned host memory).
 cudaError_t launch_load_pops(int precision, const Geom& g, const void* coef, void* fout,
-                             const double* pops, int i0, int i1, cudaStream_t s);
+                             const double* pops, size_t species, size_t direction, int i0, int i1,
+                             const StateInit& state, cudaStream_t s);
 
 // Per-precision launchers, one explicit instantiation per compilation of
 // lb_kernels.cu (-DLB_PREC=P).
@@ -258,10 +273,11 @@ cudaError_t launch_observe_prec(const CUtensorMap* tin, const void* args, dim3 g
                                 cudaStream_t s);
 template <int P>
 cudaError_t launch_load_pops_prec(const Geom& g, const void* coef, void* fout, const double* pops,
-                                  int i0, int i1, cudaStream_t s);
+                                  size_t species, size_t direction, int i0, int i1,
+                                  const StateInit& state, cudaStream_t s);
 template <int P>
-cudaError_t launch_init_prec(const Geom& g, const void* coef, void* fout, int mode,
-                             const double* fields, double rho0, double amp, double u_wall,
-                             int init_shear, unsigned long long seed, cudaStream_t s);
+cudaError_t launch_init_prec(const Geom& g, const void* coef, void* fout, const double* const* fields,
+                             double rho0, double amp, double u_wall, int init_shear,
+                             unsigned long long seed, const StateInit& state, cudaStream_t s);
 
 }  // namespace lbgb

@@ -1935,7 +1935,7 @@ __global__ void __launch_bounds__(Layout<P>::NT, P == LB_FP64 ? 1 : 2)
 #pragma unroll
                 for (int q = 0; q < 18; ++q)
                     if (q >= a.q0 && q < a.q1)
-                        a.obs_out[(size_t)(q - a.q0) * N + idx] =
+                        a.obs_dst[0][(size_t)(q - a.q0) * N + idx] =
                             widen(q < 9 ? h[q % 9].x : h[q % 9].y) * is + wgt<double>(q % 9) * rref;
             }
         } else {
@@ -1984,7 +1984,9 @@ __global__ void __launch_bounds__(Layout<P>::NT, P == LB_FP64 ? 1 : 2)
                 const double rA = rref + widen(dr[0].x), rB = rref + widen(dr[0].y);
                 const double mx = widen(jx.x) + widen(jx.y) + 0.5 * (widen(Fx.x) + widen(Fx.y));
                 const double my = widen(jy.x) + widen(jy.y) + 0.5 * (widen(Fy.x) + widen(Fy.y));
-                if (a.obs == OBS_FIELDS) {
+                if (a.obs_dst[0]) a.obs_dst[0][idx] = rA;
+                if (a.obs_dst[1]) a.obs_dst[1][idx] = rB;
+                if (a.obs_dst[2] || a.obs_dst[3]) {
                     const double tot = rA + rB;
                     const unsigned e = ((unsigned)__double2hiint(tot) >> 20) & 0x7ffu;
                     double ux, uy;
@@ -1996,10 +1998,8 @@ __global__ void __launch_bounds__(Layout<P>::NT, P == LB_FP64 ? 1 : 2)
                         ux = tot != 0.0 ? mx / tot : 0.0;
                         uy = tot != 0.0 ? my / tot : 0.0;
                     }
-                    a.obs_out[idx] = rA;
-                    a.obs_out[N + idx] = rB;
-                    a.obs_out[2 * N + idx] = ux;
-                    a.obs_out[3 * N + idx] = uy;
+                    if (a.obs_dst[2]) a.obs_dst[2][idx] = ux;
+                    if (a.obs_dst[3]) a.obs_dst[3][idx] = uy;
                 }
                 red[0] += rA;
                 red[1] += rB;
@@ -2056,19 +2056,33 @@ __global__ void __launch_bounds__(Layout<P>::NT, P == LB_FP64 ? 1 : 2)
 
 // ------------------------------------------------------------ init kernels
 // f(r, 0) = f^eq(rho_s, u) in place (the first step reads it unshifted).
-// mode 0: rho_s from the counter generator; mode 1 (+ 2, + 4): FP64 fields
-// [4][ny][nx], with (+ 2) u_x and (+ 4) u_y, else zero.
+// rho_s from the counter generator (rA null), or from FP64 fields (ux, uy null:
+// zero).  The lattice's counters and wall totals are set along with it, so that
+// an initialisation is one launch.
+__device__ __forceinline__ void init_state(const StateInit& z) {
+    if (!z.st || blockIdx.x != 0 || blockIdx.y != 0) return;
+    if (threadIdx.x == 0) {
+        DevStats st = {};
+        st.t = z.t;
+        st.next_sample = z.next_sample;
+        st.pull = z.pull;
+        *z.st = st;
+    }
+    for (int i = threadIdx.x; i < z.nwsum; i += blockDim.x) z.wsum[i] = 0.0;
+}
 template <int P>
-__global__ void k_init(Geom g, Coef<typename Prec<P>::C> k, typename Prec<P>::T2* fout, int mode,
-                       const double* fields, double rho0, double amp, double u_wall, int init_shear,
-                       unsigned long long seed) {
+__global__ void k_init(Geom g, Coef<typename Prec<P>::C> k, typename Prec<P>::T2* fout,
+                       const double* rA, const double* rB, const double* fux, const double* fuy,
+                       double rho0, double amp, double u_wall, int init_shear, unsigned long long seed,
+                       StateInit state) {
     typedef typename Prec<P>::T2 T2;
-    const long long N = (long long)g.nx * g.ny;
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < N;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(idx % g.nx), y = (int)(idx / g.nx);
+    init_state(state);
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= g.nx) return;
+    for (int y = blockIdx.y; y < g.ny; y += gridDim.y) {
+        const size_t idx = (size_t)y * g.nx + x;
         double r[2], ux, uy;
-        if (mode == 0) {
+        if (!rA) {
             for (int s = 0; s < 2; ++s) {
                 const uint64_t ctr = ((uint64_t)s * g.ny + y) * g.nx + x;
                 const uint64_t z = mix64(seed ^ mix64(ctr + 0x9E3779B97F4A7C15ULL));
@@ -2081,10 +2095,10 @@ __global__ void k_init(Geom g, Coef<typename Prec<P>::C> k, typename Prec<P>::T2
             ux = init_shear ? u_wall * (2.0 * y + 1.0 - g.ny) / (double)g.ny : 0.0;
             uy = 0.0;
         } else {
-            r[0] = fields[idx];
-            r[1] = fields[N + idx];
-            ux = mode & 2 ? fields[2 * N + idx] : 0.0;
-            uy = mode & 4 ? fields[3 * N + idx] : 0.0;
+            r[0] = rA[idx];
+            r[1] = rB[idx];
+            ux = fux ? fux[idx] : 0.0;
+            uy = fuy ? fuy[idx] : 0.0;
         }
         const double usq = ux * ux + uy * uy;
         const double rref = (double)k.rho_ref;
@@ -2113,22 +2127,32 @@ __global__ void k_init(Geom g, Coef<typename Prec<P>::C> k, typename Prec<P>::T2
 }
 
 // Restore directions [i0, i1) of a saved state: pops holds FP64 populations
-// f_is(r) of those directions as [i1 - i0][2][ny][nx]; the offsets
-// f - w_i rho_ref are encoded to the storage format (plus ghost copies).
+// f_is(r), species s of direction i at s species + (i - i0) direction; the
+// offsets f - w_i rho_ref are encoded to the storage format (plus ghost copies).
 template <int P>
 __global__ void k_load_pops(Geom g, typename Prec<P>::C rho_ref, typename Prec<P>::T2* fout,
-                            const double* pops, int i0, int i1) {
+                            const double* pops, size_t species, size_t direction, int i0, int i1,
+                            StateInit state) {
     typedef typename Prec<P>::T2 T2;
-    const long long N = (long long)g.nx * g.ny;
+    init_state(state);
     const double rref = (double)rho_ref;
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < N;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(idx % g.nx), y = (int)(idx / g.nx);
-        for (int i = i0; i < i1; ++i) {
-            const double* src = pops + (long long)(i - i0) * 2 * N;
-            const double off = wgt<double>(i) * rref, sc = (double)scale_of<P>();
-            put2<T2>(fout, g, i, x, y, encd2<T2>(sc * (src[idx] - off), sc * (src[N + idx] - off)));
-        }
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= g.nx) return;
+    for (int y = blockIdx.y; y < g.ny; y += gridDim.y) {
+        const double* src = pops + (size_t)y * g.nx + x;
+        double f[9][2];
+#pragma unroll
+        for (int i = 0; i < 9; ++i)
+            if (i >= i0 && i < i1) {
+                f[i][0] = src[(size_t)(i - i0) * direction];
+                f[i][1] = src[(size_t)(i - i0) * direction + species];
+            }
+#pragma unroll
+        for (int i = 0; i < 9; ++i)
+            if (i >= i0 && i < i1) {
+                const double off = wgt<double>(i) * rref, sc = (double)scale_of<P>();
+                put2<T2>(fout, g, i, x, y, encd2<T2>(sc * (f[i][0] - off), sc * (f[i][1] - off)));
+            }
     }
 }
 
@@ -2369,18 +2393,23 @@ cudaError_t launch_observe_prec(const CUtensorMap* tin, const void* args, dim3 g
     return cudaGetLastError();
 }
 
+// One thread per column, rows dealt over the grid: no index is divided.
+static dim3 site_grid(const Geom& g) {
+    const unsigned gx = (unsigned)((g.nx + 127) / 128);
+    const unsigned gy = gx < 152 * 128 ? 152 * 128 / gx : 1;
+    return dim3(gx, (unsigned)g.ny < gy ? (unsigned)g.ny : gy, 1);
+}
 template <int P>
-cudaError_t launch_init_prec(const Geom& g, const void* coef, void* fout, int mode,
-                             const double* fields, double rho0, double amp, double u_wall,
-                             int init_shear, unsigned long long seed, cudaStream_t s) {
+cudaError_t launch_init_prec(const Geom& g, const void* coef, void* fout, const double* const* fields,
+                             double rho0, double amp, double u_wall, int init_shear,
+                             unsigned long long seed, const StateInit& state, cudaStream_t s) {
     typedef typename Prec<P>::C C;
     typedef typename Prec<P>::T2 T2;
-    const long long N = (long long)g.nx * g.ny;
-    long long blocks = (N + 255) / 256;
-    if (blocks > 152 * 64) blocks = 152 * 64;
-    k_init<P><<<(unsigned)blocks, 256, 0, s>>>(g, *reinterpret_cast<const Coef<C>*>(coef),
-                                               reinterpret_cast<T2*>(fout), mode, fields, rho0, amp,
-                                               u_wall, init_shear, seed);
+    const double* const none[4] = {nullptr, nullptr, nullptr, nullptr};
+    const double* const* f = fields ? fields : none;
+    k_init<P><<<site_grid(g), 128, 0, s>>>(g, *reinterpret_cast<const Coef<C>*>(coef),
+                                           reinterpret_cast<T2*>(fout), f[0], f[1], f[2], f[3], rho0, amp,
+                                           u_wall, init_shear, seed, state);
     return cudaGetLastError();
 }
 
@@ -2398,22 +2427,22 @@ template cudaError_t launch_observe_prec<LB_PREC>(const CUtensorMap*, const void
                                                   cudaStream_t);
 template <int P>
 cudaError_t launch_load_pops_prec(const Geom& g, const void* coef, void* fout, const double* pops,
-                                  int i0, int i1, cudaStream_t s) {
+                                  size_t species, size_t direction, int i0, int i1,
+                                  const StateInit& state, cudaStream_t s) {
     typedef typename Prec<P>::C C;
     typedef typename Prec<P>::T2 T2;
-    const long long N = (long long)g.nx * g.ny;
-    long long blocks = (N + 255) / 256;
-    if (blocks > 152 * 64) blocks = 152 * 64;
-    k_load_pops<P><<<(unsigned)blocks, 256, 0, s>>>(
-        g, reinterpret_cast<const Coef<C>*>(coef)->rho_ref, reinterpret_cast<T2*>(fout), pops, i0, i1);
+    k_load_pops<P><<<site_grid(g), 128, 0, s>>>(g, reinterpret_cast<const Coef<C>*>(coef)->rho_ref,
+                                                reinterpret_cast<T2*>(fout), pops, species, direction, i0, i1,
+                                                state);
     return cudaGetLastError();
 }
 
 template cudaError_t launch_load_pops_prec<LB_PREC>(const Geom&, const void*, void*, const double*,
-                                                    int, int, cudaStream_t);
-template cudaError_t launch_init_prec<LB_PREC>(const Geom&, const void*, void*, int, const double*,
+                                                    size_t, size_t, int, int, const StateInit&,
+                                                    cudaStream_t);
+template cudaError_t launch_init_prec<LB_PREC>(const Geom&, const void*, void*, const double* const*,
                                                double, double, double, int, unsigned long long,
-                                               cudaStream_t);
+                                               const StateInit&, cudaStream_t);
 
 }  // namespace lbgb
 

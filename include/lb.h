@@ -250,8 +250,8 @@ lb_status lb_pool_run(lb_pool* pool, int64_t quantum, int32_t* active);
  * lb_pool_set_partition, or else the load-balance model's -- no tuning) and
  * capture its CUDA graph, so that the next lb_pool_run replays the graph
  * with no capture or instantiation in its way.  A later lb_pool_run on the
- * same member set keeps this partition.  Synchronises the pool stream when
- * it builds; LB_OK with nothing to do when no member has steps left. */
+ * same member set keeps this partition.  May synchronise the pool stream;
+ * LB_OK with nothing to do when no member has steps left. */
 lb_status lb_pool_prepare(lb_pool* pool);
 
 /* Steps done and whether the member has finished (all its steps). */

@@ -295,11 +295,13 @@ int choose_seg(const int* nstrips, const int* ntiles_y, int nlat, int G) {
         // equal items go round the CTAs: whole rounds count once, for all
         cost.assign((size_t)g, 0.0);
         double all = 0.0;
-        long long it = 0;
+        int at = 0;   // the CTA whose turn it is
         auto deal = [&](long long n, double c) {
             all += (double)(n / g) * c;
-            for (long long k = 0; k < n % g; ++k) cost[(size_t)((it + k) % g)] += c;
-            it += n;
+            for (int k = (int)(n % g); k > 0; --k) {
+                cost[(size_t)at] += c;
+                if (++at == g) at = 0;
+            }
         };
         for (int l = 0; l < nlat; ++l) {
             deal((long long)nstrips[l] * (ntiles_y[l] / seg), seg + 0.25);
@@ -459,32 +461,31 @@ void partition(Lattice* const* lats, int nlat, int seg, int shape, int sms, std:
     // cost stays within B) number at most sms, found by bisection -- at most
     // one tile above the mean, where cutting at equal cumulative cost lets
     // some runs overshoot by a whole tile.
-    std::vector<double> tc;
-    std::vector<char> sbeg;   // tile begins a strip
+    std::vector<double> tc, upto;   // tile costs; their sums with the strips' starts
     tc.reserve((size_t)tiles);
-    sbeg.reserve((size_t)tiles);
-    double sum = 0.0, cmax = 0.0;
+    upto.reserve((size_t)tiles + 1);
+    upto.push_back(0.0);
+    double cmax = 0.0;
     for (int l = 0; l < nlat; ++l)
         for (int sx = 0; sx < lats[l]->nstrips; ++sx)
             for (int ty = 0; ty < nty[(size_t)l]; ++ty) {
-                tc.push_back(cost(l, sx, ty));
-                sbeg.push_back(ty == 0 ? 1 : 0);
-                sum += tc.back() + (ty == 0 ? kItemStart : 0.0);
-                cmax = std::max(cmax, tc.back());
+                const double c = cost(l, sx, ty);
+                tc.push_back(c);
+                upto.push_back(upto.back() + c + (ty == 0 ? kItemStart : 0.0));
+                cmax = std::max(cmax, c);
             }
-    // runs needed under bound B; with starts, the first tile of each run
+    const double sum = upto.back();
+    // Runs needed under bound B; with starts, the first tile of each run.  A run
+    // from tile k costs its first tile and a start, then what the sums grow by;
+    // its end is found by bisection (costs are multiples of 0.01: sums closer
+    // than 1e-6 are equal).
     auto runs_for = [&](double B, std::vector<long long>* starts) -> long long {
         long long n = 0;
-        double acc = 0.0;
-        for (long long k = 0; k < tiles; ++k) {
-            const double add = tc[(size_t)k] + (sbeg[(size_t)k] ? kItemStart : 0.0);
-            if (n > 0 && acc + add <= B) {
-                acc += add;
-            } else {
-                ++n;
-                if (starts) starts->push_back(k);
-                acc = tc[(size_t)k] + kItemStart;
-            }
+        for (long long k = 0; k < tiles;) {
+            ++n;
+            if (starts) starts->push_back(k);
+            const double most = upto[(size_t)k + 1] + (B - tc[(size_t)k] - kItemStart) + 1e-6;
+            k = std::upper_bound(upto.begin() + (k + 2), upto.end(), most) - upto.begin() - 1;
         }
         return n;
     };

@@ -25,7 +25,10 @@
 //     periodic ghost copies.
 //  4. Couette: the wall sites' momentum exchange, summed per strip in FP64
 //     after the tile loop and, at sampled steps, added to the strip's total.
-// There is no dense contraction anywhere, so no tensor cores are used.
+// Two more step kernels share its site arithmetic: k_step_d, for lattices with
+// few tiles (a shorter chain of latencies), and k_step_m, for FP32 at tau = 1
+// (the state held by its moments).  There is no dense contraction anywhere, so
+// no tensor cores are used.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 

@@ -45,3 +45,21 @@ def test_fp64_density_range(lb, O, rho0, rho_ref, lo, hi, boundary):
     g.step(3)
     assert rel_err(gpu_pops_as_oracle(g.populations()), f) < 1e-13
     g.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(84, 152), (28, 304), (112, 152), (85, 151)])
+def test_fp64_pool_with_more_items_than_tiles(lb, nx, ny):
+    """A pool's FP64 work items are runs of rows: a small set has more of them
+    than 8-row tiles (84 x 152: 152 items, 57 tiles).  Bitwise the lattice
+    handle's populations."""
+    p = lb.make_params(nx, ny, "fp64", psi_form=lb.LB_PSI_RHO0)
+    g = lb.Lattice(p).init_seeded(4)
+    g.step(5)
+    pool = lb.Pool(p, 64 << 20, max_jobs=2)
+    j = pool.admit(p, seed=4, steps=5)
+    pool.run(5)
+    ra, rb = pool.fields(j)[:2]
+    ga, gb = g.fields()[:2]
+    assert np.array_equal(ra, ga) and np.array_equal(rb, gb)
+    pool.close()
+    g.close()

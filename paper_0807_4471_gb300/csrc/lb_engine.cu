@@ -115,10 +115,11 @@ static Region region_layout(const lb_params* p) {
     off = align_up(off + sizeof(DevStats), kAlign);
     r.slots = off;
     off = align_up(off + sizeof(double) * 4 * ntiles, kAlign);
-    // the step's wall-momentum pair of every wall site (bottom row, then top
-    // row), in the compute precision (at most two doubles)
+    // the wall-momentum pair of every wall site (bottom row, then top row) of
+    // two steps, in the compute precision
     r.wallx = off;
-    off = align_up(off + (size_t)2 * (size_t)p->nx * 2 * sizeof(double), kAlign);
+    off = align_up(off + (size_t)4 * (size_t)p->nx *
+                             (p->precision == LB_FP64 ? sizeof(double2) : sizeof(float2)), kAlign);
     // their sums per strip (at most nx strips), bottom then top
     r.wsum = off;
     off = align_up(off + (size_t)2 * (size_t)p->nx * sizeof(double), kAlign);

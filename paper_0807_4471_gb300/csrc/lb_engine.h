@@ -18,7 +18,7 @@ struct Lattice {
                              // buffer 0 | buffer 1
     DevStats* st;
     double* slots;           // observe partial sums, 4 per tile
-    char* wallx;             // the step's wall-momentum pairs: [2][nx] (bottom, top), compute type
+    char* wallx;             // two steps' wall-momentum pairs: [2][2][nx] (bottom, top), compute type
     double* wsum;            // their sums per strip and over the sampled steps: [2][nstrips]
     char* fbuf[2];
     size_t fbytes;

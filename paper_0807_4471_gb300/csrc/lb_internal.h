@@ -134,8 +134,9 @@ struct alignas(128) LatDesc {
     LatVals<C> v;
     void* fbuf[2];
     DevStats* st;
-    void* wallx;           // [2][nx] compute-type pairs: x-momentum handed to the bottom
-                           // (then top) wall by the links leaving site x, this step
+    void* wallx;           // [2][2][nx] compute-type pairs, by the parity of the window's
+                           // step: x-momentum handed to the bottom (then top) wall by
+                           // the links leaving site x in that step
     double* wsum;          // [2][nstrips]: those summed per strip (bottom, then top) and
                            // over the sampled steps
     int nstrips;           // ceil(nx / TX)

@@ -24,7 +24,8 @@
 //     (staging tile + TMA bulk tensor store, or direct stores) and the
 //     periodic ghost copies.
 //  4. Couette: the wall sites' momentum exchange, summed per strip in FP64
-//     after the tile loop and, at sampled steps, added to the strip's total.
+//     by the next launch (a window's last launch: at its end) and, at sampled
+//     steps, added to the strip's total.
 // Two more step kernels share its site arithmetic: k_step_d, for lattices with
 // few tiles (a shorter chain of latencies), and k_step_m, for FP32 at tau = 1
 // (the state held by its moments).  There is no dense contraction anywhere, so
@@ -611,7 +612,7 @@ __device__ __forceinline__ void site_velocity(C2 rho, C2 jx, C2 jy, C2 Fx, C2 Fy
 // with (a, b) = (8, 7) at the bottom wall and (5, 6) at the top
 // (c_ax = 1, c_bx = -1; w_a = w_b, so the offsets' difference is the
 // populations').  One compute-type value per site and species, kept
-// in the lattice's wall columns for the sums after the tile loop.
+// in the lattice's wall columns for the next launch's sums (wall_sums).
 template <int P, typename C, typename C2>
 __device__ __forceinline__ C2 wall_momentum(const C2 sv[9], bool down, const LatVals<C>& v) {
     const C uw = down ? -v.u_wall : v.u_wall;
@@ -714,6 +715,22 @@ __device__ __forceinline__ void site_update(
     }
 }
 
+// A float widened to double.  The conversion instruction runs on the FP64
+// pipe; a normal value's bits are moved by integer operations instead.
+__device__ __forceinline__ double widen(float x) {
+    const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+    return m == 0u ? __hiloint2double((int)b, 0) : (double)x;
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
+// The wall columns [2][nx] that a window's step `step` writes: two sets in turn.
+template <typename C2>
+__device__ __forceinline__ C2* wall_columns(void* wallx, int nx, int step) {
+    return reinterpret_cast<C2*>(wallx) + (step & 1) * 2 * nx;
+}
+
 // Wall momentum of one CTA's items that hold a wall row, in FP64, at the
 // lattices' sampled steps: the wall-site values the site phase left in the
 // lattice's wall columns, summed over the item's strip in a fixed order (lane l
@@ -723,35 +740,36 @@ __device__ __forceinline__ void site_update(
 // Sampled steps: stress_t0 + k stress_every; DevStats::next_sample is the
 // first one from the window's start on (32-bit remainder: a window is short,
 // and a 64-bit one would compile to a call).
+// The chain of dependent loads and FP64 additions takes 1.5 us, as much as half a
+// small lattice's step.  So a launch sums the previous launch's values (step
+// `step` of the window, from the wall columns of that parity) while its own
+// first loads are in flight, and only the window's last launch sums its own
+// at its end: 300 x 211 FP32 with tau = 0.8 7.39 -> 6.31 us a step, tau = 1 6.45 -> 5.35,
+// FP16 6.96 -> 5.80, 128^2 FP16 6.62 -> 5.74.  (The last warps: the first ones have the most to do.)
 template <int P, class L>
 __device__ __forceinline__ void wall_sums(const BatchArgs<typename Prec<P>::C>& a, int it0, int it_end,
-                                       int tid) {
+                                       int tid, int step) {
     typedef typename L::C C;
     typedef typename L::C2 C2;
     const int lane = tid & 31, warp = tid >> 5;
-    int n = 0;
-    for (int it = it0; it < it_end; ++it) {
+    for (int it = it0 + (L::NT / 32 - 1 - warp); it < it_end; it += L::NT / 32) {
         const int4 w = a.items[it];
         const LatDesc<C>* d = &a.lat[w.x];
         const bool bot = w.z == 0, top = w.w == d->ntiles_y;
         if (d->g.periodic || !(bot || top)) continue;
-        if (n++ % (L::NT / 32) != warp) continue;
-        const long long since = d->st->t + a.step_k - d->st->next_sample;
+        const long long since = d->st->t + step - d->st->next_sample;
         if (since < 0 || (unsigned)since % (unsigned)d->stress_every != 0u) continue;
         const int nx = d->g.nx;
         const int xe = min(w.y * L::TX + L::TX, nx);
-        const C2* wx = reinterpret_cast<const C2*>(d->wallx);
-        double sb = 0.0, st = 0.0;
-        for (int x = w.y * L::TX + lane; x < xe; x += 32) {
-            if (bot) sb += (double)wx[x].x + (double)wx[x].y;
-            if (top) st += (double)wx[nx + x].x + (double)wx[nx + x].y;
-        }
-        sb = warp_sum(sb);
-        st = warp_sum(st);
-        if (lane == 0) {
-            if (bot) d->wsum[w.y] += sb;
-            if (top) d->wsum[d->nstrips + w.y] += st;
-        }
+        const C2* wx = wall_columns<C2>(d->wallx, nx, step);
+        auto strip = [&](const C2* m, double* total) {
+            double sum = 0.0;
+            for (int x = w.y * L::TX + lane; x < xe; x += 32) sum += widen(m[x].x) + widen(m[x].y);
+            sum = warp_sum(sum);
+            if (lane == 0) *total += sum;
+        };
+        if (bot) strip(wx, d->wsum + w.y);
+        if (top) strip(wx + nx, d->wsum + d->nstrips + w.y);
     }
 }
 
@@ -1013,6 +1031,8 @@ __global__ void __launch_bounds__(Layout<P, SH>::NT, Layout<P, SH>::CTAS)
     griddep_launch_dependents();
     if (tid == 0)
         while (p_pos < L::NB && issue_next()) {}
+    if constexpr (!ALLPER)
+        if (step_k != 0) wall_sums<P, L>(a, a.cta_items[blockIdx.x], it_end, tid, step_k - 1);
     int ty_b = 0, ty = 0;   // the consumer's item end and tile (read by release)
     // Producer: the tile whose first block is at position q is done with
     // its blocks before the next tile's first one (all of them at an item's
@@ -1193,7 +1213,7 @@ __global__ void __launch_bounds__(Layout<P, SH>::NT, Layout<P, SH>::CTAS)
                         [[maybe_unused]] uint32_t srh = 0u;   // the shared hash of this thread's sites
                         if constexpr (sizeof(T2) == 4) srh = sr_hash(key, x, y, g.nx);
                         o.valid = 1;
-                        o.wallx = d->wallx;
+                        o.wallx = wall_columns<C2>(d->wallx, g.nx, step_k);
                         if constexpr (!STAGED) {
                             o.plane = g.plane;
                             o.gdx = x < 3 ? g.nx : (x >= g.nx - 3 ? -g.nx : 0);
@@ -1277,17 +1297,14 @@ __global__ void __launch_bounds__(Layout<P, SH>::NT, Layout<P, SH>::CTAS)
         if (s_fail) break;
         c_pos += ADV * (ty_b - ty_a) + 1;
     }
-    // Wall momentum of this CTA's items that hold a wall row, in FP64: the
-    // wall-site values the site phase left in the lattice's wall columns,
-    // summed over the item's strip in a fixed order (lane l takes columns
-    // l, l + 32, ..., then the butterfly), one warp per item -- so the sums
-    // do not depend on the partition or the tile shape.  Kept out of the
-    // tile loop: a per-item reduction there (barriers, FP64 shuffles) cost
+    // The wall momentum of a window's last step (see wall_sums).  Kept out of
+    // the tile loop: a per-item reduction there (barriers, FP64 shuffles) cost
     // the generic variant 1-4 % even on periodic lattices, which skip it.
-    if constexpr (!ALLPER) {
-        __syncthreads();   // this CTA's wall-site values are written
-        if (!s_fail) wall_sums<P, L>(a, a.cta_items[blockIdx.x], it_end, tid);
-    }
+    if constexpr (!ALLPER)
+        if (a.advance) {
+            __syncthreads();   // this CTA's wall-site values are written
+            if (!s_fail) wall_sums<P, L>(a, a.cta_items[blockIdx.x], it_end, tid, step_k);
+        }
     if (STAGED && tid == kStoreThread) bulk_wait_all();
     if (s_fail && tid == 0) {
         // Let copies in flight land before the CTA exits.  No slot is
@@ -1404,6 +1421,8 @@ __global__ void __launch_bounds__(DLayout<P>::NT, 1)
                 if (t_j + 8 < NR) cell(t_j + 8, t_w + 1, h1);
                 const int r = tid >> 1, c = tid & 1 ? BX - 1 : 0;   // outermost columns
                 if (tid < 2 * NR) cell(r, c, he);
+                if constexpr (!ALLPER)   // (the loads are on their way)
+                    if (step_k != 0 && it == it0 && ty == w.z) wall_sums<P, L>(a, it0, it_end, tid, step_k - 1);
                 put(t_j, t_w + 1, h0);
                 if (t_j + 8 < NR) put(t_j + 8, t_w + 1, h1);
                 if (tid < 2 * NR) put(r, c, he);
@@ -1451,7 +1470,7 @@ __global__ void __launch_bounds__(DLayout<P>::NT, 1)
                                       qy, dp, dr);
                     SiteOut<T2> o;
                     o.valid = 1;
-                    o.wallx = d->wallx;
+                    o.wallx = wall_columns<float2>(d->wallx, g.nx, step_k);
                     o.plane = g.plane;
                     o.pol = pol;
                     o.gout = fout + (long long)(y + kGY) * g.pitch + (x + g.gx);
@@ -1477,8 +1496,8 @@ __global__ void __launch_bounds__(DLayout<P>::NT, 1)
         }
         if (!(nf.x == 0.0f && nf.y == 0.0f)) atomicOr(&d->st->err, ERR_NONFINITE);
     }
-    if constexpr (!ALLPER) wall_sums<P, L>(a, it0, it_end, tid);   // (behind the tiles' last barrier)
     if (!a.advance) return;
+    if constexpr (!ALLPER) wall_sums<P, L>(a, it0, it_end, tid, step_k);   // (behind the tiles' last barrier)
     __syncthreads();
     if (tid == 0) s_last = ticket_arrive(a.ticket) == (unsigned int)(gridDim.x - 1);
     __syncthreads();
@@ -1646,6 +1665,8 @@ __global__ void __launch_bounds__(MLayout<SH>::NT, MLayout<SH>::CTAS)
             for (int q = 0; q < R; ++q)
                 if (t_j + q * L::TR < NR) hd[q] = load_mom(ya - 3 + t_j + q * L::TR, xw);
             if (tid < 2 * NR) he = load_mom(ya - 3 + (tid >> 1), xe);
+            if constexpr (!ALLPER)   // (the loads are on their way)
+                if (step_k != 0 && it == it0) wall_sums<P, L>(a, it0, it_end, tid, step_k - 1);
 #pragma unroll
             for (int q = 0; q < R; ++q)
                 if (t_j + q * L::TR < NR) put_mom(hd[q], t_j + q * L::TR, t_w + 1, false);
@@ -1781,7 +1802,7 @@ __global__ void __launch_bounds__(MLayout<SH>::NT, MLayout<SH>::CTAS)
                             // the packed product; a scalar one it does not
                             const float2 Q = pfma(pmul(rho, pset(-4.0f / 6.0f)), pfma(zx, zx, pmul(zy, zy)), dr[s]);
                             h[0] = make_float2(__fmul_rn(a.k.omw[0].x, Q.x), __fmul_rn(a.k.omw[0].y, Q.y));
-                            reinterpret_cast<float2*>(d->wallx)[(ys == 0 ? 0 : nx) + x] =
+                            wall_columns<float2>(d->wallx, nx, step_k)[(ys == 0 ? 0 : nx) + x] =
                                 wall_momentum<P>(h, ys == 0, v);
                         }
                     }
@@ -1798,11 +1819,11 @@ __global__ void __launch_bounds__(MLayout<SH>::NT, MLayout<SH>::CTAS)
         }
         if (!(nf.x == 0.0f && nf.y == 0.0f)) atomicOr(&d->st->err, ERR_NONFINITE);
     }
+    if (!a.advance) return;
     if constexpr (!ALLPER) {
         __syncthreads();   // this CTA's wall-site values are written
-        wall_sums<P, L>(a, it0, it_end, tid);
+        wall_sums<P, L>(a, it0, it_end, tid, step_k);
     }
-    if (!a.advance) return;
     __syncthreads();
     if (tid == 0) s_last = ticket_arrive(a.ticket) == (unsigned int)(gridDim.x - 1);
     __syncthreads();
@@ -1837,16 +1858,6 @@ __global__ void k_expand(Geom g, const __grid_constant__ Coef<float> k, const fl
 // reduced once per CTA instead of once per tile, one reciprocal serves both
 // velocity components, and populations take no force and no totals (2048^2 FP16:
 // 15 operations, 154 us, and 21, 222 us; FP32 from the moments about the same).
-
-// A float widened to double.  The conversion instruction runs on the FP64
-// pipe; a normal value's bits are moved by integer operations instead.
-__device__ __forceinline__ double widen(float x) {
-    const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
-    if (m - 0x00800000u < 0x7f000000u)
-        return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
-    return m == 0u ? __hiloint2double((int)b, 0) : (double)x;
-}
-__device__ __forceinline__ double widen(double x) { return x; }
 
 template <int P, int V, bool POPS>
 __global__ void __launch_bounds__(Layout<P>::NT, P == LB_FP64 ? 1 : 2)

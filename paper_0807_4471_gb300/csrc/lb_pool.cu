@@ -147,6 +147,9 @@ void drop_graph(lb_pool* P) {
 }
 
 lb_status build(lb_pool* P, Choice c) {
+    // until it succeeds there is no launch: the tables and member forms of the
+    // one before may be gone when it fails on the way
+    P->built = false;
     drop_graph(P);
     std::vector<Lattice*> lats;
     for (int j : P->active) lats.push_back(&P->members[(size_t)j].lat);

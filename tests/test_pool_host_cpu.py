@@ -1,0 +1,46 @@
+"""Host side of the lattice pool, without a GPU (see _fake_host)."""
+import pytest
+
+from _fake_host import run
+
+GROW = """
+small = lb.make_params(40, 40, "fp64", psi_form=1)
+big = lb.make_params(600, 900, "fp64", psi_form=1)
+pool = lb.lb_pool_create(small, 1 << 30, 4)
+j = lb.lb_pool_admit(pool, small, 1, 1000)
+lb.lb_pool_run(pool, 3)
+assert lb.lb_pool_segment(pool) == -1
+lb.lb_pool_admit(pool, big, 2, 1000)      # more items than the tables hold
+"""
+
+
+@pytest.mark.parametrize("api", ["cudaMalloc", "cudaMemcpyAsync"])
+def test_failed_prepare_leaves_the_pool_unbuilt(api):
+    """A member set whose launch could not be built has none: the next run builds
+    it, and does not step the previous set's launch."""
+    run(GROW + f"""
+fk.fk_fail(b"{api}", 1, 2)
+assert status(lb.lb_pool_prepare, pool) == lb.LB_ERR_NOMEM
+assert lb.lb_pool_segment(pool) == 0 and lb.lb_pool_tile_rows(pool) == 0
+fk.fk_reset()
+lb.lb_pool_run(pool, 5)
+steps = launches("k_step")
+assert len(steps) == 5
+assert {{i[1] for i in step_items(steps[0])}} == {{0, 1}}     # both members
+lb.lb_pool_destroy(pool)
+""")
+
+
+def test_pool_runs_on_after_a_failed_growth():
+    """No room for larger item tables: the smaller set runs once the large member
+    is gone."""
+    run(GROW + """
+fk.fk_reset()
+fk.fk_fail(b"cudaMalloc", 1, 2)
+assert status(lb.lb_pool_run, pool, 5) == lb.LB_ERR_NOMEM
+assert not launches("k_step")
+lb.lb_pool_release(pool, 1)
+lb.lb_pool_run(pool, 5)
+assert len(launches("k_step")) == 5
+lb.lb_pool_destroy(pool)
+""")

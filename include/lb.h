@@ -175,7 +175,10 @@ lb_status lb_init_populations(lb_handle* h, const double* f, int64_t t);
 lb_status lb_checkpoint(lb_handle* h, double* state, int64_t* t, int32_t* pulled);
 lb_status lb_restore(lb_handle* h, const double* state, int64_t t, int32_t pulled);
 
-/* Advance n >= 0 time steps of Eq. (1) (asynchronous on the stream). */
+/* Advance n >= 0 time steps of Eq. (1) (asynchronous on the stream).  When a
+ * launch fails with earlier steps of the call enqueued, the lattice's state is
+ * lost: calls that need one return LB_ERR_STATE until it is initialised or
+ * restored.  (A failure at the call's first step leaves the state as it was.) */
 lb_status lb_step(lb_handle* h, int64_t n);
 
 /* Copy the fields at the current time to host FP64 arrays [ny][nx]: the
@@ -242,7 +245,9 @@ lb_status lb_pool_admit(lb_pool* pool, const lb_params* p, uint64_t seed, int64_
 /* Advance every active member by min(quantum, its remaining steps); members
  * that reach their step count drop out of the launches.  *active (may be
  * NULL) receives the number of members with steps left afterwards.
- * Asynchronous except for re-partitioning and tuning. */
+ * Asynchronous except for re-partitioning and tuning.  A launch that fails may
+ * leave the active members without a state, as in lb_step: LB_ERR_STATE until
+ * each is restarted (lb_pool_init_fields) or released. */
 lb_status lb_pool_run(lb_pool* pool, int64_t quantum, int32_t* active);
 
 /* Set up the step launch of the current member set without taking a step:

@@ -176,8 +176,10 @@ lb_status lb_step(lb_handle* h, int64_t n) {
     lb_status s = LB_OK;
     while (n > 0 && s == LB_OK) {
         const int w = n < (1 << 20) ? (int)n : 1 << 20;
-        s = launch_window(h->launch, w, h->stream);
+        bool broken = false;
+        s = launch_window(h->launch, w, h->stream, &broken);
         if (s == LB_OK) lattice_advanced(h->lat, w, h->launch.shape);
+        if (broken) h->lat.inited = false;   // the state is lost
         n -= w;
     }
     nvtxRangePop();

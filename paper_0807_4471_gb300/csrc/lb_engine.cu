@@ -773,10 +773,16 @@ lb_status launch_run(Launch& Ln, int step_k, int advance, cudaStream_t s) {
     return cuda_status(launch_step(Ln.precision, args, Ln.variant, Ln.shape, Ln.grid, s));
 }
 
-lb_status launch_window(Launch& Ln, int n, cudaStream_t s) {
-    lb_status st = LB_OK;
-    for (int k = 0; k < n && st == LB_OK; ++k) st = launch_run(Ln, k, k == n - 1 ? n : 0, s);
-    return st;
+lb_status launch_window(Launch& Ln, int n, cudaStream_t s, bool* broken) {
+    *broken = false;
+    for (int k = 0; k < n; ++k) {
+        const lb_status st = launch_run(Ln, k, k == n - 1 ? n : 0, s);
+        if (st != LB_OK) {
+            *broken = k > 0;
+            return st;
+        }
+    }
+    return LB_OK;
 }
 
 static lb_status lattice_observe_pull(Lattice& L, int obs, double* const dst[4], int q0, int q1, int pull,

@@ -111,8 +111,9 @@ size_t launch_area_doubles(size_t tiles, size_t strips, int sms);
 // window's steps on its last launch, else 0.  The device's step counters move
 // with the window's last launch only.
 lb_status launch_run(Launch& Ln, int step_k, int advance, cudaStream_t s);
-// Enqueue n steps as one window (n < 2^30).
-lb_status launch_window(Launch& Ln, int n, cudaStream_t s);
+// Enqueue n steps as one window (n < 2^30).  *broken: a launch failed with
+// earlier ones of the window enqueued, which no launch's counters follow.
+lb_status launch_window(Launch& Ln, int n, cudaStream_t s, bool* broken);
 
 lb_status lattice_init_seeded(Lattice& L, uint64_t seed, cudaStream_t s);
 lb_status lattice_init_fields(Lattice& L, const double* rho_A, const double* rho_B,

@@ -191,7 +191,8 @@ lb_status capture_graph(lb_pool* P) {
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(P->stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_status(e);
-    lb_status s = launch_window(P->launch, kGraphChunk, P->stream);
+    bool broken;   // (nothing runs)
+    lb_status s = launch_window(P->launch, kGraphChunk, P->stream, &broken);
     e = cudaStreamEndCapture(P->stream, &g);
     if (s != LB_OK) {
         if (g) cudaGraphDestroy(g);
@@ -206,8 +207,17 @@ lb_status capture_graph(lb_pool* P) {
     return LB_OK;
 }
 
+// n steps of the active members were enqueued.
+void advanced(lb_pool* P, long long n) {
+    for (int j : P->active) {
+        Member& m = P->members[(size_t)j];
+        lattice_advanced(m.lat, n, P->launch.shape);
+        m.done += n;
+    }
+}
+
 // Run k steps of the built launch: captured chunks (a long run, or a graph that
-// is there), then single launches.
+// is there), then single launches.  The members' counts follow what was enqueued.
 lb_status run_steps(lb_pool* P, long long k) {
     const bool graph = P->graph || k >= kGraphLeast;
     while (graph && k >= kGraphChunk) {
@@ -215,17 +225,15 @@ lb_status run_steps(lb_pool* P, long long k) {
         if (s != LB_OK) return s;
         cudaError_t e = cudaGraphLaunch(P->graph, P->stream);
         if (e != cudaSuccess) return cuda_status(e);
+        advanced(P, kGraphChunk);
         k -= kGraphChunk;
     }
-    return launch_window(P->launch, (int)k, P->stream);
-}
-
-void advanced(lb_pool* P, long long k) {
-    for (int j : P->active) {
-        Member& m = P->members[(size_t)j];
-        lattice_advanced(m.lat, k, P->launch.shape);
-        m.done += k;
-    }
+    bool broken = false;
+    const lb_status s = launch_window(P->launch, (int)k, P->stream, &broken);
+    if (s == LB_OK) advanced(P, k);
+    if (broken)   // the members' states are lost
+        for (int j : P->active) P->members[(size_t)j].lat.inited = false;
+    return s;
 }
 
 // The choices open to the tuner (the fixed dimensions of lb_pool_set_partition
@@ -308,7 +316,6 @@ long long tune(lb_pool* P, long long budget_steps, lb_status* st) {
         cudaEventSynchronize(e1);
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
-        advanced(P, kTuneSteps);
         used += kTuneSteps;
         if (ms < best_ms) {
             best_ms = ms;
@@ -339,6 +346,13 @@ long long active_members(lb_pool* P, long long limit, std::vector<int>& act) {
     return k;
 }
 
+// Every member's state is whole (see run_steps).
+bool states_whole(const lb_pool* P, const std::vector<int>& act) {
+    for (int j : act)
+        if (!P->members[(size_t)j].lat.inited) return false;
+    return true;
+}
+
 }  // namespace
 
 extern "C" {
@@ -348,6 +362,7 @@ lb_status lb_pool_prepare(lb_pool* P) {
     std::vector<int> act;
     active_members(P, 1, act);
     if (act.empty()) return LB_OK;
+    if (!states_whole(P, act)) return LB_ERR_STATE;
     if (!P->built || act != P->active) {
         P->active = act;
         auto it = P->tuned.find(cache_key(P));
@@ -451,6 +466,7 @@ lb_status lb_pool_run(lb_pool* P, int64_t quantum, int32_t* active_out) {
         std::vector<int> act;
         long long k = active_members(P, remaining, act);
         if (act.empty()) break;
+        if (!states_whole(P, act)) return LB_ERR_STATE;
         if (!P->built || act != P->active) {
             P->active = act;
             P->built = false;   // the previous member set's launch no longer applies
@@ -470,7 +486,6 @@ lb_status lb_pool_run(lb_pool* P, int64_t quantum, int32_t* active_out) {
         if (k > 0) {
             s = run_steps(P, k);
             if (s != LB_OK) return s;
-            advanced(P, k);
             remaining -= k;
         }
     }
@@ -496,6 +511,7 @@ lb_status lb_pool_fields(lb_pool* P, lb_job job, double* rho_A, double* rho_B, d
                          double* uy) {
     if (!P || job < 0 || (size_t)job >= P->members.size() || !P->members[(size_t)job].used)
         return LB_ERR_INVALID;
+    if (!P->members[(size_t)job].lat.inited) return LB_ERR_STATE;
     return lattice_fields(P->members[(size_t)job].lat, rho_A, rho_B, ux, uy, P->stream);
 }
 
@@ -513,6 +529,7 @@ lb_status lb_pool_init_fields(lb_pool* P, lb_job job, const double* rho_A, const
 lb_status lb_pool_stress(lb_pool* P, lb_job job, lb_stress_out* out) {
     if (!P || !out || job < 0 || (size_t)job >= P->members.size() || !P->members[(size_t)job].used)
         return LB_ERR_INVALID;
+    if (!P->members[(size_t)job].lat.inited) return LB_ERR_STATE;
     return lattice_stress(P->members[(size_t)job].lat, out, P->stream);
 }
 

@@ -873,24 +873,44 @@ static StateInit lattice_reset(Lattice& L, long long t, int pull) {
     return z;
 }
 
+// Whether [p, p + bytes) lies in one allocation or registration as the driver
+// knows it (the two ends alone do not tell: they may be pinned apart, with
+// pageable memory between them).
+typedef CUresult (*PointerAttributeFn)(void*, CUpointer_attribute, CUdeviceptr);
+static bool in_one_range(const void* p, size_t bytes) {
+    static const PointerAttributeFn get = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault, &q) !=
+                cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<PointerAttributeFn>(f);
+    }();
+    const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    return get && get(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, at) == CUDA_SUCCESS &&
+           get(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, at) == CUDA_SUCCESS && at >= start &&
+           at - start <= size && bytes <= size - (at - start);
+}
+
 // The address under which the device reaches `bytes` of pinned host memory, or
-// null where that memory is not pinned throughout (or not aligned for doubles).
+// null where they do not lie in one pinned range (or are not aligned for doubles).
 // Kernels read and write pinned arrays over the link themselves, at the rate of
 // a copy (193 GB/s out, 211 GB/s in), which saves the staging pass, the copies
 // and their launches: lb_fields of the densities of a 512^2 FP16 lattice 81 -> 64
 // us, all four fields of 4096^2 3.9 -> 3.2 ms; lb_restore of 1024^2 910 -> 740 us.
 static double* pinned_view(const double* host, size_t bytes) {
-    cudaPointerAttributes a, b;
-    const char* last = reinterpret_cast<const char*>(host) + bytes - 1;
+    cudaPointerAttributes a;
     if (reinterpret_cast<uintptr_t>(host) % sizeof(double) != 0) return nullptr;
-    if (cudaPointerGetAttributes(&a, host) != cudaSuccess || cudaPointerGetAttributes(&b, last) != cudaSuccess) {
+    if (cudaPointerGetAttributes(&a, host) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
-    if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer || !b.devicePointer ||
-        reinterpret_cast<char*>(b.devicePointer) - reinterpret_cast<char*>(a.devicePointer) !=
-            (ptrdiff_t)(bytes - 1))
-        return nullptr;
+    if (a.type != cudaMemoryTypeHost || !a.devicePointer || !in_one_range(host, bytes)) return nullptr;
     return reinterpret_cast<double*>(a.devicePointer);
 }
 

@@ -2,6 +2,7 @@
 // one lattice region plus the step-launch area (arrival counter, lattice
 // descriptor, item tables) in one workspace.  The engine in
 // lb_engine.cu does the work; every step of the model runs in the kernels.
+#include <algorithm>
 #include <cstring>
 #include <new>
 
@@ -25,9 +26,12 @@ namespace {
 
 constexpr size_t kAlign = 256;
 
+// SMs a lattice's launch uses at most: its workspace is sized without a device.
+constexpr int kMostSms = 256;
+
 // Handle workspace: the lattice region, then the step-launch area.
 struct HandleLayout {
-    size_t lattice, ticket, desc, slots, total;
+    size_t lattice, ticket, desc, slots, room, total;   // room: doubles at slots
 };
 HandleLayout handle_layout(const lb_params* p) {
     HandleLayout H;
@@ -42,8 +46,8 @@ HandleLayout handle_layout(const lb_params* p) {
     H.desc = off;
     off = align_up(off + sizeof(LatDesc<double>), kAlign);
     H.slots = off;
-    // item tables (items <= tiles + strips; up to 1024 CTAs)
-    off = align_up(off + sizeof(double) * launch_area_doubles(ntiles, nstrips, 1024), kAlign);
+    H.room = launch_area_doubles(p->precision, ntiles, nstrips, kMostSms);
+    off = align_up(off + sizeof(double) * H.room, kAlign);
     H.total = off;
     return H;
 }
@@ -62,11 +66,11 @@ lb_status create_common(const lb_params* p, void* stream, void* ws, size_t bytes
     if (s == LB_OK) s = lattice_setup(h->lat, p, h->ws + H.lattice);
     if (s == LB_OK) {
         Lattice* one = &h->lat;
-        const int sms = device_sms(h->device);
+        const int sms = std::min(device_sms(h->device), kMostSms);
         const int shape = shape_of_rows(p->precision, moments_ok(*one), p->tile_rows,
                                         (long long)one->nstrips * one->ntiles_y, sms);
         s = launch_build(h->launch, &one, 1, h->ws + H.desc,
-                         reinterpret_cast<double*>(h->ws + H.slots),
+                         reinterpret_cast<double*>(h->ws + H.slots), H.room,
                          reinterpret_cast<unsigned int*>(h->ws + H.ticket), sms, h->stream, nullptr,
                          0, shape);
     }

@@ -369,9 +369,12 @@ static void fill_desc(LatDesc<C>& d, const Lattice& L, const Coef<C>& k, int nti
     d.stress_every = L.p.stress_every;
 }
 
-size_t launch_area_doubles(size_t tiles, size_t strips, int sms) {
-    // items (int4, at most one per 8-row tile and strip) | CTA offsets
-    return 2 * (tiles + strips) + (2 * (size_t)sms + 2) / 2 + 8;   // at most two CTAs per SM
+// Items (int4) | CTA offsets.  Segments and runs of tiles hold a tile at least
+// each.  FP64 runs are cut by rows: a run per CTA (one CTA per SM), cut again
+// where it enters a strip.  (84 x 152: 152 items, 57 tiles.)
+size_t launch_area_doubles(int precision, size_t tiles, size_t strips, int sms) {
+    const size_t items = precision == LB_FP64 ? std::max(tiles, (size_t)sms) + strips : tiles;
+    return 2 * items + (2 * (size_t)sms + 2) / 2;   // at most two CTAs per SM
 }
 
 namespace {
@@ -640,7 +643,7 @@ cudaError_t HostStage::sent(cudaStream_t s) {
 }
 
 lb_status launch_build(Launch& Ln, Lattice* const* lats, int nlat, void* descs, double* slots,
-                       unsigned int* ticket, int sms, cudaStream_t stream, HostStage* stage,
+                       size_t room, unsigned int* ticket, int sms, cudaStream_t stream, HostStage* stage,
                        int forced_seg, int shape) {
     if (nlat < 1) return LB_ERR_INVALID;
     const int prec = lats[0]->p.precision;
@@ -690,6 +693,7 @@ lb_status launch_build(Launch& Ln, Lattice* const* lats, int nlat, void* descs, 
     const size_t at_items = align_up(dsz * (size_t)nlat, 128);
     const size_t at_cta = at_items + sizeof(Item) * (size_t)nitems;
     const size_t bytes = at_cta + sizeof(int) * cta.size();
+    if (bytes - at_items > room * sizeof(double)) return LB_ERR_NOMEM;
     std::vector<char> own;
     char* hs = nullptr;
     if (stage) {

@@ -100,13 +100,13 @@ private:
 // through pageable memory and the stream is synchronised.  All lattices share the precision
 // and the coefficients of lats[0] (couplings, tau, forcing).  seg > 0 forces
 // the segment length; seg = 0 takes choose_seg's; seg < 0 cuts the tiles
-// into one contiguous run per CTA.  `slots` holds launch_area_doubles(tiles,
-// strips, sms) doubles for the lattices' total tiles and strips: the item
-// tables.
+// into one contiguous run per CTA.  `slots` holds `room` doubles for the item
+// tables, launch_area_doubles of the lattices' total 8-row tiles and strips;
+// LB_ERR_NOMEM where they do not fit.
 lb_status launch_build(Launch& Ln, Lattice* const* lats, int nlat, void* descs, double* slots,
-                       unsigned int* ticket, int sms, cudaStream_t stream, HostStage* stage,
+                       size_t room, unsigned int* ticket, int sms, cudaStream_t stream, HostStage* stage,
                        int seg = 0, int shape = SHAPE_8);
-size_t launch_area_doubles(size_t tiles, size_t strips, int sms);
+size_t launch_area_doubles(int precision, size_t tiles, size_t strips, int sms);
 // Enqueue step step_k of a window of consecutive steps (0-based); advance: the
 // window's steps on its last launch, else 0.  The device's step counters move
 // with the window's last launch only.

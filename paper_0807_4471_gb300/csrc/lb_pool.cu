@@ -159,14 +159,12 @@ lb_status build(lb_pool* P, Choice c) {
             lb_status s = lattice_to_populations(*L, P->stream);
             if (s != LB_OK) return s;
         }
-    // item tables: items are most numerous for seg = 1 (one per tile); FP64 runs
-    // are cut by rows, so a small set has up to one per CTA and strip instead
     size_t tiles = 0, strips = 0;
     for (Lattice* L : lats) {
         tiles += (size_t)L->nstrips * (size_t)L->ntiles_y;
         strips += (size_t)L->nstrips;
     }
-    const size_t need = launch_area_doubles(std::max(tiles, 2 * (size_t)P->sms), strips, P->sms);
+    const size_t need = launch_area_doubles(P->shared.precision, tiles, strips, P->sms);
     if (need > P->slot_cap) {
         cudaError_t e = cudaStreamSynchronize(P->stream);
         if (P->slots) cudaFree(P->slots);
@@ -178,7 +176,7 @@ lb_status build(lb_pool* P, Choice c) {
     }
     cudaError_t ce = kernels_configure(P->shared.precision);   // before any graph capture
     if (ce != cudaSuccess) return cuda_status(ce);
-    lb_status s = launch_build(P->launch, lats.data(), nlat, P->desc_mem, P->slots, P->ticket,
+    lb_status s = launch_build(P->launch, lats.data(), nlat, P->desc_mem, P->slots, P->slot_cap, P->ticket,
                                P->sms, P->stream, &P->stage, c.seg, c.shape);
     P->built = s == LB_OK;
     return s;

@@ -193,7 +193,8 @@ lb_status lb_fields(lb_handle* h, double* rho_A, double* rho_B, double* ux, doub
 lb_status lb_populations(lb_handle* h, double* f);
 
 /* Totals at the current time and the time-averaged wall stress of the
- * Couette walls (response R = nu0/nu_eff as defined after Fig. 3).
+ * Couette walls (response R = nu0/nu_eff as defined after Fig. 3).  The order
+ * of every sum is fixed by the lattice size and the precision alone.
  * Synchronises. */
 lb_status lb_stress(lb_handle* h, lb_stress_out* out);
 

@@ -797,12 +797,12 @@ lb_status lattice_observe(Lattice& L, int obs, double* const dst[4], int q0, int
 
 static lb_status lattice_observe_pull(Lattice& L, int obs, double* const dst[4], int q0, int q1, int pull,
                                       cudaStream_t s) {
-    // CTAs take several tiles each once every SM is full (2048 threads)
+    // CTAs take several tiles each once every SM of a GB300 is full (2048 threads
+    // on each of 152; not the device's own count: the CTAs set the order in which
+    // the totals are added, which is the same on every GPU)
     const long long tiles = (long long)L.nstrips * L.ntiles_y;
     const int threads = L.p.precision == LB_FP64 ? 256 : 512;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const long long most = (long long)device_sms(dev) * (2048 / threads);
+    const long long most = 152LL * (2048 / threads);
     dim3 grid((unsigned)std::min(tiles, most), 1, 1);
     cudaError_t e;
     if (L.p.precision == LB_FP64) {

@@ -603,35 +603,45 @@ lb_status plan_partition(const lb_params* ps, int nlat, int seg, int tile_rows, 
 }
 
 HostStage::~HostStage() {
-    for (Buffer& b : buf_) {
+    for (Buffer& b : buf_)
         if (b.done) {
             if (b.busy) cudaEventSynchronize(b.done);
             cudaEventDestroy(b.done);
         }
-        if (b.mem) cudaFreeHost(b.mem);
+    for (char* m : blocks_) cudaFreeHost(m);
+}
+
+cudaError_t HostStage::reserve(size_t bytes) {
+    cudaError_t e = cudaSuccess;
+    for (Buffer& b : buf_)
+        if (!b.done && (e = cudaEventCreateWithFlags(&b.done, cudaEventDisableTiming)) != cudaSuccess) {
+            b.done = nullptr;
+            return e;
+        }
+    if (bytes <= cap_) return e;
+    const size_t cap = align_up(std::max(bytes, 2 * cap_), 64 << 10);
+    char* m = nullptr;
+    e = cudaHostAlloc(reinterpret_cast<void**>(&m), kBuffers * cap, cudaHostAllocDefault);
+    if (e != cudaSuccess) return e;
+    blocks_.push_back(m);
+    cap_ = cap;
+    // (copies out of the buffers before may be on their way: their memory stays)
+    for (int k = 0; k < kBuffers; ++k) {
+        buf_[k].mem = m + k * cap;
+        buf_[k].busy = false;
     }
+    return e;
 }
 
 char* HostStage::get(size_t bytes) {
+    if (reserve(bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
     last_ = (last_ + 1) % kBuffers;
     Buffer& b = buf_[last_];
     if (b.busy && cudaEventSynchronize(b.done) != cudaSuccess) return nullptr;
     b.busy = false;
-    if (!b.done && cudaEventCreateWithFlags(&b.done, cudaEventDisableTiming) != cudaSuccess) {
-        b.done = nullptr;
-        return nullptr;
-    }
-    if (b.cap < bytes) {
-        if (b.mem) cudaFreeHost(b.mem);
-        b.mem = nullptr;
-        b.cap = 0;
-        const size_t cap = align_up(bytes + bytes / 2, 64 << 10);
-        if (cudaHostAlloc(reinterpret_cast<void**>(&b.mem), cap, cudaHostAllocDefault) != cudaSuccess) {
-            b.mem = nullptr;
-            return nullptr;
-        }
-        b.cap = cap;
-    }
     return b.mem;
 }
 

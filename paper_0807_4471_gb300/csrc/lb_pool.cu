@@ -28,6 +28,7 @@ constexpr int kGraphChunk = 16;   // steps per captured graph
 // take 0.2 ms, during which the device has nothing to do (16 served jobs of
 // 64..200^2, quanta of 100 steps: 7.2 -> 6.5 ms with this and the staged tables).
 constexpr int kGraphLeast = 512;
+constexpr size_t kStageLeast = 128 << 10;   // tables of a few dozen lattices
 constexpr int kTuneSteps = 6;     // timed steps per candidate (tile shape, partition)
 // A new member set is tuned only if it runs at least kTuneShare times the
 // steps that timing all candidates takes: a short-lived set (a server's
@@ -144,6 +145,22 @@ void drop_graph(lb_pool* P) {
         cudaGraphExecDestroy(P->graph);
         P->graph = nullptr;
     }
+}
+
+// Bytes of the descriptors and tables of a launch over all members with the
+// partitions a run takes untuned: contiguous runs, or segments dealt a few to a
+// CTA.  (What the tuner tries beyond it waits for the device anyway.)
+size_t stage_bytes(const lb_pool* P) {
+    size_t lats = 0, tiles = 0, strips = 0;
+    for (const Member& m : P->members)
+        if (m.used) {
+            ++lats;
+            tiles += (size_t)m.lat.nstrips * (size_t)m.lat.ntiles_y;
+            strips += (size_t)m.lat.nstrips;
+        }
+    return align_up(lats * sizeof(LatDesc<double>), 128) +
+           sizeof(double) * launch_area_doubles(P->shared.precision, std::min(tiles, 32 * (size_t)P->sms + strips),
+                                                strips, P->sms);
 }
 
 lb_status build(lb_pool* P, Choice c) {
@@ -411,6 +428,7 @@ lb_status lb_pool_create(const lb_params* shared, size_t bytes_budget, int32_t m
         P->ticket = reinterpret_cast<unsigned int*>(P->desc_mem + dbytes);
         e = cudaMemsetAsync(P->ticket, 0, sizeof(unsigned int), P->stream);
     }
+    if (e == cudaSuccess) e = P->stage.reserve(kStageLeast);
     if (e != cudaSuccess) {
         lb_pool_destroy(P);
         return cuda_status(e);
@@ -449,6 +467,8 @@ lb_status lb_pool_admit(lb_pool* P, const lb_params* p, uint64_t seed, int64_t s
     m.target = steps;
     m.done = 0;
     *job = slot;
+    // (where there is no pinned memory to be had now, the next build tries again)
+    if (P->stage.reserve(stage_bytes(P)) != cudaSuccess) cudaGetLastError();
     return LB_OK;
 }
 

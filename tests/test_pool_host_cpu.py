@@ -44,3 +44,43 @@ lb.lb_pool_run(pool, 5)
 assert len(launches("k_step")) == 5
 lb.lb_pool_destroy(pool)
 """)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "fp16"])
+@pytest.mark.parametrize("sizes", [[(128, 128)], [(64 + 8 * k, 200 - 5 * k) for k in range(24)],
+                                   [(512, 512)] * 40, [(4096, 4096)], [(2048, 2048), (30, 3000)]])
+def test_runs_allocate_nothing(prec, sizes):
+    """The buffers a launch's tables go through are there before the first run of a
+    member set; a run neither allocates nor frees (either may wait for the steps
+    that are enqueued)."""
+    run(f"""
+ps = [lb.make_params(nx, ny, "{prec}", psi_form=1) for nx, ny in {sizes}]
+pool = lb.lb_pool_create(ps[0], sum(map(lb.lb_pool_footprint, ps)), len(ps))
+for p in ps:
+    lb.lb_pool_admit(pool, p, 1, 100)
+    fk.fk_reset()
+    lb.lb_pool_run(pool, 2)
+    assert len(launches("k_step")) == 2
+    for api in ("cudaHostAlloc", "cudaFreeHost", "cudaEventCreate"):
+        assert count(api) == 0, api
+fk.fk_reset()
+lb.lb_pool_destroy(pool)
+""")
+
+
+def test_larger_tables_keep_the_old_buffers():
+    """Partitions with more items than the buffers hold (one tile each): new buffers,
+    and the old ones, out of which copies may be on their way, stay to the end."""
+    run("""
+p = lb.make_params(4096, 2048, "fp16", psi_form=1)
+pool = lb.lb_pool_create(p, lb.lb_pool_footprint(p), 1)
+lb.lb_pool_admit(pool, p, 1, 100)
+lb.lb_pool_run(pool, 2)
+lb.lb_pool_set_partition(pool, 1)
+fk.fk_reset()
+lb.lb_pool_run(pool, 2)
+assert count("cudaHostAlloc") == 1 and count("cudaFreeHost") == 0
+assert len(step_items(launches("k_step")[0])) == 69 * 256
+lb.lb_pool_destroy(pool)
+assert count("cudaFreeHost") == 2
+""")

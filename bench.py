@@ -43,7 +43,7 @@ def bytes_per_site(precision: str, tile_rows: int = 0) -> int:
 
 # the sources that define the step kernel's code
 KERNEL_SRCS = [os.path.join(ROOT, "paper_0807_4471_gb300", "csrc", f)
-               for f in ("lb_kernels.cu", "lb_layout.cuh", "lb_internal.h")]
+               for f in ("lb_kernels.cu", "lb_layout.cuh", "lb_exp_table.h", "lb_internal.h")]
 
 
 def kernel_hash() -> str:

@@ -164,8 +164,6 @@ static void fill_coef(Coef<C>& k, const lb_params* p) {
     k.psi_scale = (C)(pref * std::exp(-rref / p->rho0));
     k.inv_rho0 = (C)(1.0 / p->rho0);
     k.exp_c = (C)(-64.0 / (M_LN2 * p->rho0));
-    k.psi_a = k.psi_ref * k.psi_scale;
-    k.psi_b = -k.psi_scale * k.psi_scale;
     k.tau15[0] = (C)(1.5 * p->tau_A);
     k.tau15[1] = (C)(1.5 * p->tau_B);
     k.omega[0] = (C)(1.0 / p->tau_A);

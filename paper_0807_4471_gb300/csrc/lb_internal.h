@@ -72,8 +72,8 @@ template <> struct PairOf<double> { typedef double2 T; };
 // exact), and the cross-species ones WC = {w(1), w(2)} for both species.
 // FP64 folds factors so that a site takes fewer FP64 operations: its window
 // holds E = exp(-(rho - rho_ref)/rho0) - 1 in place of the Psi deviation
-// -psi_scale E, its cross weights are {4, 1} = {w(1), w(2)} / w(2), and
-// psi_a, psi_b and gx_rho0 carry the factors.
+// -psi_scale E, its cross weights are {4, 1} = {w(1), w(2)} / w(2), and the
+// site's -Psi (neg_psi) and gx_rho0 carry the factors.
 template <typename C>
 struct Coef {
     typedef typename PairOf<C>::T C2;
@@ -84,7 +84,6 @@ struct Coef {
     C psi_scale;       // P exp(-rho_ref / rho0)
     C inv_rho0;        // 1 / rho0
     C exp_c;           // FP64: -64 / (ln2 rho0), see pexpm1_scaled
-    C psi_a, psi_b;    // FP64: psi_ref psi_scale, -psi_scale^2
     C rho_ref;         // reference density of the stored offsets
     C tau15[2];        // 1.5 tau_s (the velocity shift is taken for v = 1.5u)
     C omega[2];        // 1 / tau
@@ -105,7 +104,7 @@ template <typename C>
 struct LatVals {
     C rho_ref, psi_ref, psi_scale, inv_rho0, gx_rho0, u_wall;
     C kolmo_w;         // 2 pi kolmo_k / ny (ny is per lattice)
-    C exp_c, psi_a, psi_b;   // (FP64)
+    C exp_c;           // (FP64)
 };
 template <typename C>
 __host__ __device__ inline LatVals<C> vals_of(const Coef<C>& k) {
@@ -118,8 +117,6 @@ __host__ __device__ inline LatVals<C> vals_of(const Coef<C>& k) {
     v.u_wall = k.u_wall;
     v.kolmo_w = k.kolmo_w;
     v.exp_c = k.exp_c;
-    v.psi_a = k.psi_a;
-    v.psi_b = k.psi_b;
     return v;
 }
 

@@ -248,13 +248,14 @@ __device__ __forceinline__ double2 dpsi_of(double2 d, const LatVals<double>& v, 
     return pexpm1_scaled(d, v.exp_c, v.inv_rho0, tab);
 }
 // -Psi_s(r) from the window value; FP64: times the factor that the stencil
-// sums of the window values lack, -psi_scale:
-// -(psi_ref - psi_scale E)(-psi_scale) = psi_ref psi_scale - psi_scale^2 E.
+// sums of the window values lack, -psi_scale.  (Not as psi_ref psi_scale -
+// psi_scale^2 E, two operations less a site: psi_scale^2 leaves the normal numbers
+// where rho_ref / rho0 is above 354.)
 __device__ __forceinline__ float2 neg_psi(float2 dpsi, const LatVals<float>& v) {
     return psub(pset(-v.psi_ref), dpsi);
 }
 __device__ __forceinline__ double2 neg_psi(double2 E, const LatVals<double>& v) {
-    return pfma(pset(v.psi_b), E, pset(v.psi_a));
+    return pmul(pset(-v.psi_scale), pfma(pset(v.psi_scale), E, pset(-v.psi_ref)));
 }
 // Adds 0 * rho to nf: NaN from the first inf or NaN density on, else zero.
 // (FP64: by the exponent bits, without an FP64 operation.)

@@ -367,6 +367,16 @@ lb_status lb_selftest_wait(void* stream, int32_t limit);
  * LB_ERR_INVALID for n < 0 or a NULL pointer with n > 0. */
 lb_status lb_selftest_math(const float* x, float* out, int64_t n, void* stream);
 
+/* Diagnostic, no counterpart in the paper: the FP64 functions of the step and
+ * of the fields next to CUDA's, on n pairs of caller values (x[k], y[k]).
+ * x, y: device arrays of n doubles; out: device array of 6 n doubles, receiving
+ * at out[6k ..]: the step's exp(-x/rho0) - 1 and the library's expm1(-x (1/rho0)),
+ * the step's reciprocal of x and 1.0 / x, the fields' quotient y / x and the
+ * division.  Asynchronous on `stream`; LB_ERR_INVALID for n < 0, rho0 <= 0 or a
+ * NULL pointer with n > 0. */
+lb_status lb_selftest_math64(double rho0, const double* x, const double* y, double* out, int64_t n,
+                             void* stream);
+
 /* Static description of a status code. */
 const char* lb_status_string(lb_status s);
 

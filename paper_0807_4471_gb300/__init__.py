@@ -111,6 +111,8 @@ def load():
             "lb_pool_segment": (C.c_int32, [H]),
             "lb_selftest_wait": (C.c_int, [H, C.c_int32]),
             "lb_selftest_math": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p]),
+            "lb_selftest_math64": (C.c_int, [C.c_double, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int64,
+                                             C.c_void_p]),
             "lb_pool_set_partition": (C.c_int, [H, C.c_int32]),
             "lb_pool_set_tile_rows": (C.c_int, [H, C.c_int32]),
             "lb_pool_tile_rows": (C.c_int32, [H]),
@@ -290,6 +292,12 @@ def lb_selftest_math(x_ptr: int, out_ptr: int, n: int, stream: int = 0):
     """Device pointers: n FP32 arguments in, 3 n FP32 values out (see include/lb.h)."""
     _check(load().lb_selftest_math(C.c_void_p(x_ptr), C.c_void_p(out_ptr), n, C.c_void_p(stream)),
            "lb_selftest_math")
+
+
+def lb_selftest_math64(rho0: float, x_ptr: int, y_ptr: int, out_ptr: int, n: int, stream: int = 0):
+    """Device pointers: n pairs of FP64 arguments in, 6 n FP64 values out (see include/lb.h)."""
+    _check(load().lb_selftest_math64(rho0, C.c_void_p(x_ptr), C.c_void_p(y_ptr), C.c_void_p(out_ptr), n,
+                                     C.c_void_p(stream)), "lb_selftest_math64")
 
 
 def lb_pool_segment(pool: int) -> int:

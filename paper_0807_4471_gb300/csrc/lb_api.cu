@@ -252,6 +252,13 @@ lb_status lb_selftest_math(const float* x, float* out, int64_t n, void* stream) 
     return cuda_status(launch_math_probe(x, out, (long long)n, reinterpret_cast<cudaStream_t>(stream)));
 }
 
+lb_status lb_selftest_math64(double rho0, const double* x, const double* y, double* out, int64_t n,
+                             void* stream) {
+    if (n < 0 || !(rho0 > 0.0) || (n > 0 && (!x || !y || !out))) return LB_ERR_INVALID;
+    if (n == 0) return LB_OK;
+    return cuda_status(launch_math64_probe(rho0, x, y, out, (long long)n, reinterpret_cast<cudaStream_t>(stream)));
+}
+
 const char* lb_status_string(lb_status s) {
     switch (s) {
         case LB_OK: return "ok";

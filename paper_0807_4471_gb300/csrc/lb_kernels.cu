@@ -1850,6 +1850,9 @@ __global__ void k_expand(Geom g, const __grid_constant__ Coef<float> k, const fl
 }
 #endif
 
+// m / t, given r = recip(t).
+__device__ __forceinline__ double over(double m, double t, double r) { return m * r; }
+
 // --------------------------------------------------------- observe kernel
 // Fields, totals or populations of one lattice's current state, with the same
 // site arithmetic as the step; CTAs take tiles b, b + G, ...  GB300 has two FP64
@@ -2007,8 +2010,8 @@ __global__ void __launch_bounds__(Layout<P>::NT, P == LB_FP64 ? 1 : 2)
                     double ux, uy;
                     if (e - 64u < 1920u) {   // well inside the normal range
                         const double r = recip(tot);
-                        ux = mx * r;
-                        uy = my * r;
+                        ux = over(mx, tot, r);
+                        uy = over(my, tot, r);
                     } else {
                         ux = tot != 0.0 ? mx / tot : 0.0;
                         uy = tot != 0.0 ? my / tot : 0.0;
@@ -2206,6 +2209,25 @@ __global__ void k_wait_selftest(unsigned int* err, int limit) {
     }
     __syncthreads();
     if (threadIdx.x == 0 && !mbar_wait_bounded(&bar, 0, limit)) atomicOr(err, ERR_TIMEOUT);
+}
+#endif
+
+#if LB_PREC == 0
+// The FP64 functions of the step and observe kernels on caller values, next to
+// CUDA's: see lb_selftest_math64.
+__global__ void k_math64_probe(double rho0, const double* __restrict__ x, const double* __restrict__ y,
+                               double* __restrict__ out, long long n) {
+    const double inv_rho0 = 1.0 / rho0, c = -64.0 / (0.693147180559945309417 * rho0);
+    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
+         k += (long long)gridDim.x * blockDim.x) {
+        const double a = x[k], b = y[k];
+        out[6 * k] = pexpm1_scaled(make_double2(a, b), c, inv_rho0, g_exp_tab).x;
+        out[6 * k + 1] = expm1(-a * inv_rho0);
+        out[6 * k + 2] = recip(a);
+        out[6 * k + 3] = 1.0 / a;
+        out[6 * k + 4] = over(b, a, recip(a));
+        out[6 * k + 5] = b / a;
+    }
 }
 #endif
 
@@ -2460,6 +2482,18 @@ template cudaError_t launch_init_prec<LB_PREC>(const Geom&, const void*, void*, 
                                                const StateInit&, cudaStream_t);
 
 }  // namespace lbgb
+
+#if LB_PREC == 0
+namespace lbgb {
+cudaError_t launch_math64_probe(double rho0, const double* x, const double* y, double* out, long long n,
+                                cudaStream_t s) {
+    long long blocks = (n + 255) / 256;
+    if (blocks > 152 * 8) blocks = 152 * 8;
+    k_math64_probe<<<(unsigned)(blocks > 0 ? blocks : 1), 256, 0, s>>>(rho0, x, y, out, n);
+    return cudaGetLastError();
+}
+}  // namespace lbgb
+#endif
 
 #if LB_PREC == 1
 namespace lbgb {

@@ -86,7 +86,7 @@ struct Coef {
     C psi_ref;         // Psi(rho_ref)
     C psi_scale;       // P exp(-rho_ref / rho0)
     C inv_rho0;        // 1 / rho0
-    C exp_c;           // FP64: -64 / (ln2 rho0), see pexpm1_scaled
+    C exp_c;           // FP64: -64 / (ln2 rho0), which picks the table entry (pexpm1_scaled)
     C rho_ref;         // reference density of the stored offsets
     C tau15[2];        // 1.5 tau_s (the velocity shift is taken for v = 1.5u)
     C omega[2];        // 1 / tau

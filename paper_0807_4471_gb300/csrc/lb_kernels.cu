@@ -233,7 +233,7 @@ __device__ __forceinline__ void load_site(const typename Prec<P>::T2* bm,
 }
 
 #if LB_PREC == 0
-static __device__ const double2 g_exp_tab[kExpN] = {LB_EXP_TABLE};
+static __device__ const ExpTable g_exp_tab = {{LB_EXP_TABLE}, {LB_EXP_ARGS}};
 __device__ __noinline__ double expm1_slow(double x) { return expm1(x); }
 #endif
 
@@ -241,10 +241,10 @@ __device__ __noinline__ double expm1_slow(double x) { return expm1(x); }
 // Psi(rho_ref + d) - Psi(rho_ref) = -P exp(-rho_ref/rho0) expm1(-d/rho0).
 // FP64: without the factor -P exp(-rho_ref/rho0), which neg_psi carries; tab:
 // the exponential table.
-__device__ __forceinline__ float2 dpsi_of(float2 d, const LatVals<float>& v, const double2*) {
+__device__ __forceinline__ float2 dpsi_of(float2 d, const LatVals<float>& v, const ExpTable*) {
     return pmul(pset(-v.psi_scale), pexpm1(pmul(d, pset(-v.inv_rho0))));
 }
-__device__ __forceinline__ double2 dpsi_of(double2 d, const LatVals<double>& v, const double2* tab) {
+__device__ __forceinline__ double2 dpsi_of(double2 d, const LatVals<double>& v, const ExpTable* tab) {
     return pexpm1_scaled(d, v.exp_c, v.inv_rho0, tab);
 }
 // -Psi_s(r) from the window value; FP64: times the factor that the stencil
@@ -291,7 +291,7 @@ __device__ __forceinline__ void cell_dev(const typename Prec<P>::T2* bm,
                                          const typename Prec<P>::T2* bp, int y, bool per, int pull,
                                          const Geom& g, const LatVals<typename Prec<P>::C>& v,
                                          typename Prec<P>::C2& r, typename Prec<P>::C2& q,
-                                         const double2* tab, typename Prec<P>::C2* j = nullptr) {
+                                         const ExpTable* tab, typename Prec<P>::C2* j = nullptr) {
     typename Prec<P>::C2 h[9];
     load_site<P, PS>(bm, b0, bp, y, per, pull, g, v, h);
     r = sum9(h);
@@ -969,9 +969,11 @@ __global__ void __launch_bounds__(Layout<P, SH>::NT, Layout<P, SH>::CTAS)
     // TAU1: momenta (jx, jy) of the first thread rows' new cells, kept for
     // the next tile, whose first sites they are; jc: this thread's entries
     // FP64: the exponential table, copied while the previous step drains
-    double2* s_tab = reinterpret_cast<double2*>(smem + L::TAB_OFF);
+    ExpTable* s_tab = reinterpret_cast<ExpTable*>(smem + L::TAB_OFF);
 #if LB_PREC == 0
-    for (int i = tid; i < kExpN; i += L::NT) s_tab[i] = g_exp_tab[i];
+    static_assert(sizeof(ExpTable) % sizeof(double2) == 0, "copied in pairs");
+    for (int i = tid; i < (int)(sizeof(ExpTable) / sizeof(double2)); i += L::NT)
+        reinterpret_cast<double2*>(s_tab)[i] = reinterpret_cast<const double2*>(&g_exp_tab)[i];
 #endif
     __shared__ __align__(16) C2 s_jcarry[kCarry * L::RX * SPT * 2];
     C2* const jc = s_jcarry + ((t_carry ? t_j : 0) * L::RX + t_lx) * (SPT * 2);
@@ -1885,9 +1887,9 @@ __global__ void __launch_bounds__(Layout<P>::NT, P == LB_FP64 ? 1 : 2)
     const Geom& g = a.g;
     const bool per = g.periodic != 0;
     const LatVals<C> v = vals_of(a.k);
-    const double2* tab = nullptr;
+    const ExpTable* tab = nullptr;
 #if LB_PREC == 0
-    tab = g_exp_tab;
+    tab = &g_exp_tab;
 #endif
     bool from_mom = false;
 #if LB_PREC == 1
@@ -2221,7 +2223,7 @@ __global__ void k_math64_probe(double rho0, const double* __restrict__ x, const 
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
          k += (long long)gridDim.x * blockDim.x) {
         const double a = x[k], b = y[k];
-        out[6 * k] = pexpm1_scaled(make_double2(a, b), c, inv_rho0, g_exp_tab).x;
+        out[6 * k] = pexpm1_scaled(make_double2(a, b), c, inv_rho0, &g_exp_tab).x;
         out[6 * k + 1] = expm1(-a * inv_rho0);
         out[6 * k + 2] = recip(a);
         out[6 * k + 3] = 1.0 / a;

@@ -184,41 +184,49 @@ __device__ __forceinline__ float recip(float v) {
 
 // E = exp(-d / rho0) - 1 of a pair in FP64, c = -64 / (ln2 rho0), inv_rho0 =
 // 1 / rho0: table-driven after P. T. P. Tang ("Table-driven implementation of
-// the expm1 function", ACM TOMS 18, 1992).  n = the integer nearest d c,
-// r = d c - n by one fused operation (|r| <= 1/2, in units of ln2 / 64), and
-// E = (T - 1) + T p with T = 2^(n/64) and T - 1 from the table and p =
-// exp(r ln2 / 64) - 1 from its Taylor polynomial of degree 6 (truncation below
-// 2^-57 relative).  Ten FP64 operations a value: GB300 runs two FP64 lanes
+// the expm1 function", ACM TOMS 18, 1992), with the accurate table of
+// lb_exp_table.h.  n = the integer nearest d c picks the table's argument b near
+// n ln2 / 64 (0 for |n| <= 1), r = -d inv_rho0 - b by one fused operation
+// (|r| < 0.0055, below 0.0163 where b = 0), and E = (T - 1) + T p with T = exp(b) and
+// p = exp(r) - 1 = r + r (r (1/2 + r/6 + ...)) from its Taylor polynomial of degree 7
+// (truncation below 2^-56 relative).  Half an ulp each comes from inv_rho0 and r (as
+// in the library's expm1(-d inv_rho0)), from p, and from the last operation; where
+// the last one rounds (|n| >= 2), r and p are at most a third of E.  Root mean
+// square errors in 2^-52, rho0 = 0.7, |d| up to 1e-3, 0.03, 0.9 rho0: 0.324, 0.306, 0.292;
+// the library's 0.325, 0.325, 0.355; with a table of rounded powers 2^(n/64), r
+// counted in units of ln2 / 64 and n = 0 up to half a unit only 0.427, 0.353, 0.326.
+// Ten FP64 operations a value: GB300 runs two FP64 lanes
 // per SM and clock, and the FP64 step is bound by them (310 per site with the
 // library's expm1 and divisions and row-by-row stencil sums, its FP64 pipe
-// 80 % busy; 512^2 took 205 us a step, with this and the column sums of
+// 80 % busy; 512^2 took 205 us a step, with a table and the column sums of
 // force_sums_warp 144 us).  Outside the table
-// (-d / rho0 beyond [-3.4, 2.0]) and for non-finite d the library's expm1.
+// (-d / rho0 beyond [-3.47, 2.07]) and for non-finite d the library's expm1.
+struct ExpTable {
+    double2 t[kExpN];      // {T, T - 1}
+    double b[kExpN];
+};
 __device__ __noinline__ double expm1_slow(double x);
 __device__ __forceinline__ double2 pexpm1_scaled(double2 d, double c, double inv_rho0,
-                                                 const double2* tab) {
-    double2 r;
+                                                 const ExpTable* tab) {
     int k[2];
     bool ok = true;
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
-        const double x = s ? d.y : d.x;
-        const double t = fma(x, c, 6755399441055744.0);   // 1.5 2^52: rounds to an integer
-        const double n = t - 6755399441055744.0;
-        (s ? r.y : r.x) = fma(x, c, -n);
+        const double t = fma(s ? d.y : d.x, c, 6755399441055744.0);   // 1.5 2^52: rounds to an integer
         k[s] = __double2loint(t) + kExpLo;
         // |n| < 2^31 (the high word of 1.5 2^52, or one less), n in the table
         ok = ok && (unsigned)(__double2hiint(t) - 0x4337ffff) <= 1u && (unsigned)k[s] < (unsigned)kExpN;
     }
     if (!ok) return make_double2(expm1_slow(-d.x * inv_rho0), expm1_slow(-d.y * inv_rho0));
-    double2 p = pset(0x1.430912f86c787p-49);              // (ln2/64)^j / j!, j = 6 .. 1
-    p = pfma(p, r, pset(0x1.5d87fe78a6731p-40));
-    p = pfma(p, r, pset(0x1.3b2ab6fba4e77p-31));
-    p = pfma(p, r, pset(0x1.c6b08d704a0c0p-23));
-    p = pfma(p, r, pset(0x1.ebfbdff82c58fp-15));
-    p = pfma(p, r, pset(0x1.62e42fefa39efp-7));
-    p = pmul(p, r);
-    const double2 ta = tab[k[0]], tb = tab[k[1]];
+    const double2 r = make_double2(fma(-d.x, inv_rho0, -tab->b[k[0]]), fma(-d.y, inv_rho0, -tab->b[k[1]]));
+    double2 p = pset(1.0 / 5040.0);
+    p = pfma(p, r, pset(1.0 / 720.0));
+    p = pfma(p, r, pset(1.0 / 120.0));
+    p = pfma(p, r, pset(1.0 / 24.0));
+    p = pfma(p, r, pset(1.0 / 6.0));
+    p = pfma(p, r, pset(0.5));
+    p = pfma(pmul(p, r), r, r);
+    const double2 ta = tab->t[k[0]], tb = tab->t[k[1]];
     return make_double2(fma(ta.x, p.x, ta.y), fma(tb.x, p.y, tb.y));
 }
 // exp(x) - 1 of a pair in FP32: branch-free, by the Cody-Waite reduction x = k ln2 + r (|r| <= ln2 / 2, ln2 split into a
@@ -301,7 +309,7 @@ struct Layout {
     static constexpr int STAGE_BYTES = STAGED ? STAGE_FULL : 0;
     // FP64: the exponential table (pexpm1_scaled)
     static constexpr int TAB_OFF = STAGE_OFF + STAGE_BYTES;
-    static constexpr int TAB_BYTES = P == LB_FP64 ? kExpN * (int)sizeof(double2) : 0;
+    static constexpr int TAB_BYTES = P == LB_FP64 ? (int)sizeof(ExpTable) : 0;
     static constexpr int SMEM = TAB_OFF + TAB_BYTES + 128;
     // staging slot (plane 0) of tile row ly, column lx: planes of a half are
     // 8 TX pairs apart

@@ -49,3 +49,45 @@ def test_reciprocal_special_values(lb):
                   np.finfo(np.float64).max, np.inf, -np.inf, -1e308, -2e-310, np.nan])
     _, _, r, want, _, _ = probe(lb, x)
     assert np.array_equal(r, want, equal_nan=True)
+
+
+def expm1_error(got, x, rho0):
+    """Error relative to exp(-x/rho0) - 1, in 2^-52."""
+    exact = np.expm1(-x.astype(np.longdouble) / np.longdouble(rho0))
+    return ((got - exact) / exact * 2.0 ** 52).astype(np.float64)
+
+
+@pytest.mark.parametrize("rho0", [0.51, 0.55, 0.6, 0.7, 0.83, 0.97, 0.1])
+@pytest.mark.parametrize("amp", [1e-6, 1e-3, 0.03, 0.3, 0.9])
+def test_expm1_is_as_good_as_the_library(lb, rho0, amp):
+    """Half a unit each from 1/rho0, from the argument, and from the last of the
+    operations that follow; the table and the series add less than a tenth.  The
+    root mean square is no larger than that of the library's expm1 of the same
+    argument (2 % for the sampling)."""
+    assert np.finfo(np.longdouble).nmant >= 63
+    rng = np.random.default_rng(11)
+    x = amp * rho0 * (2.0 * rng.random(400_000) - 1.0)
+    x = x[x != 0.0]
+    ours, lib = probe(lb, x, x, rho0)[:2]
+    e, el = expm1_error(ours, x, rho0), expm1_error(lib, x, rho0)
+    print(f"rho0 {rho0} |x| <= {amp} rho0: max {np.abs(e).max():.3f} (library {np.abs(el).max():.3f}), "
+          f"rms {np.sqrt((e * e).mean()):.4f} ({np.sqrt((el * el).mean()):.4f})")
+    assert np.abs(e).max() <= 1.6
+    assert np.sqrt((e * e).mean()) <= 1.02 * np.sqrt((el * el).mean())
+
+
+def test_expm1_at_and_beyond_the_table(lb):
+    """The table's ends (-x/rho0 = -3.47 and 2.07), its inner steps (the multiples
+    of ln2/128), and the library outside, for huge and non-finite arguments too."""
+    rho0 = 0.7
+    steps = -rho0 * np.log(2.0) / 128.0 * np.arange(-641, 385)
+    x = np.concatenate([steps, np.nextafter(steps, 1.0), np.nextafter(steps, -1.0), steps * (1 + 1e-9)])
+    x = x[x != 0.0]
+    ours, lib = probe(lb, x, x, rho0)[:2]
+    tiny = np.abs(x) < np.finfo(np.float64).tiny   # (no relative error there)
+    assert np.array_equal(ours[tiny], lib[tiny])
+    assert np.abs(expm1_error(ours[~tiny], x[~tiny], rho0)).max() <= 1.6
+    far = np.array([0.0, 2.6, 30.0, 500.0, 1e10, 1e300, np.inf, -1.5, -2.0, -400.0, -1e10, -1e300, -np.inf, np.nan])
+    # (the pair's other value is inside the table: one outside takes both to the library)
+    ours, lib = probe(lb, far, np.full(far.size, 0.01), rho0)[:2]
+    assert np.array_equal(ours, lib, equal_nan=True)

@@ -91,3 +91,26 @@ def test_expm1_at_and_beyond_the_table(lb):
     # (the pair's other value is inside the table: one outside takes both to the library)
     ours, lib = probe(lb, far, np.full(far.size, 0.01), rho0)[:2]
     assert np.array_equal(ours, lib, equal_nan=True)
+
+
+@pytest.mark.parametrize("lo,hi", [(0.5, 2.5), (1e-6, 1e6), (1e-80, 1e80)])
+@pytest.mark.parametrize("scale", [1.0, 1e-12, 1e-150, 1e-290, 1e-310, 1e200])
+def test_quotient_is_the_division(lb, lo, hi, scale):
+    """Velocities, momentum / density: rounded as the division (but for the few
+    reciprocals that are not, see above: four at most of 10^6)."""
+    rng = np.random.default_rng(7)
+    t = np.exp(np.log(lo) + (np.log(hi) - np.log(lo)) * rng.random(1_000_000))
+    m = scale * (2.0 * rng.random(t.size) - 1.0)
+    m[:100] = 0.0
+    m[100:200] = -0.0
+    got, want = probe(lb, t, m)[4:]
+    assert np.count_nonzero(got != want) <= 4
+    assert np.array_equal(np.signbit(got), np.signbit(want))
+
+
+def test_quotient_special_values(lb):
+    t = np.array([1.3, 1e-300, 1e300, -1.3, np.inf, 2e-310, np.nan])
+    m = np.array([0.0, -0.0, 1.0, -2e-310, 1e308, -np.inf, np.nan])
+    t, m = (a.ravel() for a in np.meshgrid(t, m))
+    got, want = probe(lb, t, m)[4:]
+    assert np.array_equal(got, want, equal_nan=True)

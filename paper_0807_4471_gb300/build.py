@@ -1,6 +1,6 @@
 """In-tree build of liblbgb.so (CUDA kernels + C ABI) for sm_103a.
 
-The two translation units are compiled in parallel with nvcc and linked into
+The translation units are compiled in parallel with nvcc and linked into
 ``paper_0807_4471_gb300/liblbgb.so``; objects go to ``paper_0807_4471_gb300/_build``.
 """
 from __future__ import annotations
@@ -14,9 +14,12 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(os.path.dirname(PKG), "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "liblbgb.so")
-# (source, extra defines, object name); the step kernels are compiled once
-# per storage precision so that the four compilations run in parallel.
-UNITS = [("lb_kernels.cu", [f"-DLB_PREC={p}"], f"lb_kernels_p{p}.o") for p in range(4)] + [
+# (source, extra defines, object name); the kernels are compiled per storage
+# precision and part (0: observe and initialise; else the step kernels of a tile
+# shape, see lb_kernels.cu): in parallel, and one module each to the driver.
+PARTS = {0: (1, 0), 1: (1, 2, 4, 5, 0), 2: (1, 2, 3, 4, 0), 3: (1, 2, 3, 4, 0)}
+UNITS = [("lb_kernels.cu", [f"-DLB_PREC={p}", f"-DLB_PART={k}"], f"lb_kernels_p{p}_{k}.o")
+         for p, parts in PARTS.items() for k in parts] + [
     ("lb_dispatch.cu", [], "lb_dispatch.o"),
     ("lb_engine.cu", [], "lb_engine.o"),
     ("lb_api.cu", [], "lb_api.o"),

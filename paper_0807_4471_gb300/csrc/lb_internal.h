@@ -235,13 +235,11 @@ int kernel_staged(int precision, int shape);
 // Step: the persistent multi-lattice kernel (args: BatchArgs<C>), variant
 // bit 0 = every lattice periodic, bit 1 = general forcing, bit 2 = 1 - omega
 // rounds to zero for both species (the collision reads no populations), in one of the
-// precision's tile shapes.  Observe: one lattice (args: StepArgs<C>, tin: tile-box
+// precision's tile shapes; without args the kernel is only made ready (call it so
+// before capturing launches into a graph).  Observe: one lattice (args: StepArgs<C>, tin: tile-box
 // load map), at most one CTA per 8-row tile.
 cudaError_t launch_step(int precision, const void* args, int variant, int shape, dim3 grid,
                         cudaStream_t s);
-// Opt the kernels of a precision into their shared memory (once per device;
-// call before capturing launches into a graph).
-cudaError_t kernels_configure(int precision);
 cudaError_t launch_observe(int precision, const CUtensorMap* tin, const void* args, dim3 grid,
                            cudaStream_t s);
 // Initial states (see k_init).  fields: rho_A, rho_B, u_x, u_y (velocities may
@@ -263,10 +261,10 @@ cudaError_t launch_load_pops(int precision, const Geom& g, const void* coef, voi
                              const double* pops, size_t species, size_t direction, int i0, int i1,
                              const StateInit& state, cudaStream_t s);
 
-// Per-precision launchers, one explicit instantiation per compilation of
-// lb_kernels.cu (-DLB_PREC=P).
-template <int P>
-cudaError_t configure_prec();
+// Per-precision launchers, explicitly instantiated by the compilations of
+// lb_kernels.cu (-DLB_PREC=P; launch_step_shape with -DLB_PART=SH).
+template <int P, int SH>
+cudaError_t launch_step_shape(const void* args, int variant, dim3 grid, cudaStream_t s);
 template <int P>
 cudaError_t launch_step_prec(const void* args, int variant, int shape, dim3 grid, cudaStream_t s);
 template <int P>

@@ -30,15 +30,29 @@
 // few tiles (a shorter chain of latencies), and k_step_m, for FP32 at tau = 1
 // (the state held by its moments).  There is no dense contraction anywhere, so
 // no tensor cores are used.
+//
+// Compiled once per storage precision and part (-DLB_PREC=0..3 -DLB_PART=k): part 0
+// is the observe and initialising kernels and the launchers' dispatch, part k >= 1
+// the step kernels of tile shape k (Shape; SHAPE_M8: both moment shapes).  A
+// unit's kernels are one module to the driver, which loads it at the first use of
+// one of them, at a cost that grows with all of them: with one module per
+// precision the first initialisation of a process took 1.16 ms and its first step
+// 0.68 ms (FP16), now 0.26 and 0.36.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <atomic>
 #include <cstdint>
 #include <cstdlib>
 #include <type_traits>
+#include <utility>
 
 #include "lb_internal.h"
 #include "lb_layout.cuh"
+
+#if !defined(LB_PREC) || !defined(LB_PART)
+#error "compile lb_kernels.cu with -DLB_PREC=0..3 -DLB_PART=0..5"
+#endif
 
 namespace lbgb {
 
@@ -234,7 +248,6 @@ __device__ __forceinline__ void load_site(const typename Prec<P>::T2* bm,
 
 #if LB_PREC == 0
 static __device__ const ExpTable g_exp_tab = {{LB_EXP_TABLE}, {LB_EXP_ARGS}};
-__device__ __noinline__ double expm1_slow(double x) { return expm1(x); }
 #endif
 
 // Deviation of the pseudo-potential from Psi(rho_ref), both species:
@@ -1347,7 +1360,7 @@ __global__ void __launch_bounds__(Layout<P, SH>::NT, Layout<P, SH>::CTAS)
 // registers.  One CTA per SM; the site arithmetic is k_step's.  Measured, k_step
 // -> this: 300 x 211 FP32 Couette with tau 0.8 (135 tiles) 8.3 -> 7.4 us a step,
 // 128^2 FP16 5.25 -> 4.67, 64^2 FP16 5.18 -> 4.61.
-#if LB_PREC != 0
+#if LB_PART == 4
 template <int P, int V>
 __global__ void __launch_bounds__(DLayout<P>::NT, 1)
     k_step_d(const __grid_constant__ BatchArgs<float> a) {
@@ -1537,7 +1550,7 @@ __global__ void __launch_bounds__(DLayout<P>::NT, 1)
 // Two barriers per tile: after the expansion, and before the site phase.  The
 // site phase reads no populations, so the next tile's expansion follows it
 // without one.
-#if LB_PREC == 1
+#if LB_PART == 5
 template <int V, int SH>
 __global__ void __launch_bounds__(MLayout<SH>::NT, MLayout<SH>::CTAS)
     k_step_m(const __grid_constant__ BatchArgs<float> a) {
@@ -1835,6 +1848,10 @@ __global__ void __launch_bounds__(MLayout<SH>::NT, MLayout<SH>::CTAS)
     if (tid == 0) *a.ticket = 0u;
 }
 
+#endif
+
+#if LB_PART == 0
+#if LB_PREC == 1
 // The populations of a state held by its moments, into population planes with
 // their ghost copies.
 __global__ void k_expand(Geom g, const __grid_constant__ Coef<float> k, const float2* mom, float2* fout) {
@@ -2246,80 +2263,29 @@ __global__ void k_math64_probe(double rho0, const double* __restrict__ x, const 
     }
 }
 #endif
+#endif   // LB_PART == 0
 
 // ------------------------------------------------------------- launchers
-// Step kernels of precision P in its tile shapes and the observe kernels,
-// variant by variant.
-template <int P>
-static cudaError_t configure_all() {
-    typedef Layout<P> L;
-    cudaError_t e = cudaSuccess;
-    auto opt = [&](auto kern, int bytes) {
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (e == cudaSuccess)   // room for the shape's resident CTAs
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     cudaSharedmemCarveoutMaxShared);
-    };
-    auto opt_shape = [&](auto tag) {
-        constexpr int SH = decltype(tag)::value;
-        if constexpr (has_shape(P, SH)) {
-            constexpr int bytes = Layout<P, SH>::SMEM;
-            opt(k_step<P, 0, SH>, bytes);
-            opt(k_step<P, 1, SH>, bytes);
-            opt(k_step<P, 2, SH>, bytes);
-            opt(k_step<P, 3, SH>, bytes);
-            opt(k_step<P, 4, SH>, bytes);
-            opt(k_step<P, 5, SH>, bytes);
-            opt(k_step<P, 6, SH>, bytes);
-            opt(k_step<P, 7, SH>, bytes);
-        }
-    };
-    opt_shape(std::integral_constant<int, SHAPE_8>{});
-    opt_shape(std::integral_constant<int, SHAPE_16>{});
-    opt_shape(std::integral_constant<int, SHAPE_8X2>{});
-#if LB_PREC != 0
-    constexpr int dbytes = DLayout<P>::SMEM;
-    opt(k_step_d<P, 0>, dbytes);
-    opt(k_step_d<P, 1>, dbytes);
-    opt(k_step_d<P, 2>, dbytes);
-    opt(k_step_d<P, 3>, dbytes);
-    opt(k_step_d<P, 4>, dbytes);
-    opt(k_step_d<P, 5>, dbytes);
-    opt(k_step_d<P, 6>, dbytes);
-    opt(k_step_d<P, 7>, dbytes);
-#endif
-#if LB_PREC == 1
-    auto opt_moments = [&](auto tag) {
-        constexpr int SH = decltype(tag)::value;
-        constexpr int bytes = MLayout<SH>::SMEM;
-        opt(k_step_m<0, SH>, bytes);
-        opt(k_step_m<1, SH>, bytes);
-        opt(k_step_m<2, SH>, bytes);
-        opt(k_step_m<3, SH>, bytes);
-    };
-    opt_moments(std::integral_constant<int, SHAPE_M8>{});
-    opt_moments(std::integral_constant<int, SHAPE_M8X2>{});
-#endif
-    opt(k_observe<P, 2, false>, L::SMEM_OBS);
-    opt(k_observe<P, 3, false>, L::SMEM_OBS);
-    opt(k_observe<P, 2, true>, L::SMEM_OBS);
-    opt(k_observe<P, 3, true>, L::SMEM_OBS);
-    return e;
-}
-
-// Opt every kernel of this precision into its dynamic shared memory, once
-// per device.
-template <int P>
-static cudaError_t ensure_configured() {
-    static int configured[64] = {0};
+// A kernel's opt-in to its dynamic shared memory and to room for its resident
+// CTAs: at its first launch on each device.
+struct OptIn {
+    std::atomic<unsigned long long> devices{0};
+};
+template <typename K>
+static cudaError_t opt_in(OptIn& done, K kernel, int bytes) {
     int dev = 0;
     cudaGetDevice(&dev);
-    if (dev >= 0 && dev < 64 && configured[dev]) return cudaSuccess;
-    cudaError_t e = configure_all<P>();
-    if (e == cudaSuccess && dev >= 0 && dev < 64) configured[dev] = 1;
+    const unsigned long long bit = dev >= 0 && dev < 64 ? 1ull << dev : 0;
+    if (done.devices.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess) done.devices.fetch_or(bit, std::memory_order_relaxed);
     return e;
 }
 
+#if LB_PART != 0
 // LB_PDL=0 in the environment turns the programmatic launches off (A/B
 // timing); read once per process.
 static bool pdl_enabled() {
@@ -2349,50 +2315,47 @@ static cudaError_t launch_pdl(K kernel, const A& a, int threads, int smem, dim3 
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-template <int P, int SH>
-static cudaError_t launch_step_shape(const BatchArgs<typename Prec<P>::C>& a, int variant, dim3 grid,
-                                     cudaStream_t s) {
-    typedef Layout<P, SH> L;
-    switch (variant & 7) {
-        case 0: return launch_pdl(k_step<P, 0, SH>, a, L::NT, L::SMEM, grid, s);
-        case 1: return launch_pdl(k_step<P, 1, SH>, a, L::NT, L::SMEM, grid, s);
-        case 2: return launch_pdl(k_step<P, 2, SH>, a, L::NT, L::SMEM, grid, s);
-        case 3: return launch_pdl(k_step<P, 3, SH>, a, L::NT, L::SMEM, grid, s);
-        case 4: return launch_pdl(k_step<P, 4, SH>, a, L::NT, L::SMEM, grid, s);
-        case 5: return launch_pdl(k_step<P, 5, SH>, a, L::NT, L::SMEM, grid, s);
-        case 6: return launch_pdl(k_step<P, 6, SH>, a, L::NT, L::SMEM, grid, s);
-        default: return launch_pdl(k_step<P, 7, SH>, a, L::NT, L::SMEM, grid, s);
-    }
-}
-
-#if LB_PREC != 0
-template <int P>
-static cudaError_t launch_direct(const BatchArgs<float>& a, int variant, dim3 grid, cudaStream_t s) {
-    typedef DLayout<P> L;
-    switch (variant & 7) {
-        case 0: return launch_pdl(k_step_d<P, 0>, a, L::NT, L::SMEM, grid, s);
-        case 1: return launch_pdl(k_step_d<P, 1>, a, L::NT, L::SMEM, grid, s);
-        case 2: return launch_pdl(k_step_d<P, 2>, a, L::NT, L::SMEM, grid, s);
-        case 3: return launch_pdl(k_step_d<P, 3>, a, L::NT, L::SMEM, grid, s);
-        case 4: return launch_pdl(k_step_d<P, 4>, a, L::NT, L::SMEM, grid, s);
-        case 5: return launch_pdl(k_step_d<P, 5>, a, L::NT, L::SMEM, grid, s);
-        case 6: return launch_pdl(k_step_d<P, 6>, a, L::NT, L::SMEM, grid, s);
-        default: return launch_pdl(k_step_d<P, 7>, a, L::NT, L::SMEM, grid, s);
-    }
-}
+#if LB_PART == 4
+constexpr int kVariants = 8;
+template <int P, int SH> using StepLayout = DLayout<P>;
+template <int P, int SH, int V> static constexpr auto step_kernel() { return &k_step_d<P, V>; }
+#elif LB_PART == 5   // (omega = 1 throughout: no variant bit 2)
+constexpr int kVariants = 4;
+template <int P, int SH> using StepLayout = MLayout<SH>;
+template <int P, int SH, int V> static constexpr auto step_kernel() { return &k_step_m<V, SH>; }
+#else
+constexpr int kVariants = 8;
+template <int P, int SH> using StepLayout = Layout<P, SH>;
+template <int P, int SH, int V> static constexpr auto step_kernel() { return &k_step<P, V, SH>; }
 #endif
 
-#if LB_PREC == 1
-template <int SH>
-static cudaError_t launch_moments_shape(const BatchArgs<float>& a, int variant, dim3 grid, cudaStream_t s) {
-    typedef MLayout<SH> L;
-    switch (variant & 3) {
-        case 0: return launch_pdl(k_step_m<0, SH>, a, L::NT, L::SMEM, grid, s);
-        case 1: return launch_pdl(k_step_m<1, SH>, a, L::NT, L::SMEM, grid, s);
-        case 2: return launch_pdl(k_step_m<2, SH>, a, L::NT, L::SMEM, grid, s);
-        default: return launch_pdl(k_step_m<3, SH>, a, L::NT, L::SMEM, grid, s);
-    }
+template <int P, int SH, int V>
+static cudaError_t launch_variant(const void* args, dim3 grid, cudaStream_t s) {
+    typedef StepLayout<P, SH> L;
+    static OptIn done;
+    const cudaError_t e = opt_in(done, step_kernel<P, SH, V>(), L::SMEM);
+    if (e != cudaSuccess || !args) return e;
+    return launch_pdl(step_kernel<P, SH, V>(), *reinterpret_cast<const BatchArgs<typename Prec<P>::C>*>(args), L::NT,
+                      L::SMEM, grid, s);
 }
+template <int P, int SH, int... V>
+static cudaError_t launch_one_of(const void* args, int variant, dim3 grid, cudaStream_t s,
+                                 std::integer_sequence<int, V...>) {
+    cudaError_t e = cudaErrorInvalidValue;
+    (void)((variant == V && ((e = launch_variant<P, SH, V>(args, grid, s)), true)) || ...);
+    return e;
+}
+template <int P, int SH>
+cudaError_t launch_step_shape(const void* args, int variant, dim3 grid, cudaStream_t s) {
+    return launch_one_of<P, SH>(args, variant & (kVariants - 1), grid, s, std::make_integer_sequence<int, kVariants>{});
+}
+template cudaError_t launch_step_shape<LB_PREC, LB_PART>(const void*, int, dim3, cudaStream_t);
+#if LB_PART == 5
+template cudaError_t launch_step_shape<LB_PREC, SHAPE_M8X2>(const void*, int, dim3, cudaStream_t);
+#endif
+
+#else   // LB_PART == 0
+#if LB_PREC == 1
 cudaError_t launch_expand(const Geom& g, const Coef<float>& k, const float2* mom, void* fout,
                           cudaStream_t s) {
     const long long N = (long long)g.nx * g.ny;
@@ -2405,45 +2368,44 @@ cudaError_t launch_expand(const Geom& g, const Coef<float>& k, const float2* mom
 
 template <int P>
 cudaError_t launch_step_prec(const void* args, int variant, int shape, dim3 grid, cudaStream_t s) {
-    typedef typename Prec<P>::C C;
-    cudaError_t e = ensure_configured<P>();
-    if (e != cudaSuccess) return e;
-    const BatchArgs<C>& a = *reinterpret_cast<const BatchArgs<C>*>(args);
-    if (shape == SHAPE_8) return launch_step_shape<P, SHAPE_8>(a, variant, grid, s);
-    if constexpr (has_shape(P, SHAPE_16))
-        if (shape == SHAPE_16) return launch_step_shape<P, SHAPE_16>(a, variant, grid, s);
-#if LB_PREC != 0
-    if (shape == SHAPE_D8) return launch_direct<P>(a, variant, grid, s);
-#endif
-#if LB_PREC == 1
-    if (shape == SHAPE_M8) return launch_moments_shape<SHAPE_M8>(a, variant, grid, s);
-    if (shape == SHAPE_M8X2) return launch_moments_shape<SHAPE_M8X2>(a, variant, grid, s);
-#endif
-    if constexpr (has_shape(P, SHAPE_8X2))
-        if (shape == SHAPE_8X2) return launch_step_shape<P, SHAPE_8X2>(a, variant, grid, s);
+    switch (shape) {
+        case SHAPE_8: return launch_step_shape<P, SHAPE_8>(args, variant, grid, s);
+        case SHAPE_16:
+            if constexpr (has_shape(P, SHAPE_16)) return launch_step_shape<P, SHAPE_16>(args, variant, grid, s);
+            break;
+        case SHAPE_8X2:
+            if constexpr (has_shape(P, SHAPE_8X2)) return launch_step_shape<P, SHAPE_8X2>(args, variant, grid, s);
+            break;
+        case SHAPE_D8:
+            if constexpr (has_shape(P, SHAPE_D8)) return launch_step_shape<P, SHAPE_D8>(args, variant, grid, s);
+            break;
+        case SHAPE_M8:
+            if constexpr (has_shape(P, SHAPE_M8)) return launch_step_shape<P, SHAPE_M8>(args, variant, grid, s);
+            break;
+        case SHAPE_M8X2:
+            if constexpr (has_shape(P, SHAPE_M8X2)) return launch_step_shape<P, SHAPE_M8X2>(args, variant, grid, s);
+            break;
+    }
     return cudaErrorInvalidValue;
 }
 
+template <int P, int V, bool POPS>
+static cudaError_t observe(const CUtensorMap* tin, const void* args, dim3 grid, cudaStream_t s) {
+    typedef Layout<P> L;
+    static OptIn done;
+    const cudaError_t e = opt_in(done, k_observe<P, V, POPS>, L::SMEM_OBS);
+    if (e != cudaSuccess) return e;
+    k_observe<P, V, POPS><<<grid, L::NT, L::SMEM_OBS, s>>>(
+        *tin, *reinterpret_cast<const StepArgs<typename L::C>*>(args));
+    return cudaGetLastError();
+}
 template <int P>
 cudaError_t launch_observe_prec(const CUtensorMap* tin, const void* args, dim3 grid,
                                 cudaStream_t s) {
-    typedef Layout<P> L;
-    typedef typename L::C C;
-    cudaError_t e = ensure_configured<P>();
-    if (e != cudaSuccess) return e;
-    const StepArgs<C>& a = *reinterpret_cast<const StepArgs<C>*>(args);
-    if (a.obs == OBS_POPS) {
-        if (a.g.periodic)
-            k_observe<P, 3, true><<<grid, L::NT, L::SMEM_OBS, s>>>(*tin, a);
-        else
-            k_observe<P, 2, true><<<grid, L::NT, L::SMEM_OBS, s>>>(*tin, a);
-    } else {
-        if (a.g.periodic)
-            k_observe<P, 3, false><<<grid, L::NT, L::SMEM_OBS, s>>>(*tin, a);
-        else
-            k_observe<P, 2, false><<<grid, L::NT, L::SMEM_OBS, s>>>(*tin, a);
-    }
-    return cudaGetLastError();
+    const auto& a = *reinterpret_cast<const StepArgs<typename Prec<P>::C>*>(args);
+    if (a.obs == OBS_POPS)
+        return a.g.periodic ? observe<P, 3, true>(tin, args, grid, s) : observe<P, 2, true>(tin, args, grid, s);
+    return a.g.periodic ? observe<P, 3, false>(tin, args, grid, s) : observe<P, 2, false>(tin, args, grid, s);
 }
 
 // One thread per column, rows dealt over the grid: no index is divided.
@@ -2465,19 +2427,6 @@ cudaError_t launch_init_prec(const Geom& g, const void* coef, void* fout, const 
                                            u_wall, init_shear, seed, state);
     return cudaGetLastError();
 }
-
-#ifndef LB_PREC
-#error "compile lb_kernels.cu once per storage precision with -DLB_PREC=0..3"
-#endif
-template <int P>
-cudaError_t configure_prec() {
-    return ensure_configured<P>();
-}
-
-template cudaError_t configure_prec<LB_PREC>();
-template cudaError_t launch_step_prec<LB_PREC>(const void*, int, int, dim3, cudaStream_t);
-template cudaError_t launch_observe_prec<LB_PREC>(const CUtensorMap*, const void*, dim3,
-                                                  cudaStream_t);
 template <int P>
 cudaError_t launch_load_pops_prec(const Geom& g, const void* coef, void* fout, const double* pops,
                                   size_t species, size_t direction, int i0, int i1,
@@ -2490,6 +2439,9 @@ cudaError_t launch_load_pops_prec(const Geom& g, const void* coef, void* fout, c
     return cudaGetLastError();
 }
 
+template cudaError_t launch_step_prec<LB_PREC>(const void*, int, int, dim3, cudaStream_t);
+template cudaError_t launch_observe_prec<LB_PREC>(const CUtensorMap*, const void*, dim3,
+                                                  cudaStream_t);
 template cudaError_t launch_load_pops_prec<LB_PREC>(const Geom&, const void*, void*, const double*,
                                                     size_t, size_t, int, int, const StateInit&,
                                                     cudaStream_t);
@@ -2497,10 +2449,7 @@ template cudaError_t launch_init_prec<LB_PREC>(const Geom&, const void*, void*, 
                                                double, double, double, int, unsigned long long,
                                                const StateInit&, cudaStream_t);
 
-}  // namespace lbgb
-
 #if LB_PREC == 0
-namespace lbgb {
 cudaError_t launch_math64_probe(double rho0, const double* x, const double* y, double* out, long long n,
                                 cudaStream_t s) {
     long long blocks = (n + 255) / 256;
@@ -2508,11 +2457,7 @@ cudaError_t launch_math64_probe(double rho0, const double* x, const double* y, d
     k_math64_probe<<<(unsigned)(blocks > 0 ? blocks : 1), 256, 0, s>>>(rho0, x, y, out, n);
     return cudaGetLastError();
 }
-}  // namespace lbgb
-#endif
-
-#if LB_PREC == 1
-namespace lbgb {
+#elif LB_PREC == 1
 cudaError_t launch_wait_selftest(unsigned int* err, int limit, cudaStream_t s) {
     k_wait_selftest<<<1, 32, 0, s>>>(err, limit);
     return cudaGetLastError();
@@ -2523,5 +2468,7 @@ cudaError_t launch_math_probe(const float* x, float* out, long long n, cudaStrea
     k_math_probe<<<(unsigned)(blocks > 0 ? blocks : 1), 256, 0, s>>>(x, out, n);
     return cudaGetLastError();
 }
-}  // namespace lbgb
 #endif
+#endif   // LB_PART == 0
+
+}  // namespace lbgb

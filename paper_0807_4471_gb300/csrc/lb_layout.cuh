@@ -205,7 +205,7 @@ struct ExpTable {
     double2 t[kExpN];      // {T, T - 1}
     double b[kExpN];
 };
-__device__ __noinline__ double expm1_slow(double x);
+template <typename T> __device__ __noinline__ T expm1_slow(T x) { return expm1(x); }
 __device__ __forceinline__ double2 pexpm1_scaled(double2 d, double c, double inv_rho0,
                                                  const ExpTable* tab) {
     int k[2];

@@ -191,10 +191,11 @@ lb_status build(lb_pool* P, Choice c) {
         if (e != cudaSuccess) return cuda_status(e);
         P->slot_cap = need;
     }
-    cudaError_t ce = kernels_configure(P->shared.precision);   // before any graph capture
-    if (ce != cudaSuccess) return cuda_status(ce);
     lb_status s = launch_build(P->launch, lats.data(), nlat, P->desc_mem, P->slots, P->slot_cap, P->ticket,
                                P->sms, P->stream, &P->stage, c.seg, c.shape);
+    if (s == LB_OK)   // the kernel made ready before any graph capture
+        s = cuda_status(launch_step(P->launch.precision, nullptr, P->launch.variant, P->launch.shape,
+                                    P->launch.grid, P->stream));
     P->built = s == LB_OK;
     return s;
 }

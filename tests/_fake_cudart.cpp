@@ -37,6 +37,8 @@ struct Fault {
 };
 std::map<std::string, Fault> faults;
 std::map<const void*, std::string> kernels;
+std::map<std::string, int> module_of;   // kernel name -> the module (compilation unit) it is in
+int modules = 0;
 std::vector<LaunchRec> launches;
 std::string errors;
 int sms = 152;
@@ -191,16 +193,22 @@ void* fk_launch_dst(int k, int q) {
 // An allocation of the library's kind, for a caller's workspace.
 void* fk_device(size_t bytes) { return take(bytes, cudaMemoryTypeDevice); }
 
-// ----------------------------------------------------------- registration
-void** __cudaRegisterFatBinary(void*) {
-    static void* h[1];
-    return h;
+int fk_module(const char* kernel) { return module_of.count(kernel) ? module_of[kernel] : -1; }
+// Kernels in a module whose names hold `part`.
+int fk_module_kernels(int m, const char* part) {
+    int n = 0;
+    for (auto& k : module_of) n += k.second == m && k.first.find(part) != std::string::npos;
+    return n;
 }
+
+// ----------------------------------------------------------- registration
+void** __cudaRegisterFatBinary(void*) { return (void**)(intptr_t)(8 * ++modules); }
 void __cudaRegisterFatBinaryEnd(void**) {}
 void __cudaUnregisterFatBinary(void**) {}
-void __cudaRegisterFunction(void**, const char* host, char*, const char* name, int, uint3*, uint3*, dim3*, dim3*,
-                            int*) {
+void __cudaRegisterFunction(void** module, const char* host, char*, const char* name, int, uint3*, uint3*, dim3*,
+                            dim3*, int*) {
     kernels[host] = name;
+    module_of[name] = (int)((intptr_t)module / 8);
 }
 void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}
 unsigned __cudaPushCallConfiguration(dim3 grid, dim3 block, size_t shmem, void* stream) {

@@ -108,9 +108,13 @@ typedef struct {
     double kolmo_k;            /* a_x += kolmo_amp sin(2 pi kolmo_k y / ny)    */
     int32_t rounding;          /* lb_rounding of the half formats              */
     int32_t tile_rows;         /* step-kernel tile height of an lb_create handle:
-                                  0 = library default, 8 (one site per thread)
-                                  or 16 (two per thread; not LB_FP64); results
-                                  are bitwise the same; pools choose their own */
+                                  0 = library default, 8 or 16 (not LB_FP64);
+                                  results are bitwise the same.  The library
+                                  picks the sites per thread and the CTAs per
+                                  SM.  A height asked for keeps LB_FP32 at
+                                  tau = 1 in populations, three times the bytes
+                                  of its default form (4096^2: 43 GLUPS, 54 by
+                                  default).  Pools choose their own */
 } lb_params;
 
 typedef struct {
@@ -224,8 +228,9 @@ lb_status lb_destroy(lb_handle* h);
  * graph and replayed.  The work partition (segment length of the
  * column strips) is tuned by timing candidate partitions on the first steps
  * of each new member set (those steps are real steps) and cached; a member
- * set that runs fewer than 8 times the steps the timing takes (about 400 to
- * 500 steps) keeps the load-balance model's partition instead.
+ * set that runs fewer than 8 times the steps the timing takes (48 for each
+ * candidate, some 400 in all, 850 where two tile shapes are timed) keeps the
+ * load-balance model's partition instead.
  * ------------------------------------------------------------------------ */
 typedef struct lb_pool lb_pool;
 typedef int32_t lb_job;
@@ -287,25 +292,34 @@ int32_t lb_pool_segment(const lb_pool* pool);
  * CTA, 0 back to autotuning.  Applies from the next lb_pool_run. */
 lb_status lb_pool_set_partition(lb_pool* pool, int32_t seg);
 
-/* Tile height of the step kernel: the autotuner times both tile shapes (8
- * rows, one site per thread; 16 rows, two vertically adjacent sites per
- * thread sharing their stencil rows -- not for FP64) together with the
- * partitions.  lb_pool_set_tile_rows fixes it (8 or 16; 0 back to
- * autotuning; LB_ERR_INVALID for a shape the pool's precision lacks), from
- * the next lb_pool_run; lb_pool_tile_rows returns the current launch's, or
- * 0 if none is built.  Every shape gives bitwise the same results. */
+/* Tile height of the step kernel: the autotuner times the tile shapes that
+ * compete for the member set together with the partitions -- LB_FP32 8 and 16
+ * rows, at tau = 1 (velocity shift) one and two sites per thread on 8 rows; the
+ * 16-bit formats and LB_FP64 one shape of 8 rows.  lb_pool_set_tile_rows fixes the
+ * height (8 or 16; 0 back to autotuning; LB_ERR_INVALID for one the pool's
+ * precision lacks), from the next lb_pool_run, and with it LB_FP32 at tau = 1 to
+ * populations (lb_params.tile_rows); lb_pool_tile_rows returns the current
+ * launch's, or 0 if none is built.  Every shape gives bitwise the same results. */
 lb_status lb_pool_set_tile_rows(lb_pool* pool, int32_t rows);
 int32_t lb_pool_tile_rows(const lb_pool* pool);
 
 lb_status lb_pool_destroy(lb_pool* pool);
 
-/* Host only, no device work (usable without a GPU): the work items that one
- * step launch over `nlat` lattices with parameters ps[0 .. nlat-1] would use
- * on a device with `sms` SMs.  seg > 0: segments of seg tiles, each given in
+/* Host only, no device work (usable without a GPU): the work items of a step
+ * launch in tiles over `nlat` lattices with parameters ps[0 .. nlat-1], one CTA
+ * on each of `sms` SMs.  seg > 0: segments of seg tiles, each given in
  * band order to the CTA with the least estimated work; -1: one cost-balanced
- * contiguous run of tiles per CTA; 0: the library's default for these sizes.
+ * contiguous run of tiles per CTA; 0: runs for up to 40 8-row tiles a CTA, the
+ * load-balance model's segments beyond.
  * A tile is TX x tile_rows sites (TX = 60; 28 for FP64), a strip a TX-wide
- * column of tiles; tile_rows is 8 (or 0, meaning 8) or 16 (not for FP64).  On entry *nitems is the capacity of `items` (in items of
+ * column of tiles; tile_rows is 8 (or 0, meaning 8) or 16 (not for FP64).
+ * This is the plan of launches of population kernels with one CTA per SM (a tile
+ * height of 16; 8 rows in LB_FP32).  Others follow the same rules with their own
+ * numbers: two CTAs per SM for the 16-bit formats and LB_FP32 at tau = 1 beyond
+ * 1.5 tiles per SM; runs at every size and no cost for ghost copies in LB_FP32 at
+ * tau = 1; runs also for sets of lattices that take up to a third of L2 each;
+ * and LB_FP64 launches cut rows, in groups of 1 to 8, where this plan has tiles.
+ * On entry *nitems is the capacity of `items` (in items of
  * 4 int32: lattice index, strip, first tile row, end tile row) and *grid the
  * capacity of `cta` (in entries); on return they hold the item count and the
  * number of CTAs, items lists the items CTA by CTA, the items of CTA b are

@@ -321,7 +321,8 @@ def lb_pool_destroy(pool: int):
 
 
 def lb_plan_partition(params, seg: int = 0, sms: int = 152, tile_rows: int = 8):
-    """Host-only work plan of one step launch over the lattices `params`:
+    """Host-only work plan in tiles of a step launch with one CTA per SM over the
+    lattices `params` (include/lb.h says which launches differ):
     (items int32[n, 4] = lattice, strip, first tile row, end tile row;
     cta int32[grid + 1] offsets into items; the partition applied)."""
     import numpy as np

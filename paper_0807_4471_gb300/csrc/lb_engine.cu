@@ -8,8 +8,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <functional>
-#include <queue>
 #include <utility>
 
 namespace lbgb {
@@ -429,28 +427,47 @@ void partition(Lattice* const* lats, int nlat, int seg, int shape, int sms, std:
         // each given to the CTA with the least work so far (the lowest index
         // among equals): round-robin dealing when costs are equal, while the
         // CTAs that draw the costlier edge segments take fewer of them.
-        std::vector<Item> all;
+        long long nseg = 0;
+        for (int l = 0; l < nlat; ++l) nseg += (long long)lats[l]->nstrips * ((nty[(size_t)l] + seg - 1) / seg);
+        const int G = (int)std::min<long long>(nseg, sms);
+        std::vector<std::vector<Item>> mine((size_t)G);
+        for (auto& m : mine) m.reserve((size_t)(nseg / G + 2));
+        typedef std::pair<double, int> Load;   // (work so far, CTA): a heap, smallest first
+        std::vector<Load> heap((size_t)G);
+        for (int b = 0; b < G; ++b) heap[(size_t)b] = {0.0, b};
+        // the item to the heap's first CTA, whose load then sinks to its place
+        auto deal = [&](const Item& it, double w) {
+            const Load top = {heap[0].first + w, heap[0].second};
+            mine[(size_t)top.second].push_back(it);
+            size_t at = 0;
+            for (size_t c = 1; c < heap.size(); c = 2 * at + 1) {
+                if (c + 1 < heap.size() && heap[c + 1] < heap[c]) ++c;
+                if (!(heap[c] < top)) break;
+                heap[at] = heap[c];
+                at = c;
+            }
+            heap[at] = top;
+        };
         for (int l = 0; l < nlat; ++l) {
             const int ns = lats[l]->nstrips, nt = nty[(size_t)l];
-            for (int a = 0; a < nt; a += seg)
-                for (int sx = 0; sx < ns; ++sx) all.push_back({l, sx, a, std::min(a + seg, nt)});
-        }
-        const int G = (int)std::min<long long>((long long)all.size(), sms);
-        std::vector<std::vector<int>> mine((size_t)G);
-        typedef std::pair<double, int> Load;   // (work so far, CTA): smallest first
-        std::priority_queue<Load, std::vector<Load>, std::greater<Load>> heap;
-        for (int b = 0; b < G; ++b) heap.push({0.0, b});
-        for (size_t k = 0; k < all.size(); ++k) {
-            const Load top = heap.top();
-            heap.pop();
-            double w = kItemStart;
-            for (int ty = all[k].ty_a; ty < all[k].ty_b; ++ty) w += cost(all[k].lat, all[k].strip, ty);
-            mine[(size_t)top.second].push_back((int)k);
-            heap.push({top.first + w, top.second});
+            for (int a = 0; a < nt; a += seg) {
+                const int b = std::min(a + seg, nt);
+                auto work = [&](int sx) {
+                    double w = kItemStart;
+                    for (int ty = a; ty < b; ++ty) w += cost(l, sx, ty);
+                    return w;
+                };
+                // (a strip between the first and the last two costs what its neighbours do)
+                double w = 0.0;
+                for (int sx = 0; sx < ns; ++sx) {
+                    if (sx < 2 || sx >= ns - 2) w = work(sx);
+                    deal({l, sx, a, b}, w);
+                }
+            }
         }
         for (int b = 0; b < G; ++b) {
             cta.push_back((int)items.size());
-            for (int k : mine[(size_t)b]) items.push_back(all[(size_t)k]);
+            items.insert(items.end(), mine[(size_t)b].begin(), mine[(size_t)b].end());
         }
         cta.push_back((int)items.size());
         *grid = G;

@@ -720,11 +720,9 @@ lb_status launch_build(Launch& Ln, Lattice* const* lats, int nlat, void* descs, 
     const size_t bytes = at_cta + sizeof(int) * cta.size();
     if (bytes - at_items > room * sizeof(double)) return LB_ERR_NOMEM;
     std::vector<char> own;
-    char* hs = nullptr;
-    if (stage) {
-        hs = stage->get(bytes);
-        if (!hs) return LB_ERR_CUDA;
-    } else {
+    char* hs = stage ? stage->get(bytes) : nullptr;
+    if (!hs) {   // no stage, or no pinned memory to be had
+        stage = nullptr;
         own.resize(bytes + 128);
         hs = own.data() + (128 - reinterpret_cast<uintptr_t>(own.data()) % 128) % 128;
     }
@@ -747,7 +745,9 @@ lb_status launch_build(Launch& Ln, Lattice* const* lats, int nlat, void* descs, 
     if (e == cudaSuccess)
         // (the CTA offsets follow the items on both sides)
         e = cudaMemcpyAsync(d_items, hs + at_items, bytes - at_items, cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess) e = stage ? stage->sent(stream) : cudaStreamSynchronize(stream);
+    // (also after a copy that failed: the one before it may be on its way)
+    const cudaError_t es = stage ? stage->sent(stream) : cudaStreamSynchronize(stream);
+    if (e == cudaSuccess) e = es;
     if (e != cudaSuccess) return cuda_status(e);
     Ln.precision = prec;
     Ln.variant = (allper ? 1 : 0) | (gen ? 2 : 0) | (tau1 ? 4 : 0);

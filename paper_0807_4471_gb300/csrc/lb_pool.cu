@@ -429,7 +429,7 @@ lb_status lb_pool_create(const lb_params* shared, size_t bytes_budget, int32_t m
         P->ticket = reinterpret_cast<unsigned int*>(P->desc_mem + dbytes);
         e = cudaMemsetAsync(P->ticket, 0, sizeof(unsigned int), P->stream);
     }
-    if (e == cudaSuccess) e = P->stage.reserve(kStageLeast);
+    if (e == cudaSuccess && P->stage.reserve(kStageLeast) != cudaSuccess) cudaGetLastError();
     if (e != cudaSuccess) {
         lb_pool_destroy(P);
         return cuda_status(e);

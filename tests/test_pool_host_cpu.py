@@ -84,3 +84,26 @@ assert len(step_items(launches("k_step")[0])) == 69 * 256
 lb.lb_pool_destroy(pool)
 assert count("cudaFreeHost") == 2
 """)
+
+
+def test_pool_runs_without_pinned_memory():
+    """No pinned memory to be had: tables go through pageable memory, as they do for
+    a lattice handle."""
+    run("""
+p = lb.make_params(64, 48, "fp32", psi_form=1)
+fk.fk_fail(b"cudaHostAlloc", 1, 2)
+pool = lb.lb_pool_create(p, 64 << 20, 2)
+for seed in (1, 2):
+    fk.fk_fail(b"cudaHostAlloc", 1, 2)
+    lb.lb_pool_admit(pool, p, seed, 100)
+    fk.fk_reset()
+    fk.fk_fail(b"cudaHostAlloc", 1, 2)
+    lb.lb_pool_run(pool, 3)
+    assert len(launches("k_step")) == 3 and count("cudaStreamSynchronize") >= 1
+fk.fk_fail(b"cudaHostAlloc", 1 << 30, 2)
+lb.lb_pool_set_partition(pool, 1)
+fk.fk_reset()
+lb.lb_pool_run(pool, 3)
+assert count("cudaStreamSynchronize") == 0       # pinned again
+lb.lb_pool_destroy(pool)
+""")

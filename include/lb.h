@@ -294,8 +294,8 @@ lb_status lb_pool_set_partition(lb_pool* pool, int32_t seg);
 
 /* Tile height of the step kernel: the autotuner times the tile shapes that
  * compete for the member set together with the partitions -- LB_FP32 8 and 16
- * rows, at tau = 1 (velocity shift) one and two sites per thread on 8 rows; the
- * 16-bit formats and LB_FP64 one shape of 8 rows.  lb_pool_set_tile_rows fixes the
+ * rows, at tau = 1 (velocity shift) and in the 16-bit formats shapes of 8 rows
+ * only (one and two sites per thread), LB_FP64 one shape.  lb_pool_set_tile_rows fixes the
  * height (8 or 16; 0 back to autotuning; LB_ERR_INVALID for one the pool's
  * precision lacks), from the next lb_pool_run, and with it LB_FP32 at tau = 1 to
  * populations (lb_params.tile_rows); lb_pool_tile_rows returns the current

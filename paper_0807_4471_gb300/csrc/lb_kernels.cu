@@ -929,7 +929,8 @@ __global__ void __launch_bounds__(Layout<P, SH>::NT, Layout<P, SH>::CTAS)
     // into tiles of 8 rows from their own first row on, the last one partial.
     // Its time is the number of rows a CTA sums (the FP64 pipe), so a lattice
     // is spread over the SMs row by row (128^2: 80 CTAs of one 8-row tile, 20.5 us
-    // a step; 128 CTAs of 5 rows, 16.4.  512^2: 142 -> 128 us).
+    // a step; 130 CTAs of 5 rows, 16.4.  512^2: 142 -> 128 us.  With the exacter
+    // functions and force sums since, 16.9 and 135).
     constexpr bool ROWS = P == LB_FP64;
     typedef typename L::T2 T2;
     typedef typename L::C C;

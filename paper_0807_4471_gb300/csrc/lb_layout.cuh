@@ -198,8 +198,8 @@ __device__ __forceinline__ float recip(float v) {
 // Ten FP64 operations a value: GB300 runs two FP64 lanes
 // per SM and clock, and the FP64 step is bound by them (310 per site with the
 // library's expm1 and divisions and row-by-row stencil sums, its FP64 pipe
-// 80 % busy; 512^2 took 205 us a step, with a table and the column sums of
-// force_sums_warp 144 us).  Outside the table
+// 80 % busy; 512^2 took 205 us a step, with a table, the column sums of
+// force_sums_warp and the work cut by rows 135 us).  Outside the table
 // (-d / rho0 beyond [-3.47, 2.07]) and for non-finite d the library's expm1.
 struct ExpTable {
     double2 t[kExpN];      // {T, T - 1}
